@@ -1,10 +1,12 @@
 // extern "C" boundary of the library (declared in include/sn.h).  Every entry
 // point catches C++ exceptions and turns them into a status, so nothing but
 // an sn_status crosses the ABI.
+#include <array>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
 #include <fstream>
+#include <map>
 #include <sstream>
 #include <string>
 
@@ -659,29 +661,47 @@ sn_status sn_load_plan(sn_graph *gg, const char *path) {
             !read_int_array(doc, "candidates", cands) || !read_int_array(doc, "adapt_cost", ac) ||
             !read_int_array(doc, "path", pth))
             return fail(SN_EINVAL, "sn_load_plan: malformed plan file");
-        if (nl != g->n_layers() || ns != g->n_schemas() || ne != (int64_t)g->edges.size() ||
-            nc != (int64_t)g->cands.size() || cands.size() != (size_t)nc * 5 || ac.size() != g->adapt_cost.size())
+        if (nl != g->n_layers() || ns != g->n_schemas() || ne != (int64_t)g->edges.size() || nc < 0 ||
+            cands.size() != (size_t)nc * 5 || ac.size() != g->adapt_cost.size())
             return fail(SN_EINVAL, "sn_load_plan: plan describes a different net");
-        for (size_t c = 0; c < g->cands.size(); ++c) {
-            const Candidate &k = g->cands[c];
-            if (cands[5 * c] != k.routine || cands[5 * c + 1] != k.variant || cands[5 * c + 2] != k.schema ||
-                cands[5 * c + 3] != k.layer)
-                return fail(SN_EINVAL, "sn_load_plan: candidate list differs");
+        // the file's candidates, in order, among the graph's: a build with more
+        // routines or routine parameters than the one that wrote the file keeps
+        // its own as not profiled (infinite cost)
+        std::vector<int32_t> at((size_t)nc);
+        {
+            typedef std::array<int64_t, 4> Key;  // routine, variant, schema, layer
+            std::map<Key, std::vector<int32_t>> where;  // several when a routine writes several schemas
+            std::map<Key, size_t> used;
+            for (size_t c = 0; c < g->cands.size(); ++c) {
+                const Candidate &k = g->cands[c];
+                where[Key{k.routine, k.variant, k.schema, k.layer}].push_back((int32_t)c);
+            }
+            for (size_t c = 0; c < (size_t)nc; ++c) {
+                const Key k{cands[5 * c], cands[5 * c + 1], cands[5 * c + 2], cands[5 * c + 3]};
+                const auto it = where.find(k);
+                const size_t i = used[k]++;
+                if (it == where.end() || i >= it->second.size())
+                    return fail(SN_EINVAL, "sn_load_plan: candidate list differs");
+                at[c] = it->second[i];
+            }
         }
+        std::vector<int32_t> path;
         if (!pth.empty()) {
             if ((int64_t)pth.size() != nl) return fail(SN_EINVAL, "sn_load_plan: bad path length");
-            for (int32_t i = 0; i < g->n_layers(); ++i)
-                if (pth[i] < g->cand_begin[i] || pth[i] >= g->cand_begin[i + 1])
+            for (int32_t i = 0; i < g->n_layers(); ++i) {
+                const int32_t c = pth[i] < 0 || pth[i] >= nc ? -1 : at[(size_t)pth[i]];
+                if (c < g->cand_begin[i] || c >= g->cand_begin[i + 1])
                     return fail(SN_EINVAL, "sn_load_plan: path candidate out of range");
+                path.push_back(c);
+            }
         }
-        for (size_t c = 0; c < g->cands.size(); ++c) g->cands[c].cost = cands[5 * c + 4];
+        for (Candidate &k : g->cands) k.cost = kInf;
+        for (size_t c = 0; c < at.size(); ++c) g->cands[at[c]].cost = cands[5 * c + 4];
         for (size_t i = 0; i < ac.size(); ++i) g->adapt_cost[i] = ac[i];
-        if (!pth.empty()) {
-            g->path_cand.assign(pth.begin(), pth.end());
+        g->has_path = !path.empty();
+        if (g->has_path) {
+            g->path_cand = path;
             g->path_total = total;
-            g->has_path = true;
-        } else {
-            g->has_path = false;
         }
         invalidate_plan(g);
         return SN_OK;

@@ -79,14 +79,20 @@ constexpr int kSmCount = 152;  // GB300; only used to decide which K splits to o
 // a_blocks > 0: the space-to-depth formulation (a 1x1 layer of a_blocks x 64
 // "channels" over a caller-laid-out A): implicit tiles only, BN = 64, one
 // CTA per tile, all a_blocks blocks in one stage
-static std::vector<Config> configs(const Layer &l, const Shape &in, sn_schema s, int a_blocks = 0) {
+// odd: stride 2 on an odd extent (the conv2/igemm_tc_odd routine), and only
+// that: the sub-lattice maps take any extent, which saves such layers the
+// im2col matrix, or the direct kernel where a residual joins them (5x5, 72 ->
+// 120 channels, 5 x 35 x 35 fp16 NCHW in and out: 22.5 us a pass against 69.7
+// through im2col)
+static std::vector<Config> configs(const Layer &l, const Shape &in, sn_schema s, int a_blocks = 0, bool odd = false) {
     std::vector<Config> out;
     const sn_conv_params &c = l.conv;
     if (l.type != SN_L_CONV2 || c.groups != 1) return out;
     if (s.dtype == SN_F32 || s.layout != SN_NHWC) return out;
     if (c.c_in % 8 || c.c_out % 8 || c.c_out > MAX_K) return out;
     if (c.sh != c.sw || (c.sh != 1 && c.sh != 2)) return out;
-    if (c.sh == 2 && (in.h % 2 || in.w % 2 || in.h < 2 || in.w < 2)) return out;
+    if (c.sh == 2 && (in.h < 2 || in.w < 2)) return out;  // each sub-lattice has a row and a column
+    if (odd != (c.sh == 2 && (in.h % 2 || in.w % 2))) return out;
     const int K = c.c_out;
     const int kiters = c.kh * c.kw * ((c.c_in + BK - 1) / BK);
     std::vector<int> bns;
@@ -254,8 +260,8 @@ static std::vector<Config> configs(const Layer &l, const Shape &in, sn_schema s,
 
 }  // namespace tc
 
-int32_t conv_tc_variants(const Layer &l, const Shape &in, sn_schema s) {
-    return (int32_t)tc::configs(l, in, s).size();
+int32_t conv_tc_variants(const Layer &l, const Shape &in, sn_schema s, bool odd) {
+    return (int32_t)tc::configs(l, in, s, 0, odd).size();
 }
 
 // The tile shape a layer takes inside a chained launch (one CTA per tile of
@@ -289,8 +295,8 @@ bool conv_tc_chain_shape(const Layer &l, const Shape &in, sn_schema s, int32_t v
 // the routine parameters of variant v for a layer, spelled out: output-channel
 // tile, CTAs per tile, channel blocks per stage, 128-row halves per tile, K
 // split, weight-stationary B, cluster K split, and the pixel tiling
-std::string conv_tc_config_desc(const Layer &l, const Shape &in, sn_schema s, int32_t v, int32_t a_blocks) {
-    const std::vector<tc::Config> cfgs = tc::configs(l, in, s, a_blocks);
+std::string conv_tc_config_desc(const Layer &l, const Shape &in, sn_schema s, int32_t v, bool odd) {
+    const std::vector<tc::Config> cfgs = tc::configs(l, in, s, 0, odd);
     if (v < 0 || v >= (int)cfgs.size()) return "?";
     const tc::Config &c = cfgs[v];
     char b[160];
@@ -304,13 +310,13 @@ std::string conv_tc_config_desc(const Layer &l, const Shape &in, sn_schema s, in
     return b;
 }
 
-bool conv_tc_nchw_ok(const Layer &l, const Shape &in, sn_schema s, int32_t v) {
-    const std::vector<tc::Config> cfgs = tc::configs(l, in, s);
+bool conv_tc_nchw_ok(const Layer &l, const Shape &in, sn_schema s, int32_t v, bool odd) {
+    const std::vector<tc::Config> cfgs = tc::configs(l, in, s, 0, odd);
     return v >= 0 && v < (int)cfgs.size() && cfgs[v].ksplit == 1 && !cfgs[v].sk;
 }
 
-size_t conv_tc_ws(const Layer &l, const Shape &in, sn_schema s, int32_t v, int32_t a_blocks) {
-    const std::vector<tc::Config> cfgs = tc::configs(l, in, s, a_blocks);
+size_t conv_tc_ws(const Layer &l, const Shape &in, sn_schema s, int32_t v, int32_t a_blocks, bool odd) {
+    const std::vector<tc::Config> cfgs = tc::configs(l, in, s, a_blocks, odd);
     if (v < 0 || v >= (int)cfgs.size()) return 0;
     // stream-K: two fp32 partial-tile slots per CTA, at most one CTA per SM
     if (cfgs[v].sk) return (size_t)2 * num_sms() * tc::BM * cfgs[v].BN * sizeof(float);
@@ -328,7 +334,7 @@ cudaError_t conv_tc(const LaunchArgs &a) {
     using namespace tc;
     const Layer &l = *a.layer;
     const Shape &in = a.in_shapes[0];
-    const std::vector<Config> cfgs = configs(l, in, a.schema, a.a_blocks);
+    const std::vector<Config> cfgs = configs(l, in, a.schema, a.a_blocks, a.routine == R_CONV_TC_ODD);
     if (a.variant < 0 || a.variant >= (int)cfgs.size()) return cudaErrorInvalidValue;
     const Config cf = cfgs[a.variant];
     const sn_conv_params &c = l.conv;
@@ -444,8 +450,10 @@ cudaError_t conv_tc(const LaunchArgs &a) {
         } else {
             for (int bh = 0; bh < 2; ++bh)
                 for (int bw = 0; bw < 2; ++bw) {
+                    // an odd extent's even sub-lattice has one more row or column than its odd one
                     const char *base = static_cast<const char *>(a.in[0]) + ((int64_t)bh * p.W + bw) * p.C * es;
-                    const uint64_t dims[5] = {c0dim, (uint64_t)(p.W / 2), (uint64_t)(p.H / 2), (uint64_t)p.N, CB};
+                    const uint64_t dims[5] = {c0dim, (uint64_t)((p.W - bw + 1) / 2), (uint64_t)((p.H - bh + 1) / 2),
+                                              (uint64_t)p.N, CB};
                     const uint64_t str[4] = {2 * p.C * es, 2 * (uint64_t)p.W * p.C * es,
                                              (uint64_t)p.H * p.W * p.C * es, 128};
                     if (!encode(&mA[bh * 2 + bw], dt, blk ? 5 : 4, base, dims, str, box))
@@ -581,7 +589,10 @@ static int64_t im2col_kpad(const Layer &l) {
 }
 
 // im2col -> GEMM: for layers the implicit routine cannot take (few input
-// channels such as an RGB stem, odd sizes with stride 2)
+// channels such as an RGB stem), and beside it for stride 2 on odd extents
+// (conv2/igemm_tc_odd), where a large kernel over few channels packs into
+// fewer 64-value K steps than the implicit routine's one 64-channel block per
+// tap (C = 8, 5x5: 4 against 25)
 int32_t conv_im2col_tc_variants(const Layer &l, const Shape &in, sn_schema s) {
     const sn_conv_params &c = l.conv;
     if (l.type != SN_L_CONV2 || c.groups != 1 || s.dtype == SN_F32 || s.layout != SN_NHWC) return 0;

@@ -19,6 +19,7 @@ const char *routine_name(int32_t r) {
     case R_CONV_WINO4: return "conv2/wino_f4x4_3x3";
     case R_CONV_WINO6: return "conv2/wino_f6x6_3x3";
     case R_CONV_TC: return "conv2/igemm_tc";
+    case R_CONV_TC_ODD: return "conv2/igemm_tc_odd";
     case R_DW_DIRECT: return "dwconv2/direct";
     case R_MAXPOOL: return "maxpool/direct";
     case R_GAP: return "gap/reduce";
@@ -40,6 +41,7 @@ const char *variant_name(int32_t r, int32_t v) {
     case R_CONV_WINO: return v == 0 ? "gemm=simt" : "gemm=tc";
     case R_DW_DIRECT: return v == 0 ? "nhwc:window|nchw:rows" : v == 1 ? "nhwc:tma_rows|nchw:plane_tile" : "nhwc:band";
     case R_CONV_TC:
+    case R_CONV_TC_ODD:
     case R_CONV_IM2COL_TC:
     case R_CONV_S2D_TC:
     case R_DENSE_TC: return k::conv_tc_variant_name(v);
@@ -56,8 +58,8 @@ std::string candidate_desc(const Graph &g, int32_t cand) {
     std::vector<Shape> in;
     for (int32_t j : L.inputs) in.push_back(g.layers[j].out);
     std::string params;
-    if (c.routine == R_CONV_TC && !in.empty())
-        params = k::conv_tc_config_desc(L, in[0], g.schemas[c.schema], c.variant);
+    if ((c.routine == R_CONV_TC || c.routine == R_CONV_TC_ODD) && !in.empty())
+        params = k::conv_tc_config_desc(L, in[0], g.schemas[c.schema], c.variant, c.routine == R_CONV_TC_ODD);
     else
         params = variant_name(c.routine, c.variant);
     if (!params.empty()) d += " [" + params + "]";
@@ -87,7 +89,7 @@ int32_t routine_variants(int32_t r, const Layer &l, const std::vector<Shape> &in
     const sn_conv_params &p = l.conv;
     // a conv2 with a residual input is served by the routines whose epilogue
     // adds it: direct and the tensor-core implicit GEMM
-    if (is_conv(l) && in.size() == 2 && r != R_CONV_DIRECT && r != R_CONV_TC) return 0;
+    if (is_conv(l) && in.size() == 2 && r != R_CONV_DIRECT && r != R_CONV_TC && r != R_CONV_TC_ODD) return 0;
     switch (r) {
     case R_CONV_DIRECT:
         return is_conv(l) ? 1 : 0;
@@ -102,6 +104,8 @@ int32_t routine_variants(int32_t r, const Layer &l, const std::vector<Shape> &in
                    : 0;
     case R_CONV_TC:
         return is_conv(l) ? k::conv_tc_variants(l, in[0], s) : 0;
+    case R_CONV_TC_ODD:
+        return is_conv(l) ? k::conv_tc_variants(l, in[0], s, true) : 0;
     case R_DW_DIRECT:
         if (l.type != SN_L_DWCONV2) return 0;
         // NHWC 3x3 of small maps: a third parameter, the shared-memory band kernel
@@ -132,7 +136,7 @@ size_t routine_workspace(int32_t r, int32_t v, const Layer &l, const std::vector
     if (r == R_CONV_WINO) return k::conv_wino_ws(l, in[0], s);
     if (r == R_CONV_WINO4) return k::conv_wino4_ws(l, in[0], s);
     if (r == R_CONV_WINO6) return k::conv_wino6_ws(l, in[0], s);
-    if (r == R_CONV_TC) return k::conv_tc_ws(l, in[0], s, v);
+    if (r == R_CONV_TC || r == R_CONV_TC_ODD) return k::conv_tc_ws(l, in[0], s, v, 0, r == R_CONV_TC_ODD);
     if (r == R_CONV_IM2COL_TC) return k::conv_im2col_tc_ws(l, in[0], s, v);
     if (r == R_DENSE_TC) return k::dense_tc_ws(l, in[0], s, v);
     if (r == R_CONV_S2D_TC) return k::conv_s2d_tc_ws(l, in[0], s, v);
@@ -156,7 +160,8 @@ static int weight_format_of(int32_t r, sn_schema s) {
     case R_CONV_WINO: return k::W_WINO;
     case R_CONV_WINO4: return k::W_WINO4;
     case R_CONV_WINO6: return k::W_WINO6;
-    case R_CONV_TC: return k::W_KRSC;
+    case R_CONV_TC:
+    case R_CONV_TC_ODD: return k::W_KRSC;
     case R_DW_DIRECT: return s.layout == SN_NCHW ? k::W_KCRS : k::W_RSCK;
     case R_DENSE: return k::W_KCRS;
     case R_CONV_IM2COL_TC: return k::W_KRSC_PAD64;
@@ -240,7 +245,7 @@ int32_t kernels_per_launch(int32_t r, int32_t v, const Layer &l, const std::vect
     if (s.dtype == SN_QI8) return 1;
     // a K-split tensor-core GEMM adds its reduction kernel (it is the only
     // variant with a workspace)
-    const int split = (r == R_CONV_TC || r == R_CONV_IM2COL_TC || r == R_DENSE_TC || r == R_CONV_S2D_TC) &&
+    const int split = (r == R_CONV_TC || r == R_CONV_TC_ODD || r == R_CONV_IM2COL_TC || r == R_DENSE_TC || r == R_CONV_S2D_TC) &&
                       routine_workspace(r, v, l, in, s) >
                           (r == R_CONV_IM2COL_TC ? k::conv_im2col_tc_ws(l, in[0], s, -1)
                            : r == R_CONV_S2D_TC  ? k::conv_s2d_tc_ws(l, in[0], s, -1)
@@ -253,7 +258,8 @@ int32_t kernels_per_launch(int32_t r, int32_t v, const Layer &l, const std::vect
 std::vector<sn_schema> fused_outputs(int32_t r, const Layer &l, sn_schema s) {
     // the tensor-core convolution can write its NHWC result straight in the
     // NCHW layout of the same dtype (the permutation fused into its epilogue)
-    if (r == R_CONV_TC && l.type == SN_L_CONV2 && s.layout == SN_NHWC && (s.dtype == SN_F16 || s.dtype == SN_BF16))
+    if ((r == R_CONV_TC || r == R_CONV_TC_ODD) && l.type == SN_L_CONV2 && s.layout == SN_NHWC &&
+        (s.dtype == SN_F16 || s.dtype == SN_BF16))
         return {{s.dtype, SN_NCHW}};
     // the space-to-depth stem reads either layout and its GEMM writes either
     // (NHWC from its TMA store, NCHW from the NCHW epilogue)
@@ -280,7 +286,8 @@ bool fused_variant_ok(int32_t r, const Layer &l, const std::vector<Shape> &in, s
     if (s.dtype == SN_QI8) return true;
     // the NCHW writer drains each tile in one CTA's epilogue: no K split
     // through fp32 partials, no stream-K parts
-    if (r == R_CONV_TC && !in.empty()) return k::conv_tc_nchw_ok(l, in[0], s, v);
+    if ((r == R_CONV_TC || r == R_CONV_TC_ODD) && !in.empty())
+        return k::conv_tc_nchw_ok(l, in[0], s, v, r == R_CONV_TC_ODD);
     if (r == R_CONV_S2D_TC) return true;  // one-CTA tiles without a K split
     return false;
 }
@@ -348,7 +355,8 @@ sn_status launch_routine(const LaunchArgs &a) {
     case R_CONV_WINO: e = k::conv_wino(a); break;
     case R_CONV_WINO4: e = k::conv_wino4(a); break;
     case R_CONV_WINO6: e = k::conv_wino6(a); break;
-    case R_CONV_TC: e = k::conv_tc(a); break;
+    case R_CONV_TC:
+    case R_CONV_TC_ODD: e = k::conv_tc(a); break;
     case R_DW_DIRECT: e = k::dwconv(a); break;
     case R_MAXPOOL: e = k::maxpool(a); break;
     case R_GAP: e = k::gap(a); break;

@@ -71,7 +71,8 @@ enum RoutineId : int32_t {
     R_CONV_WINO4 = 15,   // Winograd F(4x4,3x3) childnet (fp32 transformed filters)
     R_CONV_DP4A = 16,    // qint8 implicit GEMM with dp4a (NHWC)
     R_CONV_WINO6 = 17,   // Winograd F(6x6,3x3) childnet (fp32 transformed filters)
-    R_COUNT = 18
+    R_CONV_TC_ODD = 18,  // the tensor-core implicit GEMM with stride 2 on odd extents
+    R_COUNT = 19
 };
 
 // -------------------------------------------------------------------------
@@ -348,12 +349,14 @@ cudaError_t conv_im2col_tc_stage(const LaunchArgs &a, int stage);
 cudaError_t conv_s2d_tc_stage(const LaunchArgs &a, int stage);
 size_t conv_wino6_ws(const Layer &l, const Shape &in, sn_schema s);
 cudaError_t conv_tc(const LaunchArgs &a);
-int32_t conv_tc_variants(const Layer &l, const Shape &in, sn_schema s);
-size_t conv_tc_ws(const Layer &l, const Shape &in, sn_schema s, int32_t v, int32_t a_blocks = 0);  // K-split partials
+// odd: stride 2 on an odd extent (conv2/igemm_tc_odd), whose configurations are listed apart
+int32_t conv_tc_variants(const Layer &l, const Shape &in, sn_schema s, bool odd = false);
+size_t conv_tc_ws(const Layer &l, const Shape &in, sn_schema s, int32_t v, int32_t a_blocks = 0,
+                  bool odd = false);  // K-split partials
 size_t dense_tc_ws(const Layer &l, const Shape &in, sn_schema s, int32_t v);
 const char *conv_tc_variant_name(int32_t v);
-bool conv_tc_nchw_ok(const Layer &l, const Shape &in, sn_schema s, int32_t v);  // variant v can write NCHW
-std::string conv_tc_config_desc(const Layer &l, const Shape &in, sn_schema s, int32_t v, int32_t a_blocks = 0);
+bool conv_tc_nchw_ok(const Layer &l, const Shape &in, sn_schema s, int32_t v, bool odd = false);  // v can write NCHW
+std::string conv_tc_config_desc(const Layer &l, const Shape &in, sn_schema s, int32_t v, bool odd = false);
 // chained launches of consecutive tensor-core convolutions
 bool conv_tc_chain_shape(const Layer &l, const Shape &in, sn_schema s, int32_t v, bool *implicit, int *bn, int *kb,
                          int *bw, int *bh, int *bni);

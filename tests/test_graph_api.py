@@ -206,3 +206,48 @@ def test_candidate_descriptors():
     assert all("bn=" in d and "tile=" in d for d in tc)
     with pytest.raises(SnError):
         g.candidate_desc(len(t["cost"]))
+
+
+def test_plan_file_of_a_build_with_fewer_candidates(tmp_path):
+    """A plan file that lists a subset of the graph's candidates (written before
+    a routine or a routine parameter was added) loads: the path names the same
+    routines, the candidates it does not list stay unprofiled."""
+    import json
+
+    import synth
+    from paper_2110_06037_gb300._sn import COST_INF
+    layer = synth.conv(16, 16, 3, 1)
+    layer["weight"] = np.ones((16, 16, 3, 3), np.float32)
+
+    def make():
+        sch = [("f16", "nchw"), ("f16", "nhwc")]
+        return build_graph([dict(layer, inputs=[-1])], (1, 16, 8, 8), sch[0], sch[0], sch)
+
+    g = make()
+    t = g.cost_table()
+    t["cost"] = np.arange(len(t["cost"])) + 100
+    t["adapt"][t["adapt"] > 0] = 7
+    g.set_cost_table(t)
+    mine = np.flatnonzero(t["layer"] == 1)
+    path = [int(np.flatnonzero(t["layer"] == 0)[0]), int(mine[-1]), int(np.flatnonzero(t["layer"] == 2)[0])]
+    g.set_path(path)
+    f = tmp_path / "plan.json"
+    g.save_plan(f)
+    doc = json.loads(f.read_text())
+    drop = int(mine[1])  # the file never heard of this candidate
+    del doc["candidates"][drop]
+    doc["n_candidates"] -= 1
+    doc["path"] = [c - (c > drop) for c in doc["path"]]
+    f.write_text(json.dumps(doc))
+    g2 = make()
+    g2.load_plan(f)
+    t2 = g2.cost_table()
+    want = np.asarray(t["cost"]).copy()
+    want[drop] = COST_INF
+    assert list(t2["cost"]) == list(want)
+    g2.save_plan(tmp_path / "back.json")
+    assert json.loads((tmp_path / "back.json").read_text())["path"] == path
+    doc["candidates"][drop][1] = 9999  # a candidate that this build does not have
+    f.write_text(json.dumps(doc))
+    with pytest.raises(Exception):
+        g2.load_plan(f)
