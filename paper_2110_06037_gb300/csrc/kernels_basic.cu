@@ -1229,44 +1229,66 @@ __global__ void gap_nchw(const T *__restrict__ x, T *__restrict__ y, int64_t NC,
     }
 }
 
-// NHWC, 16-byte channel vectors: a block of 32 channel vectors x 8 pixel
-// slices per (image, 32-vector group); each thread sums its slice's pixels in
-// f32, the block adds the 8 slices in order through shared memory
+// NHWC, 16-byte channel vectors: a block owns eight of them (128 contiguous
+// bytes of every pixel) of one image; the other thread axis cuts the pixels
+// into blockDim / 8 slices, each summed in f32 with four loads in flight.  The
+// four slices of a warp are added by shuffles, the warps in order through
+// shared memory, so the sum does not depend on timing.  What bounds the kernel
+// is the chain of load latencies of one slice, not bytes: at 28 x 28 one block
+// of 32 vectors x 8 slices per image walked 98 pixels per thread and took
+// longer than an adapt plus the NCHW kernel (8 x 28 x 28 x 120 bf16, each op
+// between timing nodes of a replayed net, an empty op reading about 5 us: 15.5
+// us for the pair, 9.1 us for this kernel).
 template <typename T>
-__global__ void __launch_bounds__(256) gap_nhwc_vec(const T *__restrict__ x, T *__restrict__ y, int C, int HW) {
+__global__ void __launch_bounds__(1024) gap_nhwc_vec(const T *__restrict__ x, T *__restrict__ y, int C, int HW) {
     griddep_launch();
     griddep_wait();
     constexpr int E = 16 / sizeof(T);
-    __shared__ float part[8][32][E + 1];
-    const int cvl = threadIdx.x & 31, sl = threadIdx.x >> 5;
+    __shared__ float part[32][8 * E + 1];
+    const int v = threadIdx.x & 7, sl = threadIdx.x >> 3, slices = blockDim.x >> 3;
     const int n = blockIdx.y;
     const int CV = C / E;
-    const int cv = blockIdx.x * 32 + cvl;
+    const int cv = blockIdx.x * 8 + v;
     float s[E];
 #pragma unroll
     for (int e = 0; e < E; ++e) s[e] = 0.f;
     if (cv < CV) {
         const T *xn = x + (size_t)n * HW * C + (size_t)cv * E;
-        for (int p = sl; p < HW; p += 8) {
-            const uint4 v = *reinterpret_cast<const uint4 *>(xn + (size_t)p * C);
-            const T *pv = reinterpret_cast<const T *>(&v);
+        int p = sl;
+        for (; p + 3 * slices < HW; p += 4 * slices) {
+            uint4 q[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) q[k] = *reinterpret_cast<const uint4 *>(xn + (size_t)(p + k * slices) * C);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const T *pv = reinterpret_cast<const T *>(&q[k]);
+#pragma unroll
+                for (int e = 0; e < E; ++e) s[e] += ldf<T>(pv + e);
+            }
+        }
+        for (; p < HW; p += slices) {
+            const uint4 q = *reinterpret_cast<const uint4 *>(xn + (size_t)p * C);
+            const T *pv = reinterpret_cast<const T *>(&q);
 #pragma unroll
             for (int e = 0; e < E; ++e) s[e] += ldf<T>(pv + e);
         }
     }
 #pragma unroll
-    for (int e = 0; e < E; ++e) part[sl][cvl][e] = s[e];
-    __syncthreads();
-    if (sl == 0 && cv < CV) {
-        uint4 o;
-        T *po = reinterpret_cast<T *>(&o);
+    for (int e = 0; e < E; ++e) {
+        s[e] += __shfl_xor_sync(0xffffffffu, s[e], 8);
+        s[e] += __shfl_xor_sync(0xffffffffu, s[e], 16);
+    }
+    const int warp = threadIdx.x >> 5;
+    if ((threadIdx.x & 31) < 8) {
 #pragma unroll
-        for (int e = 0; e < E; ++e) {
-            float t = 0.f;
-            for (int k = 0; k < 8; ++k) t += part[k][cvl][e];
-            po[e] = cvt<T>(t / (float)HW);
-        }
-        *reinterpret_cast<uint4 *>(y + (size_t)n * C + (size_t)cv * E) = o;
+        for (int e = 0; e < E; ++e) part[warp][v * E + e] = s[e];
+    }
+    __syncthreads();
+    const int c = threadIdx.x;  // channel within the block's 8 * E
+    if (c < 8 * E && blockIdx.x * 8 * E + c < C) {
+        float t = 0.f;
+        for (int k = 0; k < (int)(blockDim.x >> 5); ++k) t += part[k][c];
+        stf<T>(y + (size_t)n * C + blockIdx.x * 8 * E + c, t / (float)HW);
     }
 }
 
@@ -1293,7 +1315,10 @@ cudaError_t gap(const LaunchArgs &a) {
         else if ((i.c * (int64_t)sizeof(T)) % 16 == 0 && (uintptr_t)a.in[0] % 16 == 0 && (uintptr_t)a.out % 16 == 0 &&
                  i.n <= 65535 && i.h * i.w * i.c < ((int64_t)1 << 31)) {
             const int CV = (int)(i.c * (int64_t)sizeof(T) / 16);
-            launch_pdl(gap_nhwc_vec<T>, dim3((unsigned)((CV + 31) / 32), (unsigned)i.n), 256, 0, a.stream,
+            // about four pixels a thread where the map has them, within 64 to 1024 threads
+            int threads = 64;
+            while (threads < 1024 && (int64_t)threads / 8 * 4 < i.h * i.w) threads *= 2;
+            launch_pdl(gap_nhwc_vec<T>, dim3((unsigned)((CV + 7) / 8), (unsigned)i.n), threads, 0, a.stream,
                        (const T *)a.in[0], (T *)a.out, (int)i.c, (int)(i.h * i.w));
         } else
             launch_pdl(gap_nhwc<T>, grid_for(i.n * i.c, 256), 256, 0, a.stream, (const T *)a.in[0], (T *)a.out, i.n,
@@ -1347,28 +1372,30 @@ cudaError_t add(const LaunchArgs &a) {
 }
 
 // per-channel scale: y[n,c,h,w] = act(x[n,c,h,w] * s[n,c]).  NHWC, 16-byte
-// vectors when C allows: one thread per 8 (16-bit) or 4 (fp32) channels of a
-// pixel; otherwise one thread per element, (n, c) from the layout.
+// vectors when C allows: the grid's y axis walks the images, its x axis the
+// image's vectors, so the channel vector is one 32-bit division by a launch
+// constant away (64-bit divisions by CV and HW per vector were most of the
+// kernel's instructions).  Otherwise one thread per element, (n, c) from the
+// layout.
 template <typename T>
-__global__ void mul_nhwc_vec(const uint4 *__restrict__ x, const T *__restrict__ s, uint4 *__restrict__ y,
-                             int64_t pixels, int64_t HW, int CV, int act) {
+__global__ void __launch_bounds__(256) mul_nhwc_vec(const uint4 *__restrict__ x, const uint4 *__restrict__ s,
+                                                    uint4 *__restrict__ y, int N, uint32_t per_image, FastDiv fd_cv,
+                                                    int act) {
     griddep_launch();
     griddep_wait();
     constexpr int E = 16 / sizeof(T);
-    const int64_t total = pixels * CV;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t pix = i / CV;
-        const int cv = (int)(i - pix * CV);
-        const int64_t n = pix / HW;
-        const uint4 xv = x[i];
-        const uint4 sv = reinterpret_cast<const uint4 *>(s + n * (int64_t)CV * E)[cv];
-        uint4 o;
-        const T *px = reinterpret_cast<const T *>(&xv), *ps = reinterpret_cast<const T *>(&sv);
-        T *po = reinterpret_cast<T *>(&o);
+    for (int n = blockIdx.y; n < N; n += gridDim.y) {
+        const uint4 *xn = x + (size_t)n * per_image, *sn = s + (size_t)n * fd_cv.d;
+        uint4 *yn = y + (size_t)n * per_image;
+        for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < per_image; i += gridDim.x * blockDim.x) {
+            const uint4 xv = xn[i], sv = sn[i - fdiv(i, fd_cv) * fd_cv.d];
+            uint4 o;
+            const T *px = reinterpret_cast<const T *>(&xv), *ps = reinterpret_cast<const T *>(&sv);
+            T *po = reinterpret_cast<T *>(&o);
 #pragma unroll
-        for (int e = 0; e < E; ++e) po[e] = cvt<T>(act_apply(ldf<T>(px + e) * ldf<T>(ps + e), act));
-        y[i] = o;
+            for (int e = 0; e < E; ++e) po[e] = cvt<T>(act_apply(ldf<T>(px + e) * ldf<T>(ps + e), act));
+            yn[i] = o;
+        }
     }
 }
 
@@ -1390,10 +1417,11 @@ cudaError_t mul(const LaunchArgs &a) {
     SN_DT_SWITCH(a.schema.dtype, T, {
         const int64_t cb = o.c * (int64_t)sizeof(T);
         if (a.schema.layout == SN_NHWC && cb % 16 == 0 && (uintptr_t)a.in[0] % 16 == 0 &&
-            (uintptr_t)a.in[1] % 16 == 0 && (uintptr_t)a.out % 16 == 0)
-            launch_pdl(mul_nhwc_vec<T>, grid_for(n * (int64_t)sizeof(T) / 16, 256), 256, 0, a.stream,
-                       (const uint4 *)a.in[0], (const T *)a.in[1], (uint4 *)a.out, o.n * HW, HW, (int)(cb / 16),
-                       a.layer->act);
+            (uintptr_t)a.in[1] % 16 == 0 && (uintptr_t)a.out % 16 == 0 && HW * (cb / 16) < ((int64_t)1 << 30) &&
+            o.n < ((int64_t)1 << 31))
+            launch_pdl(mul_nhwc_vec<T>, dim3(grid_for(HW * (cb / 16), 256, 152LL * 8), (unsigned)std::min<int64_t>(o.n, 65535)),
+                       256, 0, a.stream, (const uint4 *)a.in[0], (const uint4 *)a.in[1], (uint4 *)a.out, (int)o.n,
+                       (uint32_t)(HW * (cb / 16)), make_fastdiv((uint32_t)(cb / 16)), a.layer->act);
         else if (a.schema.layout == SN_NHWC)
             launch_pdl(mul_kernel<T, true>, grid_for(n, 256), 256, 0, a.stream, (const T *)a.in[0],
                        (const T *)a.in[1], (T *)a.out, n, o.c, HW, a.layer->act);
@@ -1421,13 +1449,80 @@ __global__ void dense_kernel(const T *__restrict__ x, const T *__restrict__ w, c
     }
 }
 
-cudaError_t dense(const LaunchArgs &a) {
-    const Shape &i = a.in_shapes[0];
-    const int64_t N = i.n, IN = a.layer->dense_in, OUT = a.layer->dense_out;
-    SN_DT_SWITCH(a.schema.dtype, T,
-                 launch_pdl(dense_kernel<T>, grid_for(N * OUT * 32, 256), 256, 0, a.stream, 
-                     (const T *)a.in[0], (const T *)a.wt, a.bias, (T *)a.out, N, IN, OUT, a.layer->act));
+// 16-byte vectors along the input features: one warp per (output feature, NB
+// images), the weight row loaded once for them, U vectors in flight.  The
+// reduction order differs from the scalar kernel's; each is one f32 sum.
+template <typename T, int NB, int U>
+__global__ void __launch_bounds__(256) dense_vec_kernel(const uint4 *__restrict__ x, const uint4 *__restrict__ w,
+                                                        const float *__restrict__ bias, T *__restrict__ y, int N,
+                                                        int IV, int OUT, int act) {
+    griddep_launch();
+    griddep_wait();
+    constexpr int E = 16 / sizeof(T);
+    const int lane = threadIdx.x & 31;
+    const int o = blockIdx.x * 8 + (threadIdx.x >> 5);
+    const int n0 = blockIdx.y * NB;
+    if (o >= OUT) return;
+    const uint4 *wr = w + (size_t)o * IV;
+    float s[NB];
+#pragma unroll
+    for (int b = 0; b < NB; ++b) s[b] = 0.f;
+    for (int i = lane; i < IV; i += 32 * U) {
+        uint4 wv[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) wv[u] = i + 32 * u < IV ? wr[i + 32 * u] : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+        for (int b = 0; b < NB; ++b) {
+            const uint4 *xr = x + (size_t)min(n0 + b, N - 1) * IV;
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (i + 32 * u >= IV) break;  // a NaN or infinity of x must not meet a zero weight
+                const uint4 xv = xr[i + 32 * u];
+                const T *px = reinterpret_cast<const T *>(&xv), *pw = reinterpret_cast<const T *>(&wv[u]);
+#pragma unroll
+                for (int e = 0; e < E; ++e) s[b] = fmaf(ldf<T>(px + e), ldf<T>(pw + e), s[b]);
+            }
+        }
+    }
+#pragma unroll
+    for (int b = 0; b < NB; ++b)
+        for (int k = 16; k > 0; k >>= 1) s[b] += __shfl_xor_sync(0xffffffffu, s[b], k);
+    if (lane < NB && n0 + lane < N) {
+        float v = s[0];
+#pragma unroll
+        for (int b = 1; b < NB; ++b)
+            if (lane == b) v = s[b];
+        stf<T>(y + (size_t)(n0 + lane) * OUT + o, act_apply(v + bias[o], act));
+    }
+}
+
+template <typename T>
+static cudaError_t dense_t(const LaunchArgs &a) {
+    const int64_t N = a.in_shapes[0].n, IN = a.layer->dense_in, OUT = a.layer->dense_out;
+    constexpr int E = 16 / (int)sizeof(T);
+    if (IN % E || (uintptr_t)a.in[0] % 16 || (uintptr_t)a.wt % 16 || N > 65535) {
+        launch_pdl(dense_kernel<T>, grid_for(N * OUT * 32, 256), 256, 0, a.stream, (const T *)a.in[0],
+                   (const T *)a.wt, a.bias, (T *)a.out, N, IN, OUT, a.layer->act);
+        return cudaGetLastError();
+    }
+    // images per warp: their weight row is read once, but a warp per (feature,
+    // image) fills the GPU better while that is under two warps a scheduler
+    // (152 SMs x 8)
+    const int nb = N >= 8 && N * OUT >= 8 * 1216 ? 8 : N >= 2 && N * OUT >= 2 * 1216 ? 2 : 1;
+    const dim3 g((unsigned)((OUT + 7) / 8), (unsigned)((N + nb - 1) / nb));
+    auto go = [&](auto kern) {
+        launch_pdl(kern, g, 256, 0, a.stream, (const uint4 *)a.in[0], (const uint4 *)a.wt, a.bias, (T *)a.out, (int)N,
+                   (int)(IN / E), (int)OUT, (int)a.layer->act);
+    };
+    if (nb == 8) go(dense_vec_kernel<T, 8, 2>);
+    else if (nb == 2) go(dense_vec_kernel<T, 2, 4>);
+    else go(dense_vec_kernel<T, 1, 4>);
     return cudaGetLastError();
+}
+
+cudaError_t dense(const LaunchArgs &a) {
+    SN_DT_SWITCH(a.schema.dtype, T, return dense_t<T>(a));
+    return cudaErrorInvalidValue;
 }
 
 }  // namespace k

@@ -1,0 +1,83 @@
+"""The vectorised pooling, scale and dense kernels (float and qint8) and the
+qint8 depthwise kernel at the sizes where their splits can go wrong: fewer
+pixels or features than a block has slices, a channel count that ends inside a
+block's vectors, column counts that are no multiple of a thread's columns, one
+and several images per warp, and sizes that fall back to the general kernels."""
+import zlib
+
+import numpy as np
+import pytest
+
+import synth
+from oracle.net import run_layer
+from paper_2110_06037_gb300 import build_graph
+
+from gpu_helpers import TOL, from_device, maxrel, stored_values, to_device
+from test_gpu_q8 import F32, _out_scales, _ref_codes, conv_layer, run_q8
+
+pytestmark = pytest.mark.gpu
+
+
+def run_float(layers, x, schema):
+    import torch
+    g = build_graph(layers, x.shape, schema, schema, [schema])
+    t = g.cost_table()
+    g.set_path([int(np.flatnonzero(t["layer"] == i)[0]) for i in range(t["n_layers"])])
+    y = g.run(to_device(x, schema))
+    torch.cuda.synchronize()
+    return from_device(y, schema)
+
+
+@pytest.mark.parametrize("n,c,h,w", [(1, 8, 1, 1), (2, 72, 3, 5), (3, 120, 28, 28), (1, 200, 31, 33), (2, 10, 9, 9)])
+@pytest.mark.parametrize("dt", ["f32", "f16", "bf16"])
+def test_gap_then_scale(n, c, h, w, dt):
+    rng = np.random.default_rng(zlib.crc32(repr((n, c, h, w, dt)).encode()))
+    x = rng.standard_normal((n, c, h, w)).astype(np.float32)
+    xs = stored_values(x, dt)
+    net = [dict(synth.gap(), inputs=[-1])]
+    pooled = run_layer(net[0], [xs], dt)
+    assert maxrel(run_float(net, x, (dt, "nhwc")), pooled) <= TOL[dt]
+    net.append(dict(synth.mul(act="none"), inputs=[-1, 0]))
+    assert maxrel(run_float(net, x, (dt, "nhwc")), run_layer(net[1], [xs, pooled], dt)) <= TOL[dt]
+
+
+@pytest.mark.parametrize("n,i,o", [(1, 8, 1), (1, 1032, 9), (9, 24, 120), (3, 520, 1001), (33, 264, 333), (2, 100, 7)])
+@pytest.mark.parametrize("dt", ["f32", "f16", "bf16"])
+def test_dense(n, i, o, dt):
+    rng = np.random.default_rng(zlib.crc32(repr((n, i, o, dt)).encode()))
+    x = rng.standard_normal((n, i, 1, 1)).astype(np.float32)
+    layer = dict(synth.dense(i, o, act="hsigmoid"), inputs=[-1])
+    layer["weight"] = (rng.standard_normal((o, i)) / np.sqrt(i)).astype(np.float32)
+    layer["bias"] = rng.standard_normal(o).astype(np.float32)
+    ref = run_layer(layer, [stored_values(x, dt)], dt)
+    assert maxrel(run_float([layer], x, (dt, "nhwc")), ref) <= TOL[dt]
+
+
+@pytest.mark.parametrize("ks,st", [(3, 1), (3, 2), (5, 1), (5, 2)])
+@pytest.mark.parametrize("c,h,w", [(4, 1, 1), (20, 7, 5), (36, 9, 18), (6, 8, 8)])
+@pytest.mark.parametrize("act", ["relu6", "hswish"])
+def test_q8_depthwise_vectors(ks, st, c, h, w, act):
+    rng = np.random.default_rng(zlib.crc32(repr((ks, st, c, h, w)).encode()))
+    layer = conv_layer(rng, c, c, ks, st, ks // 2, act=act, dw=True)
+    q_in = rng.integers(-127, 128, (3, c, h, w)).astype(np.int8)
+    s_in = F32(0.05)
+    scales = _out_scales([layer], q_in, s_in)
+    got, _ = run_q8([layer], q_in, s_in, scales, "nhwc", ["dwconv2/direct"])
+    assert np.array_equal(got, _ref_codes([layer], q_in, s_in, scales))
+
+
+@pytest.mark.parametrize("n,c,h,w", [(1, 4, 1, 1), (2, 36, 3, 5), (3, 48, 27, 29), (2, 6, 9, 9)])
+def test_q8_pool_gap_add_mul_vectors(n, c, h, w):
+    rng = np.random.default_rng(zlib.crc32(repr((n, c, h, w)).encode()))
+    q_in = rng.integers(-127, 128, (n, c, h, w)).astype(np.int8)
+    s_in = F32(0.03)
+    nets = [
+        [{"type": "maxpool", "inputs": [-1], "params": dict(kh=3, kw=3, sh=2, sw=2, ph=1, pw=1)}],
+        [{"type": "gap", "inputs": [-1]}],
+        [{"type": "add", "inputs": [-1, -1], "params": dict(act="hswish")}],
+        [{"type": "gap", "inputs": [-1]}, {"type": "mul", "inputs": [-1, 0], "params": dict(act="none")}],
+    ]
+    for layers in nets:
+        scales = _out_scales(layers, q_in, s_in)
+        got, _ = run_q8(layers, q_in, s_in, scales, "nhwc", [])
+        assert np.array_equal(got, _ref_codes(layers, q_in, s_in, scales)), layers[-1]["type"]
