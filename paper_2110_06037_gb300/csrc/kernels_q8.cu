@@ -12,6 +12,7 @@
 //
 // Integer dot products use dp4a (four int8 products added into an int32 per
 // instruction) on the CUDA cores.
+#include <algorithm>
 #include <cmath>
 #include <type_traits>
 
@@ -453,6 +454,94 @@ static bool scales_ok(const LaunchArgs &a, int n_in) {
     return out_dtype(a) != SN_QI8 || (a.qs_out > 0.0f && std::isfinite(a.qs_out));
 }
 
+// dwconv2 3x3 / 5x5, NHWC, dilation 1, C % 4 == 0: four channels (one word of
+// codes) and QB output columns per thread.  dp4a multiplies a word of four
+// channels by a weight word of which one byte is kept, so each multiply-add is
+// one instruction with no unpacking, and the input word of a column serves
+// every tap and output that reads it.  A warp reads 128 contiguous bytes.
+// Bound by instruction issue: QB x KS x KS x 4 dp4a plus 4 masks per tap,
+// against one scalar load, two conversions and a multiply-add per tap and
+// channel in the direct kernel (8 x 14 x 14 x 672, 3x3: 10.7 us against 34.8
+// between timing nodes of a replayed net, an empty op reading about 5 us).  The
+// sums are integers, so their order is free and the codes are the direct
+// kernel's.
+template <int KS, int SW, int QB, typename TO>
+__global__ void __launch_bounds__(256) q8_dw_nhwc_kernel(const int8_t *__restrict__ x, const int8_t *__restrict__ w,
+                                                         const float *__restrict__ ws, const float *__restrict__ bias,
+                                                         TO *__restrict__ y, ConvDims d, Q8Scales q, FastDiv fd_items,
+                                                         FastDiv fd_c4, FastDiv fd_P, uint32_t total) {
+    griddep_launch();
+    griddep_wait();
+    constexpr int WN = (QB - 1) * SW + KS;  // input columns that QB outputs read
+    const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= total) return;
+    const int rowi = (int)fdiv(t, fd_items);
+    const int it = (int)(t - (uint32_t)rowi * fd_items.d);
+    const int qb = (int)fdiv((uint32_t)it, fd_c4);
+    const int c0 = (it - qb * (int)fd_c4.d) * 4, q0 = qb * QB;
+    const int n = (int)fdiv((uint32_t)rowi, fd_P), p = rowi - n * d.P;
+    int acc[QB][4] = {};
+    const int w0 = q0 * SW - d.pw;
+#pragma unroll
+    for (int r = 0; r < KS; ++r) {
+        const int h = p * SW - d.ph + r;
+        if (h < 0 || h >= d.H) continue;
+        const int8_t *xr = x + (((int64_t)n * d.H + h) * d.W) * d.C + c0;
+        int win[WN];
+#pragma unroll
+        for (int i = 0; i < WN; ++i)
+            win[i] = (w0 + i >= 0 && w0 + i < d.W) ? *reinterpret_cast<const int *>(xr + (int64_t)(w0 + i) * d.C) : 0;
+#pragma unroll
+        for (int s = 0; s < KS; ++s) {
+            const unsigned wq = *reinterpret_cast<const unsigned *>(w + (int64_t)(r * KS + s) * d.C + c0);
+            const int m[4] = {(int)(wq & 0xffu), (int)(wq & 0xff00u), (int)(wq & 0xff0000u), (int)(wq & 0xff000000u)};
+#pragma unroll
+            for (int j = 0; j < QB; ++j)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) acc[j][e] = dp4a(win[j * SW + s], m[e], acc[j][e]);
+        }
+    }
+    const float4 sw = *reinterpret_cast<const float4 *>(ws + c0), bs = *reinterpret_cast<const float4 *>(bias + c0);
+    const float sw4[4] = {sw.x, sw.y, sw.z, sw.w}, bs4[4] = {bs.x, bs.y, bs.z, bs.w};
+#pragma unroll
+    for (int j = 0; j < QB; ++j) {
+        if (q0 + j >= d.Q) break;
+        Vec<TO, 4> o;
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+            o.v[e] = q8_out<TO>(q8_value(acc[j][e], q.s_x, sw4[e], bs4[e], 0.0f, d.act), q.inv_out);
+        *reinterpret_cast<Vec<TO, 4> *>(y + ((int64_t)rowi * d.Q + q0 + j) * d.C + c0) = o;
+    }
+}
+
+// the depthwise kernel above where it applies: 3x3 and 5x5, square stride 1 or
+// 2, dilation 1, whole words of channels, 32-bit work indices
+template <typename TO>
+static bool q8_dw_vec(const LaunchArgs &a, const ConvDims &d, const float *ws, Q8Scales q) {
+    if (a.schema.layout != SN_NHWC || d.groups != d.C || d.K != d.C || d.C % 4 || d.dh != 1 || d.dw != 1 ||
+        d.R != d.S || (d.R != 3 && d.R != 5) || d.sh != d.sw || (d.sh != 1 && d.sh != 2) || a.in[1] ||
+        (uintptr_t)a.in[0] % 4 || (uintptr_t)a.wt % 16 || (uintptr_t)a.out % (4 * sizeof(TO)))
+        return false;
+    constexpr int QB = 4;
+    const int64_t items = (int64_t)((d.Q + QB - 1) / QB) * (d.C / 4), total = (int64_t)d.N * d.P * items;
+    if (total >= ((int64_t)1 << 31)) return false;
+    const dim3 grid((unsigned)((total + 255) / 256));
+    const FastDiv fi = make_fastdiv((uint32_t)items), fc = make_fastdiv((uint32_t)(d.C / 4)),
+                  fp = make_fastdiv((uint32_t)d.P);
+#define SN_Q8_DW(KS, SW)                                                                                           \
+    launch_pdl(q8_dw_nhwc_kernel<KS, SW, QB, TO>, grid, 256, 0, a.stream, (const int8_t *)a.in[0],                 \
+               (const int8_t *)a.wt, ws, a.bias, (TO *)a.out, d, q, fi, fc, fp, (uint32_t)total)
+    if (d.R == 3) {
+        if (d.sh == 1) SN_Q8_DW(3, 1);
+        else SN_Q8_DW(3, 2);
+    } else {
+        if (d.sh == 1) SN_Q8_DW(5, 1);
+        else SN_Q8_DW(5, 2);
+    }
+#undef SN_Q8_DW
+    return true;
+}
+
 cudaError_t q8_conv_direct(const LaunchArgs &a) {
     if (!scales_ok(a, a.in[1] ? 2 : 1)) return cudaErrorInvalidValue;
     const ConvDims d = conv_dims(a);
@@ -460,7 +549,8 @@ cudaError_t q8_conv_direct(const LaunchArgs &a) {
     const int64_t elems = (int64_t)d.K * (d.C / d.groups) * d.R * d.S;
     const float *ws = wscales(a.wt, elems);
     SN_Q8_OUT_SWITCH(out_dtype(a), TO, {
-        if (a.schema.layout == SN_NHWC)
+        if (q8_dw_vec<TO>(a, d, ws, scales_of(a))) {
+        } else if (a.schema.layout == SN_NHWC)
             launch_pdl(q8_conv_direct_kernel<true, TO>, grid_for(total, 256), 256, 0, a.stream,
                        (const int8_t *)a.in[0], (const int8_t *)a.wt, ws, a.bias, (const int8_t *)a.in[1], (TO *)a.out,
                        d, scales_of(a));
@@ -610,7 +700,7 @@ __global__ void __launch_bounds__(256) q8_dense_kernel(const int8_t *__restrict_
     const int o = blockIdx.x * 8 + (threadIdx.x >> 5);
     if (o >= O) return;
     const int8_t *wr = w + (int64_t)o * I;
-    for (int n0 = 0; n0 < N; n0 += NB) {
+    for (int n0 = blockIdx.y * NB; n0 < N; n0 += gridDim.y * NB) {
         int acc[NB] = {};
         if (V16) {
             int i = lane * 16;
@@ -652,7 +742,12 @@ cudaError_t q8_dense(const LaunchArgs &a) {
     const Layer &l = *a.layer;
     const int N = (int)a.in_shapes[0].n, I = l.dense_in, O = l.dense_out;
     const float *ws = wscales(a.wt, (int64_t)I * O);
-    const dim3 grid((unsigned)((O + 7) / 8));
+    // images per warp: their weight row is read once, but a warp per (feature,
+    // image) fills the GPU better while that is under two warps a scheduler
+    // (152 SMs x 8); 8 images of 672 -> 168 took 11.2 us between timing nodes of
+    // a replayed net on 21 blocks, 7.1 us on 168
+    const int nb = (int64_t)N * O < 2 * 1216 ? 1 : N <= 1 ? 1 : N <= 2 ? 2 : N <= 4 ? 4 : 8;
+    const dim3 grid((unsigned)((O + 7) / 8), (unsigned)std::min((N + nb - 1) / nb, 65535));
     const bool v16 = I % 16 == 0 && (uintptr_t)a.in[0] % 16 == 0 && (uintptr_t)a.wt % 16 == 0;
 #define SN_Q8_DENSE(NB)                                                                                        \
     SN_Q8_OUT_SWITCH(out_dtype(a), TO,                                                                         \
@@ -662,11 +757,11 @@ cudaError_t q8_dense(const LaunchArgs &a) {
                           : launch_pdl(q8_dense_kernel<NB, false, TO>, grid, 256, 0, a.stream,                 \
                                        (const int8_t *)a.in[0], (const int8_t *)a.wt, ws, a.bias, (TO *)a.out, \
                                        N, I, O, l.act, scales_of(a))))
-    if (N <= 1) {
+    if (nb == 1) {
         SN_Q8_DENSE(1);
-    } else if (N <= 2) {
+    } else if (nb == 2) {
         SN_Q8_DENSE(2);
-    } else if (N <= 4) {
+    } else if (nb == 4) {
         SN_Q8_DENSE(4);
     } else {
         SN_Q8_DENSE(8);
@@ -714,13 +809,57 @@ __global__ void q8_maxpool_kernel(const int8_t *__restrict__ x, TO *__restrict__
     }
 }
 
+// NHWC, words of four codes (C % 4 == 0): the per-byte signed maximum
+template <typename TO>
+__global__ void __launch_bounds__(256) q8_maxpool_nhwc_kernel(const int8_t *__restrict__ x, TO *__restrict__ y, int C,
+                                                              int H, int W, sn_pool_params pp, float s_x, float inv,
+                                                              FastDiv fd_c4, FastDiv fd_Q, FastDiv fd_P,
+                                                              uint32_t total) {
+    griddep_launch();
+    griddep_wait();
+    const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= total) return;
+    const uint32_t pix = fdiv(t, fd_c4);
+    const int c0 = (int)(t - pix * fd_c4.d) * 4;
+    const uint32_t row = fdiv(pix, fd_Q);
+    const int q = (int)(pix - row * fd_Q.d);
+    const uint32_t n = fdiv(row, fd_P);
+    const int p = (int)(row - n * fd_P.d);
+    unsigned m = 0x80808080u;
+    bool any = false;
+    for (int r = 0; r < pp.kh; ++r) {
+        const int h = p * pp.sh - pp.ph + r;
+        if (h < 0 || h >= H) continue;
+        const int8_t *xr = x + (((int64_t)n * H + h) * W) * C + c0;
+        for (int s = 0; s < pp.kw; ++s) {
+            const int ww = q * pp.sw - pp.pw + s;
+            if (ww < 0 || ww >= W) continue;
+            m = __vmaxs4(m, *reinterpret_cast<const unsigned *>(xr + (int64_t)ww * C));
+            any = true;
+        }
+    }
+    Vec<TO, 4> o;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const int v = any ? (int)(int8_t)(m >> (8 * e)) : -(1 << 20);  // below every code, as in the general kernel
+        o.v[e] = q8_out<TO>(__fmul_rn((float)v, s_x), inv);
+    }
+    *reinterpret_cast<Vec<TO, 4> *>(y + (int64_t)pix * C + c0) = o;
+}
+
 cudaError_t q8_maxpool(const LaunchArgs &a) {
     if (!scales_ok(a, 1)) return cudaErrorInvalidValue;
     const Shape &i = a.in_shapes[0], &o = a.layer->out;
     const int64_t total = o.numel();
     const float inv = scales_of(a).inv_out;
     SN_Q8_OUT_SWITCH(out_dtype(a), TO, {
-        if (a.schema.layout == SN_NHWC)
+        if (a.schema.layout == SN_NHWC && i.c % 4 == 0 && (uintptr_t)a.in[0] % 4 == 0 &&
+            (uintptr_t)a.out % (4 * sizeof(TO)) == 0 && total / 4 < ((int64_t)1 << 31))
+            launch_pdl(q8_maxpool_nhwc_kernel<TO>, dim3((unsigned)((total / 4 + 255) / 256)), 256, 0, a.stream,
+                       (const int8_t *)a.in[0], (TO *)a.out, (int)i.c, (int)i.h, (int)i.w, a.layer->pool, a.qs_in[0],
+                       inv, make_fastdiv((uint32_t)(i.c / 4)), make_fastdiv((uint32_t)o.w),
+                       make_fastdiv((uint32_t)o.h), (uint32_t)(total / 4));
+        else if (a.schema.layout == SN_NHWC)
             launch_pdl(q8_maxpool_kernel<true, TO>, grid_for(total, 256), 256, 0, a.stream, (const int8_t *)a.in[0],
                        (TO *)a.out, (int)i.n, (int)i.c, (int)i.h, (int)i.w, (int)o.h, (int)o.w, a.layer->pool,
                        a.qs_in[0], inv);
@@ -762,14 +901,60 @@ __global__ void q8_gap_kernel(const int8_t *__restrict__ x, TO *__restrict__ y, 
     }
 }
 
+// NHWC, words of four codes (C % 4 == 0): a block owns eight words (32 bytes of
+// every pixel) of one image, its other thread axis cuts the pixels into
+// blockDim / 8 slices; the exact sums are added by shuffles and through shared
+// memory (one thread per channel, as above, walked all H*W pixels alone)
+template <typename TO>
+__global__ void __launch_bounds__(1024) q8_gap_nhwc_kernel(const int8_t *__restrict__ x, TO *__restrict__ y, int C,
+                                                           int HW, float s_x, float inv) {
+    griddep_launch();
+    griddep_wait();
+    __shared__ int part[32][33];
+    const int v = threadIdx.x & 7, sl = threadIdx.x >> 3, slices = blockDim.x >> 3;
+    const int c0 = (blockIdx.x * 8 + v) * 4;
+    int s[4] = {};
+    if (c0 < C) {
+        const int8_t *xn = x + (int64_t)blockIdx.y * HW * C + c0;
+#pragma unroll 4
+        for (int p = sl; p < HW; p += slices) {
+            const int q = *reinterpret_cast<const int *>(xn + (int64_t)p * C);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) s[e] = dp4a(q, 1 << (8 * e), s[e]);
+        }
+    }
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        s[e] += __shfl_xor_sync(0xffffffffu, s[e], 8);
+        s[e] += __shfl_xor_sync(0xffffffffu, s[e], 16);
+    }
+    const int warp = threadIdx.x >> 5;
+    if ((threadIdx.x & 31) < 8) {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) part[warp][v * 4 + e] = s[e];
+    }
+    __syncthreads();
+    const int c = blockIdx.x * 32 + threadIdx.x;
+    if (threadIdx.x < 32 && c < C) {
+        int sum = 0;
+        for (int k = 0; k < (int)(blockDim.x >> 5); ++k) sum += part[k][threadIdx.x];
+        y[(int64_t)blockIdx.y * C + c] = q8_out<TO>(__fdiv_rn(__fmul_rn(__int2float_rn(sum), s_x), (float)HW), inv);
+    }
+}
+
 cudaError_t q8_gap(const LaunchArgs &a) {
     if (!scales_ok(a, 1)) return cudaErrorInvalidValue;
     const Shape &i = a.in_shapes[0];
     const float inv = scales_of(a).inv_out;
     const int64_t nc = i.n * i.c;
     if (i.h * i.w >= (1 << 23)) return cudaErrorInvalidValue;  // int32 sums stay exact
+    int threads = 64;  // about four pixels a thread where the map has them
+    while (threads < 1024 && (int64_t)threads / 8 * 4 < i.h * i.w) threads *= 2;
     SN_Q8_OUT_SWITCH(out_dtype(a), TO, {
-        if (a.schema.layout == SN_NHWC)
+        if (a.schema.layout == SN_NHWC && i.c % 4 == 0 && (uintptr_t)a.in[0] % 4 == 0 && i.n <= 65535)
+            launch_pdl(q8_gap_nhwc_kernel<TO>, dim3((unsigned)((i.c + 31) / 32), (unsigned)i.n), threads, 0, a.stream,
+                       (const int8_t *)a.in[0], (TO *)a.out, (int)i.c, (int)(i.h * i.w), a.qs_in[0], inv);
+        else if (a.schema.layout == SN_NHWC)
             launch_pdl(q8_gap_kernel<true, TO>, grid_for(nc, 256), 256, 0, a.stream, (const int8_t *)a.in[0],
                        (TO *)a.out, (int)i.n, (int)i.c, (int)(i.h * i.w), a.qs_in[0], inv);
         else
@@ -801,6 +986,46 @@ __global__ void q8_binary_kernel(const int8_t *__restrict__ a, const int8_t *__r
     }
 }
 
+// V codes per thread: add in any layout (N = 1, per_image = all vectors), or the
+// NHWC scale (C % V == 0; an image's channel vector is one division by a launch
+// constant away).  One code and three 64-bit divisions per thread before.
+template <bool MUL, int V, typename TO>
+__global__ void __launch_bounds__(256) q8_binary_vec_kernel(const Vec<int8_t, V> *__restrict__ a,
+                                                            const Vec<int8_t, V> *__restrict__ b,
+                                                            Vec<TO, V> *__restrict__ y, int N, uint32_t per_image,
+                                                            FastDiv fd_cv, float s_a, float s_b, int act, float inv) {
+    griddep_launch();
+    griddep_wait();
+    for (int n = blockIdx.y; n < N; n += gridDim.y) {
+        const size_t base = (size_t)n * per_image;
+        for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < per_image; i += gridDim.x * blockDim.x) {
+            const Vec<int8_t, V> va = a[base + i];
+            const Vec<int8_t, V> vb = MUL ? b[(size_t)n * fd_cv.d + (i - fdiv(i, fd_cv) * fd_cv.d)] : b[base + i];
+            Vec<TO, V> o;
+#pragma unroll
+            for (int e = 0; e < V; ++e) {
+                const float fa = __fmul_rn((float)va.v[e], s_a), fb = __fmul_rn((float)vb.v[e], s_b);
+                o.v[e] = q8_out<TO>(q8_act(MUL ? __fmul_rn(fa, fb) : __fadd_rn(fa, fb), act), inv);
+            }
+            y[base + i] = o;
+        }
+    }
+}
+
+template <bool MUL, int V, typename TO>
+static bool q8_binary_vec(const LaunchArgs &a, const Shape &o, int act, float inv) {
+    const int64_t per = MUL ? o.c * o.h * o.w : o.numel();
+    if ((MUL && a.schema.layout != SN_NHWC) || (MUL ? o.c : per) % V || per / V >= ((int64_t)1 << 30) ||
+        o.n >= ((int64_t)1 << 31) || (uintptr_t)a.in[0] % V || (uintptr_t)a.in[1] % V ||
+        (uintptr_t)a.out % (V * sizeof(TO)))
+        return false;
+    const dim3 grid(grid_for(per / V, 256, 152LL * 8), MUL ? (unsigned)std::min<int64_t>(o.n, 65535) : 1u);
+    launch_pdl(q8_binary_vec_kernel<MUL, V, TO>, grid, 256, 0, a.stream, (const Vec<int8_t, V> *)a.in[0],
+               (const Vec<int8_t, V> *)a.in[1], (Vec<TO, V> *)a.out, MUL ? (int)o.n : 1, (uint32_t)(per / V),
+               make_fastdiv((uint32_t)(MUL ? o.c / V : 1)), a.qs_in[0], a.qs_in[1], act, inv);
+    return true;
+}
+
 template <bool MUL>
 static cudaError_t q8_binary(const LaunchArgs &a) {
     if (!scales_ok(a, 2)) return cudaErrorInvalidValue;
@@ -809,7 +1034,8 @@ static cudaError_t q8_binary(const LaunchArgs &a) {
     const float inv = scales_of(a).inv_out;
     const int act = a.layer->act;
     SN_Q8_OUT_SWITCH(out_dtype(a), TO, {
-        if (a.schema.layout == SN_NHWC)
+        if (q8_binary_vec<MUL, 16, TO>(a, o, act, inv) || q8_binary_vec<MUL, 4, TO>(a, o, act, inv)) {
+        } else if (a.schema.layout == SN_NHWC)
             launch_pdl(q8_binary_kernel<MUL, true, TO>, grid_for(total, 256), 256, 0, a.stream,
                        (const int8_t *)a.in[0], (const int8_t *)a.in[1], (TO *)a.out, total, (int)o.c, o.h * o.w,
                        a.qs_in[0], a.qs_in[1], act, inv);
