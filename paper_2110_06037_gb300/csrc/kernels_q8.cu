@@ -16,44 +16,12 @@
 #include <cmath>
 #include <type_traits>
 
-#include "kern_common.cuh"
+#include "q8_common.cuh"
 
 namespace sn {
 namespace k {
 
 namespace {
-
-constexpr int QMAX = 127;
-
-__device__ __forceinline__ int8_t q8_code(float y, float inv) {
-    const int q = __float2int_rn(__fmul_rn(y, inv));
-    return (int8_t)max(-QMAX, min(QMAX, q));
-}
-
-// the fused activations with one rounding per operation
-__device__ __forceinline__ float q8_act(float v, int act) {
-    if (act == SN_ACT_RELU) return fmaxf(v, 0.0f);
-    if (act == SN_ACT_NONE) return v;
-    if (act == SN_ACT_RELU6) return fminf(fmaxf(v, 0.0f), 6.0f);
-    const float t = __fdiv_rn(fminf(fmaxf(__fadd_rn(v, 3.0f), 0.0f), 6.0f), 6.0f);  // hard sigmoid
-    return act == SN_ACT_HSWISH ? __fmul_rn(v, t) : t;
-}
-
-// act(float(acc) * (s_x * s_w) + bias [+ residual value]) in fp32
-__device__ __forceinline__ float q8_value(int acc, float s_x, float s_w, float bias, float resid, int act) {
-    float y = __fadd_rn(__fmul_rn(__int2float_rn(acc), __fmul_rn(s_x, s_w)), bias);
-    y = __fadd_rn(y, resid);
-    return q8_act(y, act);
-}
-
-// the output element: a code of the output blob's scale, or, when the routine
-// writes a float schema (dequantisation fused into the epilogue), the fp32
-// value rounded to that type
-template <typename TO>
-__device__ __forceinline__ TO q8_out(float y, float inv) {
-    if constexpr (std::is_same<TO, int8_t>::value) return q8_code(y, inv);
-    else return cvt<TO>(y);
-}
 
 __device__ __forceinline__ int dp4a(int a, int b, int c) { return __dp4a(a, b, c); }
 
@@ -95,8 +63,6 @@ __global__ void q8_cast_kernel(const Ti *__restrict__ x, To *__restrict__ y, int
 
 // four consecutive elements per thread (n % 4 == 0; bases aligned to 4
 // elements of each side)
-template <typename T, int N> struct alignas(sizeof(T) * N) Vec { T v[N]; };
-
 template <typename Ti, typename To>
 __global__ void q8_cast4_kernel(const Vec<Ti, 4> *__restrict__ x, Vec<To, 4> *__restrict__ y, int64_t n4, float s,
                                 float inv) {
@@ -357,10 +323,13 @@ __global__ void q8_wcode_kernel(const float *__restrict__ w, const float *__rest
             c = (i / (S * R)) % Cg;
             kk = i / (S * R * Cg);
         }
-        const float v = w[((kk * Cg + c) * R + r) * S + s];
-        const int q = __float2int_rn(__fdiv_rn(v, scale[kk]));
-        out[i] = (int8_t)max(-QMAX, min(QMAX, q));
+        out[i] = (int8_t)q8_weight_code(w[((kk * Cg + c) * R + r) * S + s], scale[kk]);
     }
+}
+
+cudaError_t q8_weight_scales(const float *w, float *scale, int64_t K, int64_t per_k, cudaStream_t st) {
+    launch_pdl(q8_wscale_kernel, dim3((unsigned)K), 256, 0, st, w, scale, per_k);
+    return cudaGetLastError();
 }
 
 cudaError_t weight_format_q8(const float *w, void *out, int fmt, int64_t K, int64_t Cg, int64_t R, int64_t S,
@@ -368,7 +337,8 @@ cudaError_t weight_format_q8(const float *w, void *out, int fmt, int64_t K, int6
     if (fmt != W_KCRS && fmt != W_RSCK && fmt != W_KRSC) return cudaErrorInvalidValue;
     const int64_t elems = K * Cg * R * S;
     float *scale = reinterpret_cast<float *>(static_cast<char *>(out) + align16(elems));
-    launch_pdl(q8_wscale_kernel, dim3((unsigned)K), 256, 0, st, w, scale, Cg * R * S);
+    const cudaError_t e = q8_weight_scales(w, scale, K, Cg * R * S, st);
+    if (e != cudaSuccess) return e;
     launch_pdl(q8_wcode_kernel, grid_for(elems, 256), 256, 0, st, w, (const float *)scale, (int8_t *)out, fmt, K, Cg,
                R, S);
     return cudaGetLastError();

@@ -20,6 +20,7 @@ const char *routine_name(int32_t r) {
     case R_CONV_WINO6: return "conv2/wino_f6x6_3x3";
     case R_CONV_TC: return "conv2/igemm_tc";
     case R_CONV_TC_ODD: return "conv2/igemm_tc_odd";
+    case R_CONV_TC_F32: return "conv2/igemm_tc_f32";
     case R_DW_DIRECT: return "dwconv2/direct";
     case R_MAXPOOL: return "maxpool/direct";
     case R_GAP: return "gap/reduce";
@@ -60,6 +61,8 @@ std::string candidate_desc(const Graph &g, int32_t cand) {
     std::string params;
     if ((c.routine == R_CONV_TC || c.routine == R_CONV_TC_ODD) && !in.empty())
         params = k::conv_tc_config_desc(L, in[0], g.schemas[c.schema], c.variant, c.routine == R_CONV_TC_ODD);
+    else if (c.routine == R_CONV_TC_F32 || (c.routine == R_CONV_DP4A && c.variant > 0))
+        params = k::conv_split_desc(L, in[0], g.schemas[c.schema], c.variant - (c.routine == R_CONV_DP4A));
     else
         params = variant_name(c.routine, c.variant);
     if (!params.empty()) d += " [" + params + "]";
@@ -68,11 +71,12 @@ std::string candidate_desc(const Graph &g, int32_t cand) {
 
 static bool is_conv(const Layer &l) { return l.type == SN_L_CONV2; }
 
-// qint8 schema: the routines that have an int8 kernel (one variant each)
+// qint8 schema: the routines that have an int8 kernel (one variant each, but
+// the implicit GEMM: 0 = dp4a, then the tensor-core tiles)
 static int32_t q8_variants(int32_t r, const Layer &l, const std::vector<Shape> &in, sn_schema s) {
     switch (r) {
     case R_CONV_DIRECT: return is_conv(l) ? 1 : 0;
-    case R_CONV_DP4A: return k::q8_conv_dp4a_applies(l, in[0], s) ? 1 : 0;
+    case R_CONV_DP4A: return k::q8_conv_dp4a_applies(l, in[0], s) ? 1 + k::conv_split_variants(l, in[0], s) : 0;
     case R_DW_DIRECT: return l.type == SN_L_DWCONV2 ? 1 : 0;
     case R_MAXPOOL: return l.type == SN_L_MAXPOOL ? 1 : 0;
     case R_GAP: return l.type == SN_L_GAP ? 1 : 0;
@@ -88,8 +92,10 @@ int32_t routine_variants(int32_t r, const Layer &l, const std::vector<Shape> &in
     if (r == R_CONV_DP4A) return 0;
     const sn_conv_params &p = l.conv;
     // a conv2 with a residual input is served by the routines whose epilogue
-    // adds it: direct and the tensor-core implicit GEMM
-    if (is_conv(l) && in.size() == 2 && r != R_CONV_DIRECT && r != R_CONV_TC && r != R_CONV_TC_ODD) return 0;
+    // adds it: direct and the tensor-core implicit GEMMs
+    if (is_conv(l) && in.size() == 2 && r != R_CONV_DIRECT && r != R_CONV_TC && r != R_CONV_TC_ODD &&
+        r != R_CONV_TC_F32)
+        return 0;
     switch (r) {
     case R_CONV_DIRECT:
         return is_conv(l) ? 1 : 0;
@@ -106,6 +112,8 @@ int32_t routine_variants(int32_t r, const Layer &l, const std::vector<Shape> &in
         return is_conv(l) ? k::conv_tc_variants(l, in[0], s) : 0;
     case R_CONV_TC_ODD:
         return is_conv(l) ? k::conv_tc_variants(l, in[0], s, true) : 0;
+    case R_CONV_TC_F32:
+        return is_conv(l) && s.dtype == SN_F32 ? k::conv_split_variants(l, in[0], s) : 0;
     case R_DW_DIRECT:
         if (l.type != SN_L_DWCONV2) return 0;
         // NHWC 3x3 of small maps: a third parameter, the shared-memory band kernel
@@ -137,19 +145,20 @@ size_t routine_workspace(int32_t r, int32_t v, const Layer &l, const std::vector
     if (r == R_CONV_WINO4) return k::conv_wino4_ws(l, in[0], s);
     if (r == R_CONV_WINO6) return k::conv_wino6_ws(l, in[0], s);
     if (r == R_CONV_TC || r == R_CONV_TC_ODD) return k::conv_tc_ws(l, in[0], s, v, 0, r == R_CONV_TC_ODD);
+    if (r == R_CONV_TC_F32 || (r == R_CONV_DP4A && v > 0)) return k::conv_split_ws(l, in[0], s);
     if (r == R_CONV_IM2COL_TC) return k::conv_im2col_tc_ws(l, in[0], s, v);
     if (r == R_DENSE_TC) return k::dense_tc_ws(l, in[0], s, v);
     if (r == R_CONV_S2D_TC) return k::conv_s2d_tc_ws(l, in[0], s, v);
     return 0;
 }
 
-// weight format of (routine, layout)
-static int weight_format_of(int32_t r, sn_schema s) {
+// weight format of (routine, routine parameter, layout)
+static int weight_format_of(int32_t r, int32_t v, sn_schema s) {
     if (s.dtype == SN_QI8) {
         switch (r) {
         case R_CONV_DIRECT:
         case R_DW_DIRECT: return s.layout == SN_NCHW ? k::W_KCRS : k::W_RSCK;
-        case R_CONV_DP4A: return k::W_KRSC;
+        case R_CONV_DP4A: return v > 0 ? k::W_SPLIT : k::W_KRSC;
         case R_DENSE: return k::W_KCRS;
         default: return -1;
         }
@@ -162,6 +171,7 @@ static int weight_format_of(int32_t r, sn_schema s) {
     case R_CONV_WINO6: return k::W_WINO6;
     case R_CONV_TC:
     case R_CONV_TC_ODD: return k::W_KRSC;
+    case R_CONV_TC_F32: return k::W_SPLIT;
     case R_DW_DIRECT: return s.layout == SN_NCHW ? k::W_KCRS : k::W_RSCK;
     case R_DENSE: return k::W_KCRS;
     case R_CONV_IM2COL_TC: return k::W_KRSC_PAD64;
@@ -173,12 +183,11 @@ static int weight_format_of(int32_t r, sn_schema s) {
 
 sn_status prepare_weights(Graph *g, int32_t li, int32_t r, int32_t v, sn_schema s,
                           const void **wt, const float **bias, cudaStream_t st) {
-    (void)v;
     *wt = nullptr;
     *bias = nullptr;
     const Layer &L = g->layers[li];
     if (L.weight.empty()) return SN_OK;
-    const int fmt = weight_format_of(r, s);
+    const int fmt = weight_format_of(r, v, s);
     if (fmt < 0) return SN_OK;
     int64_t K, Cg, R, S;
     if (L.type == SN_L_DENSE) {
@@ -217,7 +226,8 @@ sn_status prepare_weights(Graph *g, int32_t li, int32_t r, int32_t v, sn_schema 
     Buffer src, dst;
     sn_status rc = dev_alloc(g, (size_t)K * Cg * R * S * sizeof(float), &src);
     if (rc != SN_OK) return rc;
-    const size_t dst_bytes = s.dtype == SN_QI8 ? k::q8_weight_bytes(K, elems)  // codes + per-channel scales
+    const size_t dst_bytes = fmt == k::W_SPLIT ? k::split_weight_bytes(K, Cg, R * S, s.dtype)
+                             : s.dtype == SN_QI8 ? k::q8_weight_bytes(K, elems)  // codes + per-channel scales
                              : (size_t)elems * ((fmt == k::W_WINO4 || fmt == k::W_WINO6) ? sizeof(float) : dtype_size(s.dtype));
     rc = dev_alloc(g, dst_bytes, &dst);
     if (rc != SN_OK) {
@@ -227,7 +237,8 @@ sn_status prepare_weights(Graph *g, int32_t li, int32_t r, int32_t v, sn_schema 
     cudaError_t e = cudaMemcpyAsync(src.ptr, L.weight.data(), L.weight.size() * sizeof(float),
                                     cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess)
-        e = s.dtype == SN_QI8
+        e = fmt == k::W_SPLIT ? k::weight_split(static_cast<const float *>(src.ptr), dst.ptr, s.dtype, K, Cg, R * S, st)
+            : s.dtype == SN_QI8
                 ? k::weight_format_q8(static_cast<const float *>(src.ptr), dst.ptr, fmt, K, Cg, R, S, st)
                 : k::weight_format(static_cast<const float *>(src.ptr), dst.ptr, fmt, s.dtype, K, Cg, R, S, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);  // src is freed next
@@ -242,6 +253,7 @@ sn_status prepare_weights(Graph *g, int32_t li, int32_t r, int32_t v, sn_schema 
 }
 
 int32_t kernels_per_launch(int32_t r, int32_t v, const Layer &l, const std::vector<Shape> &in, sn_schema s) {
+    if (r == R_CONV_TC_F32 || (r == R_CONV_DP4A && v > 0)) return 2;  // operand planes, GEMM
     if (s.dtype == SN_QI8) return 1;
     // a K-split tensor-core GEMM adds its reduction kernel (it is the only
     // variant with a workspace)
@@ -331,7 +343,7 @@ static cudaError_t launch_q8(const LaunchArgs &a) {
     switch (a.routine) {
     case R_CONV_DIRECT:
     case R_DW_DIRECT: return k::q8_conv_direct(a);
-    case R_CONV_DP4A: return k::q8_conv_dp4a(a);
+    case R_CONV_DP4A: return a.variant == 0 ? k::q8_conv_dp4a(a) : k::conv_split(a, a.variant - 1);
     case R_MAXPOOL: return k::q8_maxpool(a);
     case R_GAP: return k::q8_gap(a);
     case R_ADD: return k::q8_add(a);
@@ -357,6 +369,7 @@ sn_status launch_routine(const LaunchArgs &a) {
     case R_CONV_WINO6: e = k::conv_wino6(a); break;
     case R_CONV_TC:
     case R_CONV_TC_ODD: e = k::conv_tc(a); break;
+    case R_CONV_TC_F32: e = k::conv_split(a, a.variant); break;
     case R_DW_DIRECT: e = k::dwconv(a); break;
     case R_MAXPOOL: e = k::maxpool(a); break;
     case R_GAP: e = k::gap(a); break;

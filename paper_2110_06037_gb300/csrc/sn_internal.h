@@ -72,7 +72,8 @@ enum RoutineId : int32_t {
     R_CONV_DP4A = 16,    // qint8 implicit GEMM with dp4a (NHWC)
     R_CONV_WINO6 = 17,   // Winograd F(6x6,3x3) childnet (fp32 transformed filters)
     R_CONV_TC_ODD = 18,  // the tensor-core implicit GEMM with stride 2 on odd extents
-    R_COUNT = 19
+    R_CONV_TC_F32 = 19,  // fp32 on the tensor cores: operands as three bf16 planes (kernels_tc_split.cu)
+    R_COUNT = 20
 };
 
 // -------------------------------------------------------------------------
@@ -330,7 +331,8 @@ cudaError_t convert(const void *x, int dt_in, int lay_in, void *y, int dt_out, i
 cudaError_t fill_pattern(void *y, int dt, int64_t n, uint32_t seed, float scale,
                          cudaStream_t st);
 // weight re-layout / cast from fp32 KCRS (device) into a routine format
-enum WFormat { W_KCRS = 0, W_RSCK = 1, W_KRSC = 2, W_WINO = 3, W_KRSC_PAD64 = 4, W_S2D = 5, W_WINO4 = 6, W_WINO6 = 7 };
+enum WFormat { W_KCRS = 0, W_RSCK = 1, W_KRSC = 2, W_WINO = 3, W_KRSC_PAD64 = 4, W_S2D = 5, W_WINO4 = 6, W_WINO6 = 7,
+               W_SPLIT = 8 };
 cudaError_t weight_format(const float *w_kcrs, void *out, int fmt, int dt, int64_t K,
                           int64_t Cg, int64_t R, int64_t S, cudaStream_t st);
 
@@ -375,6 +377,13 @@ int32_t conv_s2d_tc_variants(const Layer &l, const Shape &in, sn_schema s);
 size_t conv_s2d_tc_ws(const Layer &l, const Shape &in, sn_schema s, int32_t v);
 cudaError_t conv_s2d_tc(const LaunchArgs &a);
 cudaError_t dense_tc(const LaunchArgs &a);
+// convolution on exact bf16 planes of the operands (fp32, qint8; NHWC)
+int32_t conv_split_variants(const Layer &l, const Shape &in, sn_schema s);
+std::string conv_split_desc(const Layer &l, const Shape &in, sn_schema s, int32_t v);
+size_t conv_split_ws(const Layer &l, const Shape &in, sn_schema s);
+size_t split_weight_bytes(int64_t K, int64_t C, int64_t RS, int dt);
+cudaError_t weight_split(const float *w_kcrs, void *out, int dt, int64_t K, int64_t C, int64_t RS, cudaStream_t st);
+cudaError_t conv_split(const LaunchArgs &a, int32_t v);
 cudaError_t dwconv(const LaunchArgs &a);
 bool dw3_band_applies(const Layer &l, const Shape &in, sn_schema s);  // NHWC small-map depthwise kernel
 cudaError_t maxpool(const LaunchArgs &a);

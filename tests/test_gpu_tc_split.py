@@ -1,0 +1,170 @@
+"""Tensor-core convolution on exact bf16 planes of the operands (fp32 and
+qint8): channel counts that are no multiple of a block, of eight or of four,
+ragged tiles, stride 2 on odd extents, several accumulator drains, residuals,
+infinities, and a wait that runs out."""
+import zlib
+
+import numpy as np
+import pytest
+
+import synth
+from oracle import q8
+from oracle.net import run_layer
+from paper_2110_06037_gb300 import SN_OPT_CHECK, SN_OPT_WAIT_LIMIT, SnError, _sn, build_graph, routine_name
+
+from gpu_helpers import from_device, to_device
+from test_gpu_q8 import F32, _out_scales, _ref_codes, codes_from_device, codes_to_device, conv_layer
+
+pytestmark = pytest.mark.gpu
+
+CASES = [
+    # N, C, H, W, K, k, s, pad, dil
+    (1, 3, 9, 9, 16, 3, 1, 1, 1),       # channels padded from 3 to 8
+    (2, 64, 8, 8, 64, 1, 1, 0, 1),      # plain, one K step
+    (1, 132, 5, 7, 68, 1, 1, 0, 1),     # plain, ragged rows, K past a tile
+    (2, 40, 9, 11, 66, 3, 1, 1, 1),     # K % 4 != 0: element stores
+    (1, 72, 13, 7, 24, 5, 2, 2, 1),     # stride 2 on odd extents
+    (3, 24, 12, 12, 8, 3, 1, 2, 2),     # dilation
+    (1, 328, 7, 7, 136, 3, 1, 1, 1),    # 54 K steps: fourteen drains in fp32, four in qint8
+    (5, 64, 28, 28, 200, 3, 1, 1, 1),   # more tiles than SMs: both accumulator buffers in turn
+]
+
+
+def tc_candidates(g, layer):
+    t = g.cost_table()
+    return [int(c) for c in np.flatnonzero(t["layer"] == layer) if " [tc " in g.candidate_desc(int(c))], t
+
+
+def force(g, t, layer, c):
+    path = [int(np.flatnonzero(t["layer"] == i)[0]) for i in range(t["n_layers"])]
+    path[layer] = c
+    g.set_path(path)
+
+
+@pytest.mark.parametrize("case", CASES)
+@pytest.mark.parametrize("residual", [False, True])
+def test_f32(case, residual):
+    """Error bound, per output, against fp64: a drain covers 256 products in 16
+    accumulation steps of 16 products; allowing a truncated unit (2^-23) for
+    each step and one for its alignment, 2^-18 of sum |x w| covers a drain, the
+    round-to-nearest sums of the drains (at most 54, 2^-24 each) and the dropped
+    plane products (2^-25); bias and residual add two roundings of the result."""
+    import torch
+    N, C, H, W, K, k, s, pd, dil = case
+    sch = ("f32", "nhwc")
+    rng = np.random.default_rng(zlib.crc32(repr(case).encode()))
+    x = rng.standard_normal((N, C, H, W)).astype(np.float32)
+    layer = synth.conv(C, K, k, s, pd, act="none", d=dil)
+    layer["weight"] = rng.standard_normal((K, C, k, k)).astype(np.float32)
+    layer["bias"] = rng.standard_normal(K).astype(np.float32)
+    other = dict(layer, weight=rng.standard_normal((K, C, k, k)).astype(np.float32))
+    mag = run_layer(dict(layer, weight=np.abs(layer["weight"]), bias=np.zeros(K, np.float32)), [np.abs(x).astype(np.float64)])
+    ref = run_layer(layer, [x.astype(np.float64)])
+    net, li = [dict(layer, inputs=[-1])], 1
+    if residual:  # another convolution of the same input joins the layer
+        net, li = [dict(other, inputs=[-1]), dict(layer, inputs=[-1, 0])], 2
+    g = build_graph(net, x.shape, sch, sch, [sch])
+    cands, t = tc_candidates(g, li)
+    assert cands
+    for c in cands:
+        force(g, t, li, c)
+        xd = to_device(x, sch)
+        if residual:  # the joined value is the library's own first layer
+            g1 = build_graph(net[:1], x.shape, sch, sch, [sch])
+            force(g1, g1.cost_table(), 1, int(np.flatnonzero(g1.cost_table()["layer"] == 1)[0]))
+            want = ref + from_device(g1.run(xd), sch).reshape(ref.shape)
+        else:
+            want = ref
+        y = g.run(xd)
+        torch.cuda.synchronize()
+        got = from_device(y, sch).reshape(want.shape)
+        bound = 2.0 ** -18 * mag + 2.0 ** -22 * np.abs(want) + 2.0 ** -22
+        assert (np.abs(got - want) <= bound).all(), (g.candidate_desc(c), float((np.abs(got - want) / bound).max()))
+        # far below the bound in the mean: the error of an fp32 sum, not of a 16-bit one
+        assert np.linalg.norm(got - want) <= 2e-6 * np.linalg.norm(want), g.candidate_desc(c)
+
+
+def test_f32_infinities_and_large_values():
+    """Operands that the planes cannot carry give what plain fp32 arithmetic gives."""
+    import torch
+    sch = ("f32", "nhwc")
+    rng = np.random.default_rng(3)
+    x = rng.standard_normal((1, 16, 6, 6)).astype(np.float32)
+    x[0, 3, 1, 1] = np.inf
+    x[0, 5, 4, 4] = -np.inf
+    x[0, 7, 4, 0] = np.nan
+    x[0, 2, 0, 4] = 3.4e38  # above the largest bf16
+    layer = synth.conv(16, 8, 3, 1, 1, act="none")
+    layer["weight"] = (rng.standard_normal((8, 16, 3, 3)) * 0.25).astype(np.float32)
+    layer["weight"][0, 3] = 0.5  # a plane of this weight is zero
+    layer["bias"] = np.zeros(8, np.float32)
+    g = build_graph([dict(layer, inputs=[-1])], x.shape, sch, sch, [sch])
+    cands, t = tc_candidates(g, 1)
+    direct = [int(c) for c in np.flatnonzero(t["layer"] == 1) if routine_name(int(t["routine"][c])) == "conv2/direct"]
+    outs = []
+    for c in direct + cands:
+        force(g, t, 1, c)
+        y = g.run(to_device(x, sch))
+        torch.cuda.synchronize()
+        outs.append(from_device(y, sch))
+    for o in outs[1:]:
+        assert np.array_equal(np.isnan(o), np.isnan(outs[0])) and np.array_equal(np.isinf(o), np.isinf(outs[0]))
+        fine = np.isfinite(outs[0])
+        assert np.array_equal(np.sign(o[~np.isnan(o)]), np.sign(outs[0][~np.isnan(outs[0])]))
+        assert np.allclose(o[fine], outs[0][fine], rtol=1e-5, atol=1e-5)
+
+
+@pytest.mark.parametrize("case", [c for c in CASES if c[1] % 4 == 0 and c[4] % 4 == 0])
+@pytest.mark.parametrize("extreme", [False, True])
+@pytest.mark.parametrize("out_dt", ["qi8", "f16", "f32"])
+def test_q8_bit_exact(case, extreme, out_dt):
+    import torch
+    N, C, H, W, K, k, s, pd, dil = case
+    rng = np.random.default_rng(zlib.crc32(repr(case).encode()))
+    # another qint8 layer of the same input joins, as a shortcut does
+    short = conv_layer(rng, C, K, k, s, pd, dil, act="none")
+    layer = dict(conv_layer(rng, C, K, k, s, pd, dil, act="relu"), inputs=[-1, 0])
+    q_in = rng.integers(-127, 128, (N, C, H, W)).astype(np.int8)
+    if extreme:  # every product 127 * 127: the sums come closest to 2^24
+        q_in[:] = 127
+        layer["weight"][:] = np.abs(layer["weight"]).max()
+    s_in = F32(0.02)
+    scales = _out_scales([short, layer], q_in, s_in)
+    lam = [("qi8", "nhwc")] + ([(out_dt, "nhwc")] if out_dt != "qi8" else [])
+    g = build_graph([short, layer], q_in.shape, ("qi8", "nhwc"), (out_dt, "nhwc"), lam)
+    for i, v in zip((-1, 0, 1), [s_in] + scales):
+        g.set_qscale(i, float(v))
+    cands, t = tc_candidates(g, 2)
+    cands = [c for c in cands if t["schema"][c] == 0 and t["out_schema"][c] == len(lam) - 1]
+    assert cands
+    first = [int(c) for c in np.flatnonzero(t["layer"] == 1) if t["schema"][c] == 0 and t["out_schema"][c] == 0][0]
+    q_s = q8.run_layer(short, [q_in], [s_in], scales[0])
+    want = q8.run_layer(layer, [q_in, q_s], [s_in, scales[0]], scales[1],
+                        **({} if out_dt == "qi8" else {"out_dtype": out_dt}))
+    for c in cands:
+        path = [int(np.flatnonzero(t["layer"] == 0)[0]), first, c, int(np.flatnonzero(t["layer"] == 3)[0])]
+        g.set_path(path)
+        y = g.run(codes_to_device(q_in, "nhwc"))
+        torch.cuda.synchronize()
+        got = codes_from_device(y, "nhwc") if out_dt == "qi8" else from_device(y, (out_dt, "nhwc"))
+        assert np.array_equal(got.reshape(want.shape), want.astype(got.dtype)), g.candidate_desc(c)
+
+
+def test_expired_wait_reports_timeout_and_recovers():
+    import torch
+    x, layers = synth.single_conv(2, 14, 64, 128, 3, 1)
+    sch = ("f32", "nhwc")
+    g = build_graph(layers, x.shape, sch, sch, [sch])
+    cands, t = tc_candidates(g, 1)
+    force(g, t, 1, cands[0])
+    g.set_option(SN_OPT_CHECK, 1)
+    xd = to_device(x, sch)
+    y0 = g.run(xd).clone()
+    g.set_option(SN_OPT_WAIT_LIMIT, 1)
+    with pytest.raises(SnError) as e:
+        g.run(xd)
+    assert e.value.status == _sn.SN_ETIMEOUT
+    g.set_option(SN_OPT_WAIT_LIMIT, 0)
+    y1 = g.run(xd)
+    torch.cuda.synchronize()
+    assert torch.equal(y0, y1)
