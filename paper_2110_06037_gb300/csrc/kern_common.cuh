@@ -34,13 +34,25 @@ template <> __device__ __forceinline__ __nv_bfloat16 cvt<__nv_bfloat16>(float v)
     return __float2bfloat16_rn(v);
 }
 
+// t / 6 correctly rounded, for t = 0 and the t in [2.4e-38, 6] (Markstein's
+// correction of a product with the reciprocal: the remainder t - 6q is exact,
+// and one step from it rounds like the division; compared with the division for
+// every float of that range).  The hard activations' t is 0 or at least 2^-22.
+// The division itself is a chain with a branch, once per element of an
+// epilogue.
+__device__ __forceinline__ float sixth(float t) {
+    constexpr float r = 1.0f / 6.0f;
+    const float q = __fmul_rn(t, r);
+    return __fmaf_rn(__fmaf_rn(-6.0f, q, t), r, q);
+}
+
 // The common activations first, as before the hard-swish pair was added: in
 // an unrolled epilogue every extra test of `act` is paid per element.
 __device__ __forceinline__ float act_apply(float v, int act) {
     if (act == SN_ACT_RELU) return fmaxf(v, 0.0f);
     if (act == SN_ACT_NONE) return v;
     if (act == SN_ACT_RELU6) return fminf(fmaxf(v, 0.0f), 6.0f);
-    const float t = fminf(fmaxf(v + 3.0f, 0.0f), 6.0f) / 6.0f;  // hard sigmoid
+    const float t = sixth(fminf(fmaxf(v + 3.0f, 0.0f), 6.0f));  // hard sigmoid
     return act == SN_ACT_HSWISH ? v * t : t;
 }
 

@@ -24,7 +24,7 @@ __device__ __forceinline__ float q8_act(float v, int act) {
     if (act == SN_ACT_RELU) return fmaxf(v, 0.0f);
     if (act == SN_ACT_NONE) return v;
     if (act == SN_ACT_RELU6) return fminf(fmaxf(v, 0.0f), 6.0f);
-    const float t = __fdiv_rn(fminf(fmaxf(__fadd_rn(v, 3.0f), 0.0f), 6.0f), 6.0f);  // hard sigmoid
+    const float t = sixth(fminf(fmaxf(__fadd_rn(v, 3.0f), 0.0f), 6.0f));  // hard sigmoid: v / 6 to the bit
     return act == SN_ACT_HSWISH ? __fmul_rn(v, t) : t;
 }
 

@@ -719,8 +719,8 @@ __global__ void __launch_bounds__(THREADS, 1)
                                     make_uint4(wq[0], wq[1], wq[2], wq[3]);
                             }
                         };
-                        if (p.act == SN_ACT_RELU)
-                            finish_rows([](float x) { return fmaxf(x, 0.0f); });
+                        if (p.act == SN_ACT_RELU || p.act == SN_ACT_RELU6)
+                            finish_rows([hi = p.act == SN_ACT_RELU ? INFINITY : 6.0f](float x) { return fminf(fmaxf(x, 0.0f), hi); });
                         else if (p.act == SN_ACT_NONE)
                             finish_rows([](float x) { return x; });
                         else
@@ -818,8 +818,8 @@ __global__ void __launch_bounds__(THREADS, 1)
                                 make_uint4(wq[0], wq[1], wq[2], wq[3]);
                         }
                     };
-                    if (p.act == SN_ACT_RELU)
-                        stage_rows([](float x) { return fmaxf(x, 0.0f); });
+                    if (p.act == SN_ACT_RELU || p.act == SN_ACT_RELU6)
+                        stage_rows([hi = p.act == SN_ACT_RELU ? INFINITY : 6.0f](float x) { return fminf(fmaxf(x, 0.0f), hi); });
                     else if (p.act == SN_ACT_NONE)
                         stage_rows([](float x) { return x; });
                     else
