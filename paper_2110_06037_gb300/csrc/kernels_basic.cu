@@ -528,21 +528,26 @@ __device__ __forceinline__ void fma16(float (&acc)[E], const uint4 &x, const uin
 }
 
 // One thread: QB consecutive output columns x E channels (16 bytes) of one
-// output row.  The grid's y axis walks the N x P output rows, its x axis the
-// (column block, channel vector) pairs of a row with the channel vector
-// fastest (coalesced 16-byte accesses); all index math is 32-bit, one
-// division per thread (64-bit division and modulo by runtime values cost
-// more than the arithmetic of the taps).
-template <typename T, int QB, int SW>  // SW = 1 or 2: 3x3 fast path for that stride; 0 = any
+// output row.  Threads walk the (row, column block, channel vector) items with
+// the channel vector fastest (coalesced 16-byte accesses) and no thread idle at
+// a row's end; the three indices are divisions by launch constants.
+// SW = 1 or 2, KS = 3 or 5: the window path for that stride and kernel, where a
+// tap row's input columns are loaded once for the QB outputs that read them
+// (5x5, 4 outputs: 8 loads a row instead of 20 conditional ones; 8 x 28 x 28 x
+// 120 bf16 between timing nodes of a replayed net, an empty op reading about 5
+// us: 10.7 us against 16.6); SW = 0: any.
+template <typename T, int QB, int SW, int KS>
 __global__ void __launch_bounds__(256, 2) dw_nhwc_vec(const T *__restrict__ x, const T *__restrict__ w,
                                                       const float *__restrict__ bias, T *__restrict__ y, ConvDims d,
-                                                      int CV, int QBLK) {
+                                                      FastDiv fd_items, FastDiv fd_cv, FastDiv fd_P, uint32_t total) {
     griddep_launch();
     griddep_wait();
     constexpr int E = 16 / sizeof(T);
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= QBLK * CV) return;
-    const int qb = t / CV, cv = t - qb * CV;
+    const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= total) return;
+    const int rowi = (int)fdiv(t, fd_items);
+    const int item = (int)(t - (uint32_t)rowi * fd_items.d);
+    const int qb = (int)fdiv((uint32_t)item, fd_cv), cv = item - qb * (int)fd_cv.d;
     const int c0 = cv * E, q0 = qb * QB;
     float b[E];
     {
@@ -552,9 +557,9 @@ __global__ void __launch_bounds__(256, 2) dw_nhwc_vec(const T *__restrict__ x, c
 #pragma unroll
         for (int e = 0; e < E; ++e) b[e] = bb[e];
     }
-    for (int rowi = blockIdx.y; rowi < d.N * d.P; rowi += gridDim.y) {
-        const int n = rowi / d.P, p = rowi - n * d.P;
-        if constexpr (std::is_same<T, __half>::value && SW > 0) {
+    {
+        const int n = (int)fdiv((uint32_t)rowi, fd_P), p = rowi - n * d.P;
+        if constexpr (std::is_same<T, __half>::value && SW > 0 && KS == 3) {
             // fp16 3x3: packed half2 multiply-adds accumulating in fp16, in the
             // same order as the ring kernel (bias, rows, columns)
             __half2 hacc[QB][4];
@@ -610,7 +615,7 @@ __global__ void __launch_bounds__(256, 2) dw_nhwc_vec(const T *__restrict__ x, c
                 }
                 *reinterpret_cast<uint4 *>(yrow + (int64_t)(q0 + j) * d.C) = o;
             }
-            continue;
+            return;
         }
         float acc[QB][E];
 #pragma unroll
@@ -618,12 +623,12 @@ __global__ void __launch_bounds__(256, 2) dw_nhwc_vec(const T *__restrict__ x, c
 #pragma unroll
             for (int e = 0; e < E; ++e) acc[j][e] = b[e];
         if (SW > 0) {
-            // 3x3 fast path: the input window of each tap row (QB outputs need
-            // (QB-1)*SW + 3 columns) is loaded once and reused by the three taps
-            constexpr int WN = (QB - 1) * (SW > 0 ? SW : 1) + 3;
+            // the input window of each tap row (QB outputs need (QB-1)*SW + KS
+            // columns) is loaded once and reused by the KS taps
+            constexpr int WN = (QB - 1) * (SW > 0 ? SW : 1) + KS;
             const int wbase = q0 * SW - d.pw;
 #pragma unroll
-            for (int r = 0; r < 3; ++r) {
+            for (int r = 0; r < KS; ++r) {
                 const int h = p * d.sh - d.ph + r * d.dh;
                 if (h < 0 || h >= d.H) continue;
                 const T *xrow = x + (((int64_t)n * d.H + h) * d.W) * d.C + c0;
@@ -635,8 +640,8 @@ __global__ void __launch_bounds__(256, 2) dw_nhwc_vec(const T *__restrict__ x, c
                                                     : make_uint4(0u, 0u, 0u, 0u);
                 }
 #pragma unroll
-                for (int s = 0; s < 3; ++s) {
-                    const uint4 wq = *reinterpret_cast<const uint4 *>(w + (int64_t)(r * 3 + s) * d.C + c0);
+                for (int s = 0; s < KS; ++s) {
+                    const uint4 wq = *reinterpret_cast<const uint4 *>(w + (int64_t)(r * KS + s) * d.C + c0);
 #pragma unroll
                     for (int j = 0; j < QB; ++j) fma16<T>(acc[j], win[j * (SW > 0 ? SW : 1) + s], wq);
                 }
@@ -1067,10 +1072,25 @@ cudaError_t dwconv(const LaunchArgs &a) {
                 else launch_pdl(dw3_nhwc_halo<T, 2, 3>, gb, 256, sm2, a.stream, x, w, a.bias, y, d);
             } else {
                 const int QBLK = (d.Q + 3) / 4, CV = (int)cvec;
-                const dim3 gb((unsigned)((QBLK * CV + 255) / 256), (unsigned)std::min<int64_t>((int64_t)d.N * d.P, 65535));
-                if (k3 && d.sw == 1) launch_pdl(dw_nhwc_vec<T, 4, 1>, gb, 256, 0, a.stream, x, w, a.bias, y, d, CV, QBLK);
-                else if (k3 && d.sw == 2) launch_pdl(dw_nhwc_vec<T, 4, 2>, gb, 256, 0, a.stream, x, w, a.bias, y, d, CV, QBLK);
-                else launch_pdl(dw_nhwc_vec<T, 4, 0>, gb, 256, 0, a.stream, x, w, a.bias, y, d, CV, QBLK);
+                const int64_t items = (int64_t)QBLK * CV, threads = (int64_t)d.N * d.P * items;
+                if (threads >= ((int64_t)1 << 31)) {
+                    launch_pdl(dw_nhwc<T>, grid_for(total, 256), 256, 0, a.stream, x, w, a.bias, y, d);
+                } else {
+                    // blocks of 128 until there are four of 256 for every SM
+                    const unsigned bs = threads < 152LL * 4 * 256 ? 128u : 256u;
+                    const unsigned gb = (unsigned)((threads + bs - 1) / bs);
+                    const FastDiv fi = make_fastdiv((uint32_t)items), fc = make_fastdiv((uint32_t)CV),
+                                  fp = make_fastdiv((uint32_t)d.P);
+                    const bool k5 = d.R == 5 && d.S == 5 && d.dw == 1;
+                    auto go = [&](auto kern) {
+                        launch_pdl(kern, gb, bs, 0, a.stream, x, w, a.bias, y, d, fi, fc, fp, (uint32_t)threads);
+                    };
+                    if (k3 && d.sw == 1) go(dw_nhwc_vec<T, 4, 1, 3>);
+                    else if (k3 && d.sw == 2) go(dw_nhwc_vec<T, 4, 2, 3>);
+                    else if (k5 && d.sw == 1) go(dw_nhwc_vec<T, 4, 1, 5>);
+                    else if (k5 && d.sw == 2) go(dw_nhwc_vec<T, 4, 2, 5>);
+                    else go(dw_nhwc_vec<T, 4, 0, 0>);
+                }
             }
         } else if (a.schema.layout == SN_NHWC) {
             launch_pdl(dw_nhwc<T>, grid_for(total, 256), 256, 0, a.stream, x, w, a.bias, y, d);
