@@ -1525,10 +1525,11 @@ static cudaError_t dense_t(const LaunchArgs &a) {
                    (const T *)a.wt, a.bias, (T *)a.out, N, IN, OUT, a.layer->act);
         return cudaGetLastError();
     }
-    // images per warp: their weight row is read once, but a warp per (feature,
-    // image) fills the GPU better while that is under two warps a scheduler
-    // (152 SMs x 8)
-    const int nb = N >= 8 && N * OUT >= 8 * 1216 ? 8 : N >= 2 && N * OUT >= 2 * 1216 ? 2 : 1;
+    // images per warp: large weights are read once for as many as there are;
+    // small ones stay in L2, and a warp per (feature, image) fills the GPU
+    // better until there are eight a scheduler (152 SMs x 4 x 16 / 8 blocks)
+    const bool big = IN * OUT >= ((int64_t)1 << 19);
+    const int nb = big ? (N >= 4 ? 8 : N >= 2 ? 2 : 1) : N * OUT >= 8 * 9728 ? 8 : N * OUT >= 2 * 9728 ? 2 : 1;
     const dim3 g((unsigned)((OUT + 7) / 8), (unsigned)((N + nb - 1) / nb));
     auto go = [&](auto kern) {
         launch_pdl(kern, g, 256, 0, a.stream, (const uint4 *)a.in[0], (const uint4 *)a.wt, a.bias, (T *)a.out, (int)N,

@@ -659,7 +659,7 @@ cudaError_t q8_conv_dp4a(const LaunchArgs &a) {
 // dense: one warp per output feature, NB images per pass over its weight row
 // (16-byte loads and dp4a when in_features % 16 == 0)
 // ===========================================================================
-template <int NB, bool V16, typename TO>
+template <int NB, int V, typename TO>  // V: codes per load (16, 4 or 1)
 __global__ void __launch_bounds__(256) q8_dense_kernel(const int8_t *__restrict__ x, const int8_t *__restrict__ w,
                                                        const float *__restrict__ ws, const float *__restrict__ bias,
                                                        TO *__restrict__ y, int N, int I, int O, int act,
@@ -672,7 +672,7 @@ __global__ void __launch_bounds__(256) q8_dense_kernel(const int8_t *__restrict_
     const int8_t *wr = w + (int64_t)o * I;
     for (int n0 = blockIdx.y * NB; n0 < N; n0 += gridDim.y * NB) {
         int acc[NB] = {};
-        if (V16) {
+        if (V == 16) {
             int i = lane * 16;
             for (; i < I; i += 512) {
                 const int4 wv = *reinterpret_cast<const int4 *>(wr + i);
@@ -685,6 +685,13 @@ __global__ void __launch_bounds__(256) q8_dense_kernel(const int8_t *__restrict_
                     acc[b] = dp4a(xv.z, wv.z, acc[b]);
                     acc[b] = dp4a(xv.w, wv.w, acc[b]);
                 }
+            }
+        } else if (V == 4) {
+            for (int i = lane * 4; i < I; i += 128) {
+                const int wv = *reinterpret_cast<const int *>(wr + i);
+#pragma unroll
+                for (int b = 0; b < NB; ++b)
+                    if (n0 + b < N) acc[b] = dp4a(*reinterpret_cast<const int *>(x + (int64_t)(n0 + b) * I + i), wv, acc[b]);
             }
         } else {
             for (int i = lane; i < I; i += 32) {
@@ -712,21 +719,25 @@ cudaError_t q8_dense(const LaunchArgs &a) {
     const Layer &l = *a.layer;
     const int N = (int)a.in_shapes[0].n, I = l.dense_in, O = l.dense_out;
     const float *ws = wscales(a.wt, (int64_t)I * O);
-    // images per warp: their weight row is read once, but a warp per (feature,
-    // image) fills the GPU better while that is under two warps a scheduler
-    // (152 SMs x 8); 8 images of 672 -> 168 took 11.2 us between timing nodes of
-    // a replayed net on 21 blocks, 7.1 us on 168
-    const int nb = (int64_t)N * O < 2 * 1216 ? 1 : N <= 1 ? 1 : N <= 2 ? 2 : N <= 4 ? 4 : 8;
+    // images per warp: large weights are read once for as many as there are;
+    // small ones stay in L2, and a warp per (feature, image) fills the GPU
+    // better until there are sixteen a scheduler (8 images of 672 -> 168 took
+    // 11.2 us between timing nodes of a replayed net on 21 blocks, 7.1 us on 168)
+    const int64_t no = (int64_t)N * O;
+    const int nb = (int64_t)I * O >= ((int64_t)1 << 20) ? (N >= 5 ? 8 : N >= 3 ? 4 : N)
+                   : no >= 8 * 9728 ? 8 : no >= 4 * 9728 ? 4 : no >= 2 * 9728 ? 2 : 1;
     const dim3 grid((unsigned)((O + 7) / 8), (unsigned)std::min((N + nb - 1) / nb, 65535));
     const bool v16 = I % 16 == 0 && (uintptr_t)a.in[0] % 16 == 0 && (uintptr_t)a.wt % 16 == 0;
-#define SN_Q8_DENSE(NB)                                                                                        \
-    SN_Q8_OUT_SWITCH(out_dtype(a), TO,                                                                         \
-                     (v16 ? launch_pdl(q8_dense_kernel<NB, true, TO>, grid, 256, 0, a.stream,                  \
-                                       (const int8_t *)a.in[0], (const int8_t *)a.wt, ws, a.bias, (TO *)a.out, \
-                                       N, I, O, l.act, scales_of(a))                                           \
-                          : launch_pdl(q8_dense_kernel<NB, false, TO>, grid, 256, 0, a.stream,                 \
-                                       (const int8_t *)a.in[0], (const int8_t *)a.wt, ws, a.bias, (TO *)a.out, \
-                                       N, I, O, l.act, scales_of(a))))
+    const bool v4 = I % 4 == 0 && (uintptr_t)a.in[0] % 4 == 0 && (uintptr_t)a.wt % 4 == 0;
+    auto go = [&](auto kern, auto *out) {
+        launch_pdl(kern, grid, 256, 0, a.stream, (const int8_t *)a.in[0], (const int8_t *)a.wt, ws, a.bias, out, N, I, O,
+                   (int)l.act, scales_of(a));
+    };
+#define SN_Q8_DENSE(NB)                                                                 \
+    SN_Q8_OUT_SWITCH(out_dtype(a), TO,                                                  \
+                     (v16  ? go(q8_dense_kernel<NB, 16, TO>, (TO *)a.out)               \
+                      : v4 ? go(q8_dense_kernel<NB, 4, TO>, (TO *)a.out)                \
+                           : go(q8_dense_kernel<NB, 1, TO>, (TO *)a.out)))
     if (nb == 1) {
         SN_Q8_DENSE(1);
     } else if (nb == 2) {

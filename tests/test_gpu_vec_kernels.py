@@ -41,7 +41,7 @@ def test_gap_then_scale(n, c, h, w, dt):
     assert maxrel(run_float(net, x, (dt, "nhwc")), run_layer(net[1], [xs, pooled], dt)) <= TOL[dt]
 
 
-@pytest.mark.parametrize("n,i,o", [(1, 8, 1), (1, 1032, 9), (9, 24, 120), (3, 520, 1001), (33, 264, 333), (2, 100, 7)])
+@pytest.mark.parametrize("n,i,o", [(1, 8, 1), (1, 1032, 9), (6, 1024, 520), (9, 24, 120), (3, 520, 1001), (33, 264, 333), (2, 100, 7)])
 @pytest.mark.parametrize("dt", ["f32", "f16", "bf16"])
 def test_dense(n, i, o, dt):
     rng = np.random.default_rng(zlib.crc32(repr((n, i, o, dt)).encode()))
@@ -81,3 +81,29 @@ def test_q8_pool_gap_add_mul_vectors(n, c, h, w):
         scales = _out_scales(layers, q_in, s_in)
         got, _ = run_q8(layers, q_in, s_in, scales, "nhwc", [])
         assert np.array_equal(got, _ref_codes(layers, q_in, s_in, scales)), layers[-1]["type"]
+
+
+@pytest.mark.parametrize("n,i,o", [(1, 4, 1), (8, 168, 672), (3, 1032, 1024), (9, 2048, 520), (40, 20, 2000)])
+def test_q8_dense_words(n, i, o):
+    rng = np.random.default_rng(n * 1000 + i)
+    layer = {"type": "dense", "inputs": [-1], "params": dict(in_features=i, out_features=o, act="hsigmoid"),
+             "weight": (rng.standard_normal((o, i)) / np.sqrt(i)).astype(F32),
+             "bias": rng.standard_normal(o).astype(F32)}
+    q_in = rng.integers(-127, 128, (n, i, 1, 1)).astype(np.int8)
+    s_in = F32(0.01)
+    scales = _out_scales([layer], q_in, s_in)
+    got, _ = run_q8([layer], q_in, s_in, scales, "nhwc", ["dense/simt"])
+    assert np.array_equal(got, _ref_codes([layer], q_in, s_in, scales))
+
+
+@pytest.mark.parametrize("ks,st,dil", [(5, 1, 1), (5, 2, 1), (3, 1, 1), (3, 2, 1), (7, 1, 1)])
+@pytest.mark.parametrize("c,h,w", [(8, 1, 1), (24, 7, 5), (40, 9, 18)])
+@pytest.mark.parametrize("dt", ["f32", "f16", "bf16"])
+def test_depthwise_windows(ks, st, dil, c, h, w, dt):
+    rng = np.random.default_rng(zlib.crc32(repr((ks, st, c, h, w, dt)).encode()))
+    x = rng.standard_normal((3, c, h, w)).astype(np.float32)
+    layer = dict(synth.dwconv(c, ks, st, act="hswish"), inputs=[-1])
+    layer["weight"] = (rng.standard_normal((c, 1, ks, ks)) / ks).astype(np.float32)
+    layer["bias"] = rng.standard_normal(c).astype(np.float32)
+    ref = run_layer(layer, [stored_values(x, dt)], dt)
+    assert maxrel(run_float([layer], x, (dt, "nhwc")), ref) <= TOL[dt]
