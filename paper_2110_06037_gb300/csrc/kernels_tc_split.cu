@@ -3,9 +3,14 @@
 //
 //   fp32   x = x0 + x1 + x2 with x0 = bf16(x), x1 = bf16(x - x0), x2 = x - x0 -
 //          x1: 8 + 8 + 8 significant bits, so the sum is exact.  Of the nine
-//          plane products the six with i + j <= 2 are formed (x0 w0 into one
-//          accumulator, the five small ones into a second); the dropped ones
-//          are below 2^-26 of |x w|.
+//          plane products the six with i + j <= 2 are formed, each i + j in an
+//          accumulator of its own; the dropped ones are below 2^-26 of |x w|.
+//          With 64-channel tiles the planes of B lie behind one another as rows
+//          of one operand: x0 [w0 w1 w2], x1 [w0 w1] and x2 [w0] are three MMAs
+//          of N = 192, 128 and 64 whose columns land on the accumulator of
+//          their i + j (an MMA of N = 64 alone takes as long to issue as one of
+//          N = 128).  128-channel tiles take six MMAs and two accumulators
+//          (x0 w0, the small products).
 //   qint8  a code in [-127, 127] is a bf16 value, and a sum of at most 1024
 //          code products stays below 2^24, so the fp32 accumulator holds the
 //          integer sum exactly.
@@ -97,8 +102,10 @@ struct Lay {
     static constexpr int STAGES = (227 * 1024 - 2048 - EPI_WARPS * (int)STAGE_OUT) / (int)STAGE < 6
                                       ? (227 * 1024 - 2048 - EPI_WARPS * (int)STAGE_OUT) / (int)STAGE
                                       : 6;
-    static constexpr int ACC = PLANES == 3 ? 2 : 1;  // accumulators per buffer: x0 w0, the small products
-    static constexpr uint32_t COLS = 2 * ACC * BN;   // TMEM columns, two buffers
+    static constexpr bool STACK = PLANES == 3 && BN == 64;          // planes of B as rows of one operand
+    static constexpr int ACC = PLANES == 1 ? 1 : STACK ? 3 : 2;     // accumulators per buffer
+    static constexpr int BUF = STACK ? 256 : ACC * BN;              // TMEM columns from one buffer to the other
+    static constexpr uint32_t COLS = 2 * BUF;
     static constexpr size_t SMEM = (size_t)STAGES * STAGE + EPI_WARPS * STAGE_OUT + 1024;
     static_assert(STAGES >= 2 && COLS <= 512, "stage ring and TMEM");
 };
@@ -228,11 +235,18 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1)
                         break;
                     }
                     tc_fence_after();
-                    const uint32_t d = tmem + (uint32_t)(b * L::ACC * BN);
+                    const uint32_t d = tmem + (uint32_t)(b * L::BUF);
                     const uint64_t da = desc0 + (uint64_t)((s * L::STAGE) >> 4), db = da + (L::A_BYTES >> 4);
                     // 16-value steps of this block that hold channels (the rest is zero fill)
                     const int ks = min(BK / 16, (p.Cp - cb * BK + 15) / 16);
-                    if constexpr (F32) {
+                    if constexpr (L::STACK) {
+                        const uint32_t id3 = idesc_f16<__nv_bfloat16>(BM, 3 * BN), id2 = idesc_f16<__nv_bfloat16>(BM, 2 * BN);
+                        for (int k = 0; k < ks; ++k) {
+                            umma<1>(d, da + 2 * k, db + 2 * k, id3, (!first || k > 0) ? 1u : 0u);
+                            umma<1>(d + BN, da + (L::A_PL >> 4) + 2 * k, db + 2 * k, id2, 1u);
+                            umma<1>(d + 2 * BN, da + 2 * (L::A_PL >> 4) + 2 * k, db + 2 * k, idesc, 1u);
+                        }
+                    } else if constexpr (F32) {
                         // small products first within the block; each accumulator sums in its own order
                         constexpr int I[6] = {0, 1, 2, 0, 1, 0}, J[6] = {2, 1, 0, 1, 0, 0};
 #pragma unroll
@@ -281,7 +295,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1)
                     break;
                 }
                 tc_fence_after();
-                const uint32_t ta = tmem + ((uint32_t)(g4 * 32) << 16) + (uint32_t)(b * L::ACC * BN + half * HC);
+                const uint32_t ta = tmem + ((uint32_t)(g4 * 32) << 16) + (uint32_t)(b * L::BUF + half * HC);
 #pragma unroll
                 for (int j = 0; j < HC; j += 32) {
                     uint32_t v[32];
@@ -289,6 +303,13 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1)
                     if constexpr (F32) {
                         uint32_t lo[32];
                         tmem_ld32(ta + BN + j, lo);
+                        if constexpr (L::STACK) {
+                            uint32_t l2[32];
+                            tmem_ld32(ta + 2 * BN + j, l2);
+#pragma unroll
+                            for (int e = 0; e < 32; ++e)
+                                lo[e] = __float_as_uint(__uint_as_float(lo[e]) + __uint_as_float(l2[e]));
+                        }
 #pragma unroll
                         for (int e = 0; e < 32; ++e) acc[j + e] += __uint_as_float(v[e]) + __uint_as_float(lo[e]);
                     } else {
