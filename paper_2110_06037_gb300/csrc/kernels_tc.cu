@@ -71,6 +71,7 @@ struct Config {
     int csk = 1;       // 2: a cluster of two CTAs splits each tile's K steps, reducing on chip
     int sk = 0;        // 1: stream-K, one equal range of the tiles' K steps per SM
     int halo = 0;      // 1: 3x3 stride 1, 8 x 16 pixel tiles, one A box per row of taps
+    int lat = 0;       // > 0: small layers, one tile per cluster of `lat` CTAs (kernels_tc_lat.cu)
 };
 
 constexpr int kSmCount = 152;  // GB300; only used to decide which K splits to offer
@@ -192,12 +193,23 @@ static std::vector<Config> configs(const Layer &l, const Shape &in, sn_schema s,
                     out.push_back(cf);
                 }
     };
+    // one tile per cluster of 1, 2, 4 or 8 CTAs, for layers whose tiles do not
+    // fill the GPU: offered up to two CTAs per SM (a CTA takes half an SM), each
+    // with a K step at least; appended last
+    auto push_lat = [&](Config cf, int64_t mtiles) {
+        for (int ncl : {1, 2, 4, 8})
+            if (mtiles * ((K + 63) / 64) * ncl <= 2 * kSmCount && kiters >= ncl) {
+                cf.BN = 64, cf.G = 1, cf.KB = 1, cf.ksplit = 1, cf.lat = ncl;
+                out.push_back(cf);
+            }
+    };
     if (plain && a_blocks == 0) {
         push_all({false, 0, 0, 0, 0, 1, 1, 1}, (N * P * Q + BM - 1) / BM);
         push_bst({false, 0, 0, 0, 0, 1, 1, 1});
         push_ms2({false, 0, 0, 0, 0, 1, 1, 1}, (N * P * Q + 2 * BM - 1) / (2 * BM));
         push_csk({false, 0, 0, 0, 0, 1, 1, 1}, (N * P * Q + BM - 1) / BM);
         push_sk({false, 0, 0, 0, 0, 1, 1, 1}, (N * P * Q + BM - 1) / BM);
+        push_lat({false, 0, 0, 0, 0, 1, 1, 1}, (N * P * Q + BM - 1) / BM);
         return out;
     }
     struct Geo {
@@ -253,6 +265,7 @@ static std::vector<Config> configs(const Layer &l, const Shape &in, sn_schema s,
                 out.push_back(cf);
             }
         }
+        for (const Geo &gg : geos(BM)) push_lat({true, 0, gg.bw, gg.bh, gg.bni, 1, 1, 1}, tiles_of(gg));
     }
     return out;
 }
@@ -300,7 +313,11 @@ std::string conv_tc_config_desc(const Layer &l, const Shape &in, sn_schema s, in
     if (v < 0 || v >= (int)cfgs.size()) return "?";
     const tc::Config &c = cfgs[v];
     char b[160];
-    if (c.implicit)
+    if (c.lat && c.implicit)
+        snprintf(b, sizeof(b), "bn=%d cluster=%d tile=%dx%dx%d", c.BN, c.lat, c.BW, c.BH, c.BNI);
+    else if (c.lat)
+        snprintf(b, sizeof(b), "bn=%d cluster=%d plain tile=%d", c.BN, c.lat, tc::BM);
+    else if (c.implicit)
         snprintf(b, sizeof(b), "bn=%d cta=%d kb=%d rows=%d ksplit=%d bst=%d csk=%d%s tile=%dx%dx%d", c.BN, c.G,
                  c.KB, 128 * c.ms * c.G, c.ksplit, c.bst ? 1 : 0, c.csk,
                  c.sk ? " streamk" : c.halo ? " halo" : "", c.BW, c.BH, c.BNI);
@@ -312,7 +329,7 @@ std::string conv_tc_config_desc(const Layer &l, const Shape &in, sn_schema s, in
 
 bool conv_tc_nchw_ok(const Layer &l, const Shape &in, sn_schema s, int32_t v, bool odd) {
     const std::vector<tc::Config> cfgs = tc::configs(l, in, s, 0, odd);
-    return v >= 0 && v < (int)cfgs.size() && cfgs[v].ksplit == 1 && !cfgs[v].sk;
+    return v >= 0 && v < (int)cfgs.size() && cfgs[v].ksplit == 1 && !cfgs[v].sk && !cfgs[v].lat;
 }
 
 size_t conv_tc_ws(const Layer &l, const Shape &in, sn_schema s, int32_t v, int32_t a_blocks, bool odd) {
@@ -362,7 +379,8 @@ cudaError_t conv_tc(const LaunchArgs &a) {
     // (one CTA's epilogue per tile, so no K split through fp32 partials)
     p.y_nchw = 0;
     if (a.out_schema.dtype >= 0 && !schema_eq(a.out_schema, a.schema)) {
-        if (a.out_schema.dtype != a.schema.dtype || a.out_schema.layout != SN_NCHW || cf.ksplit != 1 || cf.sk)
+        if (a.out_schema.dtype != a.schema.dtype || a.out_schema.layout != SN_NCHW || cf.ksplit != 1 || cf.sk ||
+            cf.lat)
             return cudaErrorInvalidValue;
         p.y_nchw = 1;
     }
@@ -427,9 +445,9 @@ cudaError_t conv_tc(const LaunchArgs &a) {
         const uint64_t ydims[2] = {(uint64_t)p.K, (uint64_t)p.Mout};
         const uint64_t ystr[1] = {p.K * es};
         const uint32_t ybox[2] = {64, 32};
-        if (!encode(&mY, dt, 2, a.out, ydims, ystr, ybox, CU_TENSOR_MAP_SWIZZLE_128B)) return cudaErrorInvalidValue;
+        if (!cf.lat && !encode(&mY, dt, 2, a.out, ydims, ystr, ybox, CU_TENSOR_MAP_SWIZZLE_128B)) return cudaErrorInvalidValue;
         mR = mY;  // the residual has the output's layout
-        if (p.res && !encode(&mR, dt, 2, p.res, ydims, ystr, ybox, CU_TENSOR_MAP_SWIZZLE_128B))
+        if (!cf.lat && p.res && !encode(&mR, dt, 2, p.res, ydims, ystr, ybox, CU_TENSOR_MAP_SWIZZLE_128B))
             return cudaErrorInvalidValue;
     } else {
         p.BW = cf.BW, p.BH = cf.BH, p.BNI = cf.BNI;
@@ -469,9 +487,9 @@ cudaError_t conv_tc(const LaunchArgs &a) {
         const uint64_t ydims[4] = {(uint64_t)p.K, (uint64_t)p.Q, (uint64_t)p.P, (uint64_t)p.N};
         const uint64_t ystr[3] = {p.K * es, (uint64_t)p.Q * p.K * es, (uint64_t)p.P * p.Q * p.K * es};
         const uint32_t ybox[4] = {64, sbw, sbh, sbn};
-        if (!encode(&mY, dt, 4, a.out, ydims, ystr, ybox, CU_TENSOR_MAP_SWIZZLE_128B)) return cudaErrorInvalidValue;
+        if (!cf.lat && !encode(&mY, dt, 4, a.out, ydims, ystr, ybox, CU_TENSOR_MAP_SWIZZLE_128B)) return cudaErrorInvalidValue;
         mR = mY;
-        if (p.res && !encode(&mR, dt, 4, p.res, ydims, ystr, ybox, CU_TENSOR_MAP_SWIZZLE_128B))
+        if (!cf.lat && p.res && !encode(&mR, dt, 4, p.res, ydims, ystr, ybox, CU_TENSOR_MAP_SWIZZLE_128B))
             return cudaErrorInvalidValue;
     }
     if (p.mtiles <= 0 || (int64_t)p.mtiles * p.ntiles * p.ksplit > INT32_MAX) return cudaErrorInvalidValue;
@@ -496,6 +514,7 @@ cudaError_t conv_tc(const LaunchArgs &a) {
         while ((1 << p.lbw) < cf.BW) ++p.lbw;
         while ((1 << p.lbwh) < cf.BW * cf.BH) ++p.lbwh;
     }
+    if (cf.lat) return launch_lat(dt, cf.BN, cf.lat, mA, mB, p, a.stream);
     const bool bf = dt == SN_BF16;
 #define SN_TC_LAUNCH(TT, BNV, GV, KBV)                                                            \
     return cf.implicit ? launch<TT, BNV, true, GV, KBV>(mA, mB, mY, mR, p, a.stream)               \

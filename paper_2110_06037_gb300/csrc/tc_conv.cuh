@@ -1051,6 +1051,11 @@ static cudaError_t launch(const CUtensorMap *mA, const CUtensorMap &mB, const CU
 cudaError_t launch_halo(int dtype, int bn, int g, const CUtensorMap *mA, const CUtensorMap &mB,
                         const CUtensorMap &mY, const CUtensorMap &mR, const Params &p, cudaStream_t st);
 
+// small layers (kernels_tc_lat.cu): a cluster of ncl in {1, 2, 4, 8} CTAs per
+// 128-pixel x 64-channel tile
+cudaError_t launch_lat(int dtype, int bn, int ncl, const CUtensorMap *mA, const CUtensorMap &mB, const Params &p,
+                       cudaStream_t st);
+
 // stream-K launches (kernels_tc_sk.cu): one-CTA tiles of bn in {128, 256}
 // output channels, kb channel blocks per stage
 cudaError_t launch_sk(int dtype, int bn, int kb, bool implicit, const CUtensorMap *mA, const CUtensorMap &mB,
