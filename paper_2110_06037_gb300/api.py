@@ -16,10 +16,29 @@ from ._sn import check, lib
 
 TORCH_DTYPES = {"f32": "float32", "f16": "float16", "bf16": "bfloat16", "qi8": "int8"}
 
+_SHAPE4 = C.c_int64 * 4  # building the ctypes array type costs as much as filling one
+_SCHEMAS = {}            # ("f16", "nhwc") -> sn_schema, passed by value
+_torch_module = None
+
 
 def _torch():
-    import torch
-    return torch
+    global _torch_module
+    if _torch_module is None:
+        import torch
+        _torch_module = torch
+    return _torch_module
+
+
+def _schema(s):
+    """_sn.schema, one object per value: marshalling a small adapt costs the host
+    more than the GPU (9.0 us a call on the GB300's Arm host before these three,
+    against a 7 us kernel)."""
+    if type(s) is tuple:
+        v = _SCHEMAS.get(s)
+        if v is None:
+            v = _SCHEMAS[s] = _sn.schema(s)
+        return v
+    return _sn.schema(s)
 
 
 class _TorchAllocator:
@@ -50,10 +69,13 @@ def storage_shape(shape_nchw, layout):
 
 
 def _stream_ptr(stream):
+    if stream is not None:
+        return stream.cuda_stream
     torch = _torch()
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return C.c_void_p(stream.cuda_stream)
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)  # the handle without a Stream object around it
+    if raw is None:
+        return torch.cuda.current_stream().cuda_stream
+    return raw(torch.cuda.current_device())
 
 
 class Graph:
@@ -259,7 +281,7 @@ class Graph:
     def run(self, x, out=None, stream=None):
         if out is None:
             out = self.new_output()
-        check(lib().sn_run(self.h, C.c_void_p(x.data_ptr()), C.c_void_p(out.data_ptr()), _stream_ptr(stream)))
+        check(lib().sn_run(self.h, x.data_ptr(), out.data_ptr(), _stream_ptr(stream)))
         return out
 
     def run_host(self, x_host, out_host, stream=None):
@@ -303,23 +325,21 @@ class Graph:
 
 def convert(x, from_schema, to_schema, shape_nchw, out=None, stream=None):
     """The adapt routine on its own: cast and/or permute a blob (bit-exact)."""
-    torch = _torch()
     if out is None:
+        torch = _torch()
         out = torch.empty(storage_shape(shape_nchw, to_schema[1]),
                           dtype=getattr(torch, TORCH_DTYPES[to_schema[0]]), device="cuda")
-    shp = (C.c_int64 * 4)(*shape_nchw)
-    check(lib().sn_convert(C.c_void_p(x.data_ptr()), _sn.schema(from_schema), C.c_void_p(out.data_ptr()),
-                           _sn.schema(to_schema), shp, _stream_ptr(stream)))
+    check(lib().sn_convert(x.data_ptr(), _schema(from_schema), out.data_ptr(), _schema(to_schema),
+                           _SHAPE4(*shape_nchw), _stream_ptr(stream)))
     return out
 
 
 def convert_q(x, from_schema, to_schema, shape_nchw, qscale, out=None, stream=None):
     """The adapt routine with a qi8 side: quantise, dequantise or permute codes."""
-    torch = _torch()
     if out is None:
+        torch = _torch()
         out = torch.empty(storage_shape(shape_nchw, to_schema[1]),
                           dtype=getattr(torch, TORCH_DTYPES[to_schema[0]]), device="cuda")
-    shp = (C.c_int64 * 4)(*shape_nchw)
-    check(lib().sn_convert_q(C.c_void_p(x.data_ptr()), _sn.schema(from_schema), C.c_void_p(out.data_ptr()),
-                             _sn.schema(to_schema), shp, C.c_float(qscale), _stream_ptr(stream)))
+    check(lib().sn_convert_q(x.data_ptr(), _schema(from_schema), out.data_ptr(), _schema(to_schema),
+                             _SHAPE4(*shape_nchw), qscale, _stream_ptr(stream)))
     return out
