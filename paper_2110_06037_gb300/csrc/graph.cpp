@@ -407,11 +407,14 @@ sn_status graph_finalize(Graph *g) {
                 for (int32_t v = 0; v < nv; ++v) cands.push_back({r, v, s, i, kInf});
                 if (nv == 0) continue;
                 // the same routine writing another schema of Lambda (fused boundary)
-                for (const sn_schema &o : fused_outputs(r, L[i], g->schemas[s]))
+                const std::vector<sn_schema> fo = fused_outputs(r, L[i], g->schemas[s]);
+                if (fo.empty()) continue;
+                const std::vector<char> ok = fused_variants_ok(r, L[i], in, g->schemas[s], nv);
+                for (const sn_schema &o : fo)
                     for (int32_t so = 0; so < g->n_lambda; ++so)
                         if (so != s && schema_eq(g->schemas[so], o))
                             for (int32_t v = 0; v < nv; ++v) {
-                                if (!fused_variant_ok(r, L[i], in, g->schemas[s], v)) continue;
+                                if (!ok[(size_t)v]) continue;
                                 Candidate c{r, v, s, i, kInf};
                                 c.out_schema = so;
                                 cands.push_back(c);

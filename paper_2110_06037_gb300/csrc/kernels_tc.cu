@@ -203,6 +203,17 @@ static std::vector<Config> configs(const Layer &l, const Shape &in, sn_schema s,
                 out.push_back(cf);
             }
     };
+    // the same kernel, one CTA per tile, for larger tile counts and 128-channel
+    // tiles: two CTAs an SM overlap one's drain with the other's K steps, and
+    // the next layer's CTAs set up beside the last ones
+    auto push_half = [&](Config cf, int64_t mtiles) {
+        for (int bn : bns) {
+            const int64_t tiles = mtiles * ((K + bn - 1) / bn);
+            if (bn == 256 || tiles > 16 * kSmCount || (bn == 64 && tiles <= 2 * kSmCount)) continue;
+            cf.BN = bn, cf.G = 1, cf.KB = 1, cf.ksplit = 1, cf.lat = 1;
+            out.push_back(cf);
+        }
+    };
     if (plain && a_blocks == 0) {
         push_all({false, 0, 0, 0, 0, 1, 1, 1}, (N * P * Q + BM - 1) / BM);
         push_bst({false, 0, 0, 0, 0, 1, 1, 1});
@@ -210,6 +221,7 @@ static std::vector<Config> configs(const Layer &l, const Shape &in, sn_schema s,
         push_csk({false, 0, 0, 0, 0, 1, 1, 1}, (N * P * Q + BM - 1) / BM);
         push_sk({false, 0, 0, 0, 0, 1, 1, 1}, (N * P * Q + BM - 1) / BM);
         push_lat({false, 0, 0, 0, 0, 1, 1, 1}, (N * P * Q + BM - 1) / BM);
+        push_half({false, 0, 0, 0, 0, 1, 1, 1}, (N * P * Q + BM - 1) / BM);
         return out;
     }
     struct Geo {
@@ -266,6 +278,7 @@ static std::vector<Config> configs(const Layer &l, const Shape &in, sn_schema s,
             }
         }
         for (const Geo &gg : geos(BM)) push_lat({true, 0, gg.bw, gg.bh, gg.bni, 1, 1, 1}, tiles_of(gg));
+        for (const Geo &gg : geos(BM)) push_half({true, 0, gg.bw, gg.bh, gg.bni, 1, 1, 1}, tiles_of(gg));
     }
     return out;
 }
@@ -327,9 +340,10 @@ std::string conv_tc_config_desc(const Layer &l, const Shape &in, sn_schema s, in
     return b;
 }
 
-bool conv_tc_nchw_ok(const Layer &l, const Shape &in, sn_schema s, int32_t v, bool odd) {
-    const std::vector<tc::Config> cfgs = tc::configs(l, in, s, 0, odd);
-    return v >= 0 && v < (int)cfgs.size() && cfgs[v].ksplit == 1 && !cfgs[v].sk && !cfgs[v].lat;
+std::vector<char> conv_tc_nchw_ok(const Layer &l, const Shape &in, sn_schema s, bool odd) {
+    std::vector<char> ok;
+    for (const tc::Config &c : tc::configs(l, in, s, 0, odd)) ok.push_back(c.ksplit == 1 && !c.sk && !c.lat);
+    return ok;
 }
 
 size_t conv_tc_ws(const Layer &l, const Shape &in, sn_schema s, int32_t v, int32_t a_blocks, bool odd) {
@@ -445,7 +459,7 @@ cudaError_t conv_tc(const LaunchArgs &a) {
         const uint64_t ydims[2] = {(uint64_t)p.K, (uint64_t)p.Mout};
         const uint64_t ystr[1] = {p.K * es};
         const uint32_t ybox[2] = {64, 32};
-        if (!cf.lat && !encode(&mY, dt, 2, a.out, ydims, ystr, ybox, CU_TENSOR_MAP_SWIZZLE_128B)) return cudaErrorInvalidValue;
+        if (cf.lat <= 1 && !encode(&mY, dt, 2, a.out, ydims, ystr, ybox, CU_TENSOR_MAP_SWIZZLE_128B)) return cudaErrorInvalidValue;
         mR = mY;  // the residual has the output's layout
         if (!cf.lat && p.res && !encode(&mR, dt, 2, p.res, ydims, ystr, ybox, CU_TENSOR_MAP_SWIZZLE_128B))
             return cudaErrorInvalidValue;
@@ -487,7 +501,7 @@ cudaError_t conv_tc(const LaunchArgs &a) {
         const uint64_t ydims[4] = {(uint64_t)p.K, (uint64_t)p.Q, (uint64_t)p.P, (uint64_t)p.N};
         const uint64_t ystr[3] = {p.K * es, (uint64_t)p.Q * p.K * es, (uint64_t)p.P * p.Q * p.K * es};
         const uint32_t ybox[4] = {64, sbw, sbh, sbn};
-        if (!cf.lat && !encode(&mY, dt, 4, a.out, ydims, ystr, ybox, CU_TENSOR_MAP_SWIZZLE_128B)) return cudaErrorInvalidValue;
+        if (cf.lat <= 1 && !encode(&mY, dt, 4, a.out, ydims, ystr, ybox, CU_TENSOR_MAP_SWIZZLE_128B)) return cudaErrorInvalidValue;
         mR = mY;
         if (!cf.lat && p.res && !encode(&mR, dt, 4, p.res, ydims, ystr, ybox, CU_TENSOR_MAP_SWIZZLE_128B))
             return cudaErrorInvalidValue;
@@ -514,7 +528,7 @@ cudaError_t conv_tc(const LaunchArgs &a) {
         while ((1 << p.lbw) < cf.BW) ++p.lbw;
         while ((1 << p.lbwh) < cf.BW * cf.BH) ++p.lbwh;
     }
-    if (cf.lat) return launch_lat(dt, cf.BN, cf.lat, mA, mB, p, a.stream);
+    if (cf.lat) return launch_lat(dt, cf.BN, cf.lat, mA, mB, mY, p, a.stream);
     const bool bf = dt == SN_BF16;
 #define SN_TC_LAUNCH(TT, BNV, GV, KBV)                                                            \
     return cf.implicit ? launch<TT, BNV, true, GV, KBV>(mA, mB, mY, mR, p, a.stream)               \

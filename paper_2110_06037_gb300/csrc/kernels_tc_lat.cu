@@ -14,9 +14,9 @@
 //     its own, so that only boxes of A are left on the critical path;
 //   * a CTA keeps to half an SM (three stages, one accumulator), so the next
 //     kernel's CTAs can set up and copy their weights beside it;
-//   * rows go from registers straight to global memory (no staging, no TMA
-//     store), the residual's and the bias' loads are in flight before the
-//     accumulator is ready.
+//   * the residual's and the bias' loads are in flight before the accumulator
+//     is ready; a cluster's rows go from registers straight to global memory, a
+//     single CTA's tile through the stage memory and a TMA store.
 // The sum of a tile is deterministic: fixed ranges, fixed order.  Waits are
 // bounded as in tc_conv.cuh.
 // Measured (fp16, a pass of a replayed net): MobileNetV2 at batch 1 239.6 ->
@@ -46,10 +46,11 @@ __device__ __forceinline__ void st_async_v4(uint32_t caddr, uint32_t cbar, uint3
 }
 
 template <typename T, int BN, int NCL>
-__global__ void __launch_bounds__(LAT_THREADS)
+__global__ void __launch_bounds__(LAT_THREADS, 2)
     conv_tc_lat_kernel(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ CUtensorMap mA1,
                        const __grid_constant__ CUtensorMap mA2, const __grid_constant__ CUtensorMap mA3,
-                       const __grid_constant__ CUtensorMap mB, const __grid_constant__ Params p) {
+                       const __grid_constant__ CUtensorMap mB, const __grid_constant__ CUtensorMap mY,
+                       const __grid_constant__ Params p) {
     constexpr uint32_t A_BYTES = BM * BK * 2, STAGE = A_BYTES + BN * BK * 2;
     constexpr int CW = BN / NCL;  // columns this CTA finishes
     static_assert(CW >= 8 && CW % 8 == 0, "whole 16-byte pieces of a row");
@@ -72,6 +73,12 @@ __global__ void __launch_bounds__(LAT_THREADS)
     const Work w = work_of(p, tile, BN, p.BW > 0, 1, 1);
     // this CTA's K steps
     const int it0 = p.kiters * (int)rank / NCL, it1 = p.kiters * ((int)rank + 1) / NCL, nit = it1 - it0;
+    if (threadIdx.x == 32) {  // the maps are kernel parameters, not data of the previous kernel
+        const CUtensorMap *maps[6] = {&mB, &mA0, &mA1, &mA2, &mA3, &mY};
+        for (int i = 0; i < 6; ++i)
+            if (i < 2 || (i < 5 ? p.stride != 1 : NCL == 1))
+                asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(maps[i])) : "memory");
+    }
     if (threadIdx.x == 0) {
         for (int s = 0; s < LAT_STAGES; ++s) {
             mbar_init(&full_bar[s], 1);
@@ -167,7 +174,89 @@ __global__ void __launch_bounds__(LAT_THREADS)
             if (i == nit) umma_commit<1>(&accf_bar);
             consumed_sh = i;
         }
-    } else {  // ---------------- epilogue: warp w drains rows 32 w .. 32 w + 31
+    } else if constexpr (NCL == 1) {  // ---------------- epilogue: warp w drains rows 32 w .. 32 w + 31
+        // 32 columns at a time; the tile goes out through the stage memory, which
+        // the MMAs are done with once the accumulator is ready: a warp's 32 rows x
+        // 64 channels, 128-byte swizzled, one TMA store (clipped at the edges)
+        const int r0 = warp * 32, row = r0 + lane;
+        const bool imp = p.BW > 0;
+        const int sq = w.q0 + (imp ? r0 & (p.BW - 1) : 0), sp = w.p0 + (imp ? (r0 >> p.lbw) & (p.BH - 1) : 0),
+                  sn_ = w.i0 + (imp ? r0 >> p.lbwh : 0);
+        bool valid;
+        int64_t pix;
+        if (imp) {
+            const int q = w.q0 + (row & (p.BW - 1)), pp = w.p0 + ((row >> p.lbw) & (p.BH - 1)), n = w.i0 + (row >> p.lbwh);
+            valid = q < p.Q && pp < p.P && n < p.N;
+            pix = ((int64_t)n * p.P + pp) * p.Q + q;
+        } else {
+            pix = w.m0 + row;
+            valid = pix < p.Mout;
+        }
+        const T *res = p.res && valid ? static_cast<const T *>(p.res) + pix * p.K : nullptr;
+        uint4 rq[4];
+        auto load_res = [&](int k) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                rq[j] = res && k + 8 * j < p.K ? *reinterpret_cast<const uint4 *>(res + k + 8 * j) : make_uint4(0u, 0u, 0u, 0u);
+        };
+        griddep_wait();
+        load_res(w.n0);
+        const bool ok = mbar_wait(&accf_bar, 0u, p.wait_limit);
+        if (!__all_sync(0xffffffffu, ok)) {
+            if (lane == 0) atomicOr(p.err, ERR_ACC_WAIT);
+            abort_sh = 1;
+        } else {
+            tc_fence_after();
+            const uint32_t ta = tmem + ((uint32_t)(warp * 32) << 16);
+            auto drain = [&](auto act) {
+#pragma unroll
+                for (int c = 0; c < BN / 32; ++c) {
+                    const int k0 = w.n0 + 32 * c;
+                    if (k0 >= p.K) break;
+                    uint8_t *buf = smem + (c >> 1) * (BM * 128) + warp * 4096;
+                    uint32_t v[32];
+                    tmem_ld32(ta + 32 * c, v);
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const float4 b0 = __ldg(reinterpret_cast<const float4 *>(p.bias + k0 + 8 * j)),
+                                     b1 = __ldg(reinterpret_cast<const float4 *>(p.bias + k0 + 8 * j) + 1);
+                        const float b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+                        const uint32_t rw[4] = {rq[j].x, rq[j].y, rq[j].z, rq[j].w};
+                        uint32_t o[4];
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            const float2 r2 = unpack2<T>(rw[e]);
+                            o[e] = pack2<T>(act(__uint_as_float(v[8 * j + 2 * e]) + b[2 * e] + r2.x),
+                                            act(__uint_as_float(v[8 * j + 2 * e + 1]) + b[2 * e + 1] + r2.y));
+                        }
+                        const int piece = (c & 1) * 4 + j;
+                        *reinterpret_cast<uint4 *>(buf + lane * 128 + ((piece ^ (lane & 7)) << 4)) =
+                            make_uint4(o[0], o[1], o[2], o[3]);
+                    }
+                    if (c + 1 < BN / 32) load_res(k0 + 32);
+                    if ((c & 1) || k0 + 32 >= p.K) {  // the 64-channel block is complete
+                        fence_proxy_async_smem();
+                        __syncwarp();
+                        if (lane == 0) {
+                            const int kb = w.n0 + 64 * (c >> 1);
+                            if (imp) tma_store_4d(&mY, buf, kb, sq, sp, sn_);
+                            else tma_store_2d(&mY, buf, kb, (int)(w.m0 + r0));
+                            bulk_commit();
+                        }
+                        __syncwarp();
+                    }
+                }
+            };
+            if (p.act == SN_ACT_RELU || p.act == SN_ACT_RELU6)
+                drain([hi = p.act == SN_ACT_RELU ? INFINITY : 6.0f](float x) { return fminf(fmaxf(x, 0.0f), hi); });
+            else if (p.act == SN_ACT_NONE)
+                drain([](float x) { return x; });
+            else
+                drain([act = p.act](float x) { return act_apply(x, act); });
+            if (lane == 0) bulk_wait_read_0();  // the stores have read the stage memory
+            __syncwarp();
+        }
+    } else {  // ---------------- epilogue of a cluster: warp w drains rows 32 w .. 32 w + 31
         const int row = warp * 32 + lane;
         const int k0 = w.n0 + (int)rank * CW;  // first output channel of this CTA's columns
         bool valid;
@@ -210,48 +299,42 @@ __global__ void __launch_bounds__(LAT_THREADS)
                 for (int j = 0; j < 8; ++j) {
                     const int col = 32 * c + 4 * j;
                     const uint32_t dst = (uint32_t)(col / CW);
-                    if (NCL > 1 && dst != rank) {
+                    if (dst != rank) {
                         const uint32_t at = su32(xch + ((int)rank * (CW / 4) + (col % CW) / 4) * BM + row);
                         st_async_v4(mapa(at, dst), mapa(su32(&x_bar[warp]), dst), v[4 * j], v[4 * j + 1], v[4 * j + 2],
                                     v[4 * j + 3]);
-                    } else if (NCL == 1) {
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) own[col % CW + e] = __uint_as_float(v[4 * j + e]);
                     }
                 }
             }
-            if constexpr (NCL > 1) {  // this CTA's own columns: a runtime offset, so read again
+            // this CTA's own columns: a runtime offset, so read again
 #pragma unroll
-                for (int c = 0; c < CW / 8; ++c) {
-                    uint32_t v[8];
-                    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
-                                 : "r"(ta + rank * CW + 8 * c));
-                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+            for (int c = 0; c < CW / 8; ++c) {
+                uint32_t v[8];
+                asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                             : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
+                             : "r"(ta + rank * CW + 8 * c));
+                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) own[8 * c + e] = __uint_as_float(v[e]);
-                }
-                ok = mbar_wait_cluster(&x_bar[warp], 0u, p.wait_limit);
-                ok = __all_sync(0xffffffffu, ok);
-                if (!ok) {
-                    if (lane == 0) atomicOr(p.err, ERR_EPI_WAIT);
-                    abort_sh = 1;
-                }
+                for (int e = 0; e < 8; ++e) own[8 * c + e] = __uint_as_float(v[e]);
+            }
+            ok = mbar_wait_cluster(&x_bar[warp], 0u, p.wait_limit);
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) {
+                if (lane == 0) atomicOr(p.err, ERR_EPI_WAIT);
+                abort_sh = 1;
             }
             if (ok) {
                 float sum[CW];
 #pragma unroll
-                for (int e = 0; e < CW; ++e) sum[e] = NCL > 1 ? 0.f : own[e];
-                if constexpr (NCL > 1) {
+                for (int e = 0; e < CW; ++e) sum[e] = 0.f;
 #pragma unroll
-                    for (int r = 0; r < NCL; ++r)
+                for (int r = 0; r < NCL; ++r)
 #pragma unroll
-                        for (int j = 0; j < CW / 4; ++j) {
-                            float4 x = make_float4(own[4 * j], own[4 * j + 1], own[4 * j + 2], own[4 * j + 3]);
-                            if (r != (int)rank) x = xch[(r * (CW / 4) + j) * BM + row];
-                            sum[4 * j] += x.x, sum[4 * j + 1] += x.y, sum[4 * j + 2] += x.z, sum[4 * j + 3] += x.w;
-                        }
-                }
+                    for (int j = 0; j < CW / 4; ++j) {
+                        float4 x = make_float4(own[4 * j], own[4 * j + 1], own[4 * j + 2], own[4 * j + 3]);
+                        if (r != (int)rank) x = xch[(r * (CW / 4) + j) * BM + row];
+                        sum[4 * j] += x.x, sum[4 * j + 1] += x.y, sum[4 * j + 2] += x.z, sum[4 * j + 3] += x.w;
+                    }
                 T *y = static_cast<T *>(p.y) + pix * p.K + k0;
 #pragma unroll
                 for (int j = 0; j < CW / 8; ++j) {
@@ -296,7 +379,8 @@ __global__ void __launch_bounds__(LAT_THREADS)
 }
 
 template <typename T, int BN, int NCL>
-static cudaError_t launch_lat_t(const CUtensorMap *mA, const CUtensorMap &mB, const Params &p, cudaStream_t st) {
+static cudaError_t launch_lat_t(const CUtensorMap *mA, const CUtensorMap &mB, const CUtensorMap &mY, const Params &p,
+                                cudaStream_t st) {
     constexpr size_t smem = (size_t)LAT_STAGES * (BM + BN) * BK * 2 + (NCL > 1 ? (size_t)BM * BN * 4 : 0) + 1024;
     auto kern = conv_tc_lat_kernel<T, BN, NCL>;
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -318,26 +402,26 @@ static cudaError_t launch_lat_t(const CUtensorMap *mA, const CUtensorMap &mB, co
         attr[1].val.clusterDim.z = 1;
         cfg.numAttrs = 2;
     }
-    return cudaLaunchKernelEx(&cfg, kern, mA[0], mA[1], mA[2], mA[3], mB, p);
+    return cudaLaunchKernelEx(&cfg, kern, mA[0], mA[1], mA[2], mA[3], mB, mY, p);
 }
 
 template <typename T>
-static cudaError_t launch_lat_d(int bn, int ncl, const CUtensorMap *mA, const CUtensorMap &mB, const Params &p,
-                                cudaStream_t st) {
-    if (bn == 64) {
-        if (ncl == 1) return launch_lat_t<T, 64, 1>(mA, mB, p, st);
-        if (ncl == 2) return launch_lat_t<T, 64, 2>(mA, mB, p, st);
-        if (ncl == 4) return launch_lat_t<T, 64, 4>(mA, mB, p, st);
-        if (ncl == 8) return launch_lat_t<T, 64, 8>(mA, mB, p, st);
-    }
+static cudaError_t launch_lat_d(int bn, int ncl, const CUtensorMap *mA, const CUtensorMap &mB, const CUtensorMap &mY,
+                                const Params &p, cudaStream_t st) {
+    if (bn == 128 && ncl == 1) return launch_lat_t<T, 128, 1>(mA, mB, mY, p, st);
+    if (bn != 64) return cudaErrorInvalidValue;
+    if (ncl == 1) return launch_lat_t<T, 64, 1>(mA, mB, mY, p, st);
+    if (ncl == 2) return launch_lat_t<T, 64, 2>(mA, mB, mY, p, st);
+    if (ncl == 4) return launch_lat_t<T, 64, 4>(mA, mB, mY, p, st);
+    if (ncl == 8) return launch_lat_t<T, 64, 8>(mA, mB, mY, p, st);
     return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_lat(int dtype, int bn, int ncl, const CUtensorMap *mA, const CUtensorMap &mB, const Params &p,
-                       cudaStream_t st) {
+cudaError_t launch_lat(int dtype, int bn, int ncl, const CUtensorMap *mA, const CUtensorMap &mB, const CUtensorMap &mY,
+                       const Params &p, cudaStream_t st) {
     if (p.ksplit != 1 || p.y_nchw || p.kiters < ncl || (uintptr_t)p.y % 16) return cudaErrorInvalidValue;
-    if (dtype == SN_BF16) return launch_lat_d<__nv_bfloat16>(bn, ncl, mA, mB, p, st);
-    return launch_lat_d<__half>(bn, ncl, mA, mB, p, st);
+    if (dtype == SN_BF16) return launch_lat_d<__nv_bfloat16>(bn, ncl, mA, mB, mY, p, st);
+    return launch_lat_d<__half>(bn, ncl, mA, mB, mY, p, st);
 }
 
 }  // namespace tc

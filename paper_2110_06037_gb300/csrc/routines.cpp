@@ -294,14 +294,13 @@ std::vector<sn_schema> fused_outputs(int32_t r, const Layer &l, sn_schema s) {
     }
 }
 
-bool fused_variant_ok(int32_t r, const Layer &l, const std::vector<Shape> &in, sn_schema s, int32_t v) {
-    if (s.dtype == SN_QI8) return true;
+std::vector<char> fused_variants_ok(int32_t r, const Layer &l, const std::vector<Shape> &in, sn_schema s, int32_t nv) {
     // the NCHW writer drains each tile in one CTA's epilogue: no K split
-    // through fp32 partials, no stream-K parts
-    if ((r == R_CONV_TC || r == R_CONV_TC_ODD) && !in.empty())
-        return k::conv_tc_nchw_ok(l, in[0], s, v, r == R_CONV_TC_ODD);
-    if (r == R_CONV_S2D_TC) return true;  // one-CTA tiles without a K split
-    return false;
+    // through fp32 partials, no stream-K parts, no cluster tiles
+    if (s.dtype != SN_QI8 && (r == R_CONV_TC || r == R_CONV_TC_ODD) && !in.empty())
+        return k::conv_tc_nchw_ok(l, in[0], s, r == R_CONV_TC_ODD);
+    // qint8 routines, and the stem's one-CTA tiles without a K split
+    return std::vector<char>((size_t)nv, s.dtype == SN_QI8 || r == R_CONV_S2D_TC);
 }
 
 int32_t childnet_stages(int32_t r, sn_schema s) {

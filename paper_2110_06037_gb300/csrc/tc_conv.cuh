@@ -1052,9 +1052,9 @@ cudaError_t launch_halo(int dtype, int bn, int g, const CUtensorMap *mA, const C
                         const CUtensorMap &mY, const CUtensorMap &mR, const Params &p, cudaStream_t st);
 
 // small layers (kernels_tc_lat.cu): a cluster of ncl in {1, 2, 4, 8} CTAs per
-// 128-pixel x 64-channel tile
-cudaError_t launch_lat(int dtype, int bn, int ncl, const CUtensorMap *mA, const CUtensorMap &mB, const Params &p,
-                       cudaStream_t st);
+// 128-pixel x 64-channel tile, or one CTA per 128 x 128 tile
+cudaError_t launch_lat(int dtype, int bn, int ncl, const CUtensorMap *mA, const CUtensorMap &mB, const CUtensorMap &mY,
+                       const Params &p, cudaStream_t st);
 
 // stream-K launches (kernels_tc_sk.cu): one-CTA tiles of bn in {128, 256}
 // output channels, kb channel blocks per stage
