@@ -283,6 +283,12 @@ SN_API sn_status sn_set_path(sn_graph *g, const int32_t *candidate, int32_t n_la
                                ranges do not overlap share bytes of the plan's
                                arena (sn_plan_memory); 0 = every blob its own
                                bytes.  The outputs are the same either way.   */
+#define SN_OPT_PAIR 5       /* 1 (default) = a 1x1 convolution on the tensor-core
+                               routine and the depthwise convolution that alone
+                               reads it run as one launch (the values are those
+                               of the two launches; not with SN_OPT_CHAIN, and
+                               never while profiling or in sn_run_timed);
+                               0 = one launch per layer.                       */
 #define SN_OPT_WAIT_LIMIT 3 /* SM clock cycles that one pipeline wait of a
                                tensor-core routine (conv2/igemm_tc and the
                                routines built on it) may take before the kernel

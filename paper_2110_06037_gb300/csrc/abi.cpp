@@ -296,6 +296,11 @@ sn_status sn_set_option(sn_graph *gg, int32_t option, int64_t value) {
                 g->opt_share = value ? 1 : 0;
                 invalidate_plan(g);
             }
+        } else if (option == SN_OPT_PAIR) {
+            if (g->opt_pair != (value ? 1 : 0)) {
+                g->opt_pair = value ? 1 : 0;
+                invalidate_plan(g);
+            }
         } else if (option == SN_OPT_CHAIN) {
             if (g->opt_chain != (value ? 1 : 0)) {
                 g->opt_chain = value ? 1 : 0;
@@ -536,6 +541,9 @@ sn_status sn_plan_stats(sn_graph *gg, int32_t *n_ops, int32_t *n_kernels, void *
             const PlanOp &op = g->plan[q];
             if (q < g->op_chain.size() && g->op_chain[q] >= 0) {  // one launch per chain
                 kern += g->chains[g->op_chain[q]].first_op == (int32_t)q ? 1 : 0;
+            } else if (paired(g, q)) {  // two layers, one launch
+                kern += 1;
+                ++q;
             } else if (op.kind == PlanOp::ADAPT) {
                 kern += 1;
             } else {

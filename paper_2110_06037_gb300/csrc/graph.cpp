@@ -99,6 +99,7 @@ void invalidate_plan(Graph *g) {
     }
     g->chains.clear();
     g->op_chain.clear();
+    g->op_pair.clear();
     if (g->gexec) {
         cudaGraphExecDestroy(g->gexec);
         g->gexec = nullptr;

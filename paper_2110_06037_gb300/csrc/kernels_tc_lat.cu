@@ -381,7 +381,10 @@ __global__ void __launch_bounds__(LAT_THREADS, 2)
 template <typename T, int BN, int NCL>
 static cudaError_t launch_lat_t(const CUtensorMap *mA, const CUtensorMap &mB, const CUtensorMap &mY, const Params &p,
                                 cudaStream_t st) {
-    constexpr size_t smem = (size_t)LAT_STAGES * (BM + BN) * BK * 2 + (NCL > 1 ? (size_t)BM * BN * 4 : 0) + 1024;
+    // (at least a third of an SM: no more than two CTAs share one, so tensor
+    // memory never runs out while a CTA of the next kernel waits for this one)
+    constexpr size_t need = (size_t)LAT_STAGES * (BM + BN) * BK * 2 + (NCL > 1 ? (size_t)BM * BN * 4 : 0) + 1024;
+    constexpr size_t smem = need > 80 * 1024 ? need : 80 * 1024;
     auto kern = conv_tc_lat_kernel<T, BN, NCL>;
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;

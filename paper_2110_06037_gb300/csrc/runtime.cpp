@@ -59,6 +59,33 @@ sn_status ensure_tile_counts(Graph *g, cudaStream_t st) {
     return SN_OK;
 }
 
+// Pairs of plan ops that one launch can run: a 1x1 stride-1 convolution on the
+// tensor-core routine and the depthwise convolution next in the plan that alone
+// reads its (graph-owned) output, both in one 16-bit NHWC schema.  The values
+// are those of the two launches, so the selected path and its routines stay.
+bool paired(const Graph *g, size_t q) { return q < g->op_pair.size() && g->op_pair[q]; }
+
+static void find_pairs(Graph *g) {
+    g->op_pair.assign(g->plan.size(), 0);
+    if (!g->opt_pair || g->profiling || g->opt_chain) return;
+    for (size_t q = 0; q + 1 < g->plan.size(); ++q) {
+        const PlanOp &a = g->plan[q], &b = g->plan[q + 1];
+        if (a.kind != PlanOp::LAYER || b.kind != PlanOp::LAYER || a.in_slots.size() != 1 || b.in_slots.size() != 1) continue;
+        if (b.in_slots[0] != a.out_slot || a.out_slot < g->n_ext || (q > 0 && g->op_pair[q - 1])) continue;
+        const Candidate &ca = g->cands[a.cand], &cb = g->cands[b.cand];
+        if (ca.routine != R_CONV_TC || cb.routine != R_DW_DIRECT || ca.schema != cb.schema || cand_out(ca) != ca.schema ||
+            cand_out(cb) != cb.schema)
+            continue;
+        int readers = 0;
+        for (const PlanOp &op : g->plan)
+            for (int32_t s : op.in_slots) readers += s == a.out_slot;
+        const Layer &la = g->layers[a.layer];
+        if (readers == 1 && la.inputs.size() == 1 &&
+            k::expand_dw_plan(la, g->layers[la.inputs[0]].out, g->layers[b.layer], g->schemas[ca.schema]).MT > 0)
+            g->op_pair[q] = 1;
+    }
+}
+
 static sn_status place_slots(Graph *g) {
     const size_t ns = g->slots.size();
     std::vector<int32_t> first(ns, INT32_MAX), last(ns, -1);
@@ -72,6 +99,9 @@ static sn_status place_slots(Graph *g) {
         for (int32_t s : op.in_slots) touch(s, (int32_t)q, (int32_t)q);
         touch(op.out_slot, (int32_t)q, (int32_t)q);
     }
+    for (size_t q = 0; q + 1 < g->plan.size(); ++q)
+        if (paired(g, q))  // the first op's input is read while the second's output is written
+            for (int32_t s : g->plan[q].in_slots) touch(s, (int32_t)q, (int32_t)q + 1);
     if (g->opt_chain && !g->profiling)
         for (const auto &r : chain_runs(g))
             for (int32_t q = r.first; q <= r.second; ++q) {
@@ -230,6 +260,7 @@ sn_status build_plan(Graph *g, cudaStream_t st) {
             return fail(SN_ESTATE, "the path keeps a blob in qi8 without a scale (sn_set_qscale or sn_calibrate)");
         }
     }
+    find_pairs(g);
     {
         sn_status rc = place_slots(g);
         if (rc != SN_OK) return rc;
@@ -342,21 +373,15 @@ sn_status build_chains(Graph *g, cudaStream_t st) {
     return SN_OK;
 }
 
-static sn_status launch_op(Graph *g, const PlanOp &op, const IoPtrs &io, cudaStream_t st) {
+static void *slot_ptr(const Graph *g, const IoPtrs &io, int32_t s) {
     const int32_t m_in = (int32_t)io.in.size();
-    auto ptr = [&](int32_t s) -> void * {
-        if (s < m_in) return const_cast<void *>(io.in[s]);
-        if (s < g->n_ext) return io.out[s - m_in];
-        return g->slots[s].ptr;
-    };
-    if (op.kind == PlanOp::ADAPT) {
-        const int32_t si = op.in_slots[0], so = op.out_slot;
-        const sn_schema a = g->slot_schema[si], b = g->slot_schema[so];
-        const float qs = a.dtype == SN_QI8 ? g->slot_qscale[si] : g->slot_qscale[so];  // the qi8 side's
-        cudaError_t e = convert_blob(ptr(si), a, ptr(so), b, g->slot_shape[si], qs, st);
-        if (e != cudaSuccess) return fail(SN_ECUDA, std::string("adapt: ") + cudaGetErrorString(e));
-        return SN_OK;
-    }
+    if (s < m_in) return const_cast<void *>(io.in[s]);
+    if (s < g->n_ext) return io.out[s - m_in];
+    return g->slots[s].ptr;
+}
+
+// everything the routine of a layer op needs
+static LaunchArgs op_args(Graph *g, const PlanOp &op, const IoPtrs &io, cudaStream_t st) {
     const Layer &L = g->layers[op.layer];
     const Candidate &c = g->cands[op.cand];
     LaunchArgs a;
@@ -367,11 +392,11 @@ static sn_status launch_op(Graph *g, const PlanOp &op, const IoPtrs &io, cudaStr
     a.schema = g->schemas[c.schema];
     a.out_schema = g->schemas[cand_out(c)];
     for (size_t k = 0; k < op.in_slots.size(); ++k) {
-        a.in[k] = ptr(op.in_slots[k]);
+        a.in[k] = slot_ptr(g, io, op.in_slots[k]);
         a.in_shapes.push_back(g->layers[L.inputs[k]].out);
         a.qs_in[k] = g->slot_qscale[op.in_slots[k]];
     }
-    a.out = ptr(op.out_slot);
+    a.out = slot_ptr(g, io, op.out_slot);
     a.qs_out = g->slot_qscale[op.out_slot];
     a.wt = op.wt;
     a.bias = op.bias;
@@ -381,7 +406,33 @@ static sn_status launch_op(Graph *g, const PlanOp &op, const IoPtrs &io, cudaStr
     a.tile_counts = static_cast<int *>(g->tile_counts.ptr);
     a.tile_counts_n = (int64_t)(g->tile_counts.bytes / sizeof(int));
     a.stream = st;
-    return launch_routine(a);
+    return a;
+}
+
+// ops q and q + 1 in one launch (in two where the caller's output buffer is not
+// aligned to the 16-byte stores of the pair)
+static sn_status launch_op(Graph *g, const PlanOp &op, const IoPtrs &io, cudaStream_t st);
+static sn_status launch_pair(Graph *g, size_t q, const IoPtrs &io, cudaStream_t st) {
+    const LaunchArgs a = op_args(g, g->plan[q], io, st), b = op_args(g, g->plan[q + 1], io, st);
+    if ((uintptr_t)b.out % 16) {
+        const sn_status rc = launch_op(g, g->plan[q], io, st);
+        return rc != SN_OK ? rc : launch_op(g, g->plan[q + 1], io, st);
+    }
+    const cudaError_t e = k::expand_dw(a, b, k::expand_dw_plan(*a.layer, a.in_shapes[0], *b.layer, a.schema));
+    if (e != cudaSuccess) return fail(SN_ECUDA, std::string("expand + depthwise: ") + cudaGetErrorString(e));
+    return SN_OK;
+}
+
+static sn_status launch_op(Graph *g, const PlanOp &op, const IoPtrs &io, cudaStream_t st) {
+    if (op.kind == PlanOp::ADAPT) {
+        const int32_t si = op.in_slots[0], so = op.out_slot;
+        const sn_schema a = g->slot_schema[si], b = g->slot_schema[so];
+        const float qs = a.dtype == SN_QI8 ? g->slot_qscale[si] : g->slot_qscale[so];  // the qi8 side's
+        cudaError_t e = convert_blob(slot_ptr(g, io, si), a, slot_ptr(g, io, so), b, g->slot_shape[si], qs, st);
+        if (e != cudaSuccess) return fail(SN_ECUDA, std::string("adapt: ") + cudaGetErrorString(e));
+        return SN_OK;
+    }
+    return launch_routine(op_args(g, op, io, st));
 }
 
 sn_status run_plan(Graph *g, const IoPtrs &io, cudaStream_t st, std::vector<cudaEvent_t> *evs) {
@@ -399,6 +450,11 @@ sn_status run_plan(Graph *g, const IoPtrs &io, cudaStream_t st, std::vector<cuda
                                                 static_cast<int32_t *>(c.done.ptr), c.done_count, st);
                 if (e != cudaSuccess) return fail(SN_ECUDA, std::string("chained launch: ") + cudaGetErrorString(e));
             }
+            continue;
+        }
+        if (!evs && paired(g, i)) {
+            sn_status rc = launch_pair(g, i++, io, st);
+            if (rc != SN_OK) return rc;
             continue;
         }
         // external records: timing nodes when the stream is being captured

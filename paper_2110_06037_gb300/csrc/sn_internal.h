@@ -233,6 +233,8 @@ struct Graph {
     int opt_chain = 0;                // run runs of tensor-core convolutions as chained launches
     std::vector<ChainPlan> chains;    // built with the plan
     std::vector<int32_t> op_chain;    // per plan op: its chain, or -1
+    std::vector<char> op_pair;        // per plan op: 1 = launched together with the next op (expand_dw)
+    int opt_pair = 1;                 // SN_OPT_PAIR
     bool profiling = false;           // plans built while profiling may lack qint8 scales
     cudaGraphExec_t gexec = nullptr;
     std::vector<const void *> gexec_in;
@@ -311,6 +313,8 @@ void fastest_per_schema(const Graph &g, std::vector<int64_t> &F, std::vector<int
 // plan + run
 sn_status build_plan(Graph *g, cudaStream_t st);
 sn_status build_chains(Graph *g, cudaStream_t st);
+// whether plan ops q and q + 1 run as one launch (a pointwise convolution and its depthwise reader)
+bool paired(const Graph *g, size_t q);
 // [first op, last op] of every run of plan ops that a chained launch would run
 std::vector<std::pair<int32_t, int32_t>> chain_runs(const Graph *g);
 sn_status run_plan(Graph *g, const IoPtrs &io, cudaStream_t st,
@@ -385,6 +389,13 @@ size_t conv_split_ws(const Layer &l, const Shape &in, sn_schema s);
 size_t split_weight_bytes(int64_t K, int64_t C, int64_t RS, int dt);
 cudaError_t weight_split(const float *w_kcrs, void *out, int dt, int64_t K, int64_t C, int64_t RS, cudaStream_t st);
 cudaError_t conv_split(const LaunchArgs &a, int32_t v);
+// a pointwise convolution and the depthwise convolution that alone reads it in
+// one launch: pixel tiles per CTA (0: not this pair), output rows per band, bands
+struct ExpandDwPlan {
+    int32_t MT, PB, bands;
+};
+ExpandDwPlan expand_dw_plan(const Layer &conv, const Shape &in, const Layer &dw, sn_schema s);
+cudaError_t expand_dw(const LaunchArgs &conv, const LaunchArgs &dw, const ExpandDwPlan &pl);
 cudaError_t dwconv(const LaunchArgs &a);
 bool dw3_band_applies(const Layer &l, const Shape &in, sn_schema s);  // NHWC small-map depthwise kernel
 cudaError_t maxpool(const LaunchArgs &a);
