@@ -62,6 +62,7 @@ __global__ void __launch_bounds__(LAT_THREADS, 2)
     __shared__ uint32_t tmem_sh;
     __shared__ volatile int abort_sh;
     __shared__ int issued_sh[LAT_STAGES], consumed_sh;
+    __shared__ __align__(16) float bias_sh[BN];  // like all weights not written by the previous kernel
 
     griddep_launch();
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -93,6 +94,7 @@ __global__ void __launch_bounds__(LAT_THREADS, 2)
         if (NCL > 1)
             for (int i = 0; i < 4; ++i) mbar_expect_tx(&x_bar[i], (NCL - 1) * 32 * CW * 4);
     }
+    if (threadIdx.x < BN) bias_sh[threadIdx.x] = __ldg(p.bias + w.n0 + threadIdx.x);  // zero-padded to 256 channels
     if (warp == 4) tmem_alloc<1>(&tmem_sh, BN);
     tc_fence_before();
     if (NCL > 1) cluster_sync_all();  // every CTA's barriers exist before a peer signals them
@@ -156,11 +158,13 @@ __global__ void __launch_bounds__(LAT_THREADS, 2)
             int s = 0, i = 0;
             uint32_t par = 0;
             for (; i < nit; ++i) {
+                // (no look at abort_sh: a shared-memory access of this thread queues
+                // behind the MMAs' operand reads, ~200 cycles; every wait is bounded)
                 if (!mbar_wait(&full_bar[s], par, p.wait_limit)) {
                     atomicOr(p.err, ERR_MMA_WAIT);
                     abort_sh = 1;
+                    break;
                 }
-                if (abort_sh) break;
                 tc_fence_after();
                 const uint64_t da = desc0 + (uint64_t)((s * STAGE) >> 4), db = da + (A_BYTES >> 4);
 #pragma unroll
@@ -218,8 +222,8 @@ __global__ void __launch_bounds__(LAT_THREADS, 2)
                     tmem_ld32(ta + 32 * c, v);
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
-                        const float4 b0 = __ldg(reinterpret_cast<const float4 *>(p.bias + k0 + 8 * j)),
-                                     b1 = __ldg(reinterpret_cast<const float4 *>(p.bias + k0 + 8 * j) + 1);
+                        const float4 b0 = *reinterpret_cast<const float4 *>(bias_sh + 32 * c + 8 * j),
+                                     b1 = *reinterpret_cast<const float4 *>(bias_sh + 32 * c + 8 * j + 4);
                         const float b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
                         const uint32_t rw[4] = {rq[j].x, rq[j].y, rq[j].z, rq[j].w};
                         uint32_t o[4];
@@ -269,12 +273,7 @@ __global__ void __launch_bounds__(LAT_THREADS, 2)
             pix = w.m0 + row;
             valid = pix < p.Mout;
         }
-        float acc[CW];  // starts as the bias (zero-padded to a multiple of 256 channels)
-#pragma unroll
-        for (int j = 0; j < CW / 4; ++j) {
-            const float4 b4 = __ldg(reinterpret_cast<const float4 *>(p.bias + k0) + j);
-            acc[4 * j] = b4.x, acc[4 * j + 1] = b4.y, acc[4 * j + 2] = b4.z, acc[4 * j + 3] = b4.w;
-        }
+        const float *bias = bias_sh + rank * CW;
         griddep_wait();
         uint4 res[CW / 8];
 #pragma unroll
@@ -336,19 +335,27 @@ __global__ void __launch_bounds__(LAT_THREADS, 2)
                         sum[4 * j] += x.x, sum[4 * j + 1] += x.y, sum[4 * j + 2] += x.z, sum[4 * j + 3] += x.w;
                     }
                 T *y = static_cast<T *>(p.y) + pix * p.K + k0;
+                auto store = [&](auto act) {
 #pragma unroll
-                for (int j = 0; j < CW / 8; ++j) {
-                    if (!valid || k0 + 8 * j >= p.K) break;
-                    const uint32_t rw[4] = {res[j].x, res[j].y, res[j].z, res[j].w};
-                    uint32_t o[4];
+                    for (int j = 0; j < CW / 8; ++j) {
+                        if (!valid || k0 + 8 * j >= p.K) break;
+                        const uint32_t rw[4] = {res[j].x, res[j].y, res[j].z, res[j].w};
+                        uint32_t o[4];
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const float2 r2 = unpack2<T>(rw[e]);
-                        const int i = 8 * j + 2 * e;
-                        o[e] = pack2<T>(act_apply(sum[i] + acc[i] + r2.x, p.act), act_apply(sum[i + 1] + acc[i + 1] + r2.y, p.act));
+                        for (int e = 0; e < 4; ++e) {
+                            const float2 r2 = unpack2<T>(rw[e]);
+                            const int i = 8 * j + 2 * e;
+                            o[e] = pack2<T>(act(sum[i] + bias[i] + r2.x), act(sum[i + 1] + bias[i + 1] + r2.y));
+                        }
+                        *reinterpret_cast<uint4 *>(y + 8 * j) = make_uint4(o[0], o[1], o[2], o[3]);
                     }
-                    *reinterpret_cast<uint4 *>(y + 8 * j) = make_uint4(o[0], o[1], o[2], o[3]);
-                }
+                };
+                if (p.act == SN_ACT_RELU || p.act == SN_ACT_RELU6)
+                    store([hi = p.act == SN_ACT_RELU ? INFINITY : 6.0f](float x) { return fminf(fmaxf(x, 0.0f), hi); });
+                else if (p.act == SN_ACT_NONE)
+                    store([](float x) { return x; });
+                else
+                    store([act = p.act](float x) { return act_apply(x, act); });
             }
         }
     }
@@ -374,8 +381,10 @@ __global__ void __launch_bounds__(LAT_THREADS, 2)
         tc_fence_after();
         tmem_dealloc<1>(tmem, BN);
     }
-    // no CTA leaves while a peer may still write into its shared memory
-    if (NCL > 1) cluster_sync_all();
+    // no CTA leaves while a peer may still write into its shared memory (relaxed:
+    // nothing read after it depends on it; a releasing arrive would wait for
+    // this CTA's global stores to be performed, ~1800 cycles)
+    if (NCL > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
 }
 
 template <typename T, int BN, int NCL>
