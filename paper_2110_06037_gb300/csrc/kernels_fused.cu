@@ -27,7 +27,6 @@ namespace fused {
 
 using namespace tc;
 
-constexpr int FUSED_THREADS = 256;
 constexpr int MAX_MT = 4;
 
 struct FParams {
@@ -41,9 +40,10 @@ struct FParams {
     long long wait_limit;
 };
 
-// T: storage type; KS: 3 or 5; SW: stride
-template <typename T, int KS, int SW>
-__global__ void __launch_bounds__(FUSED_THREADS, 2)
+// T: storage type; KS: 3 or 5; SW: stride; NT: threads (512 while a CTA has an SM
+// to itself, where the depthwise part is a latency)
+template <typename T, int KS, int SW, int NT>
+__global__ void __launch_bounds__(NT, 512 / NT)
     expand_dw_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUtensorMap mB,
                      const __grid_constant__ FParams p, int MT, uint32_t tmem_cols) {
     constexpr int QB = 4;  // output columns per thread
@@ -53,6 +53,7 @@ __global__ void __launch_bounds__(FUSED_THREADS, 2)
     __shared__ __align__(8) uint64_t full_bar[MAX_MT];
     __shared__ __align__(8) uint64_t accf_bar[MAX_MT];
     __shared__ uint4 dww[KS * KS * 8];
+    __shared__ __align__(16) float be_sh[64], bd_sh[64];
     __shared__ uint32_t tmem_sh;
     __shared__ volatile int abort_sh;
     __shared__ int issued_sh, done_sh;
@@ -82,10 +83,14 @@ __global__ void __launch_bounds__(FUSED_THREADS, 2)
         fence_mbar_init();
     }
     // the depthwise weights of the slice (like all weights, not written by the previous kernel)
-    for (int i = threadIdx.x; i < KS * KS * 8; i += FUSED_THREADS) {
+    for (int i = threadIdx.x; i < KS * KS * 8; i += NT) {
         const int c = e0 + (i & 7) * 8;
         dww[i] = c < p.E ? __ldg(reinterpret_cast<const uint4 *>(static_cast<const T *>(p.wd) + (int64_t)(i >> 3) * p.E + c))
                          : make_uint4(0u, 0u, 0u, 0u);
+    }
+    if (threadIdx.x < 64) {  // (zero-padded to 256 channels)
+        be_sh[threadIdx.x] = __ldg(p.be + e0 + threadIdx.x);
+        bd_sh[threadIdx.x] = __ldg(p.bd + e0 + threadIdx.x);
     }
     if (warp == 0) tmem_alloc<1>(&tmem_sh, tmem_cols);
     tc_fence_before();
@@ -131,10 +136,11 @@ __global__ void __launch_bounds__(FUSED_THREADS, 2)
         done_sh = mt;
     }
     __syncwarp();
-    // expanded values: warp w drains lanes 32 (w % 4) .., columns 32 (w / 4) ..
-    const int g4 = warp & 3, half = warp >> 2;
+    // expanded values: warp w drains lanes 32 (w % 4) .., columns 32 (w / 4 % 2)
+    // .. of every tile (256 threads) or every other one
+    const int g4 = warp & 3, half = (warp >> 2) & 1;
     auto mid = [&](int i) { return smem + (i >> 7) * tile_bytes + (i & 127) * 128; };  // pixel i's 128 bytes
-    for (int mt = 0; mt < mtn; ++mt) {
+    for (int mt = warp >> 3; mt < mtn; mt += NT / 256) {
         const bool ok = mbar_wait(&accf_bar[mt], 0u, p.wait_limit);
         if (!__all_sync(0xffffffffu, ok)) {
             if (lane == 0) atomicOr(p.err, ERR_ACC_WAIT);
@@ -150,8 +156,8 @@ __global__ void __launch_bounds__(FUSED_THREADS, 2)
         auto put = [&](auto act) {
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-                const float4 b0 = __ldg(reinterpret_cast<const float4 *>(p.be + e0 + half * 32 + 8 * j)),
-                             b1 = __ldg(reinterpret_cast<const float4 *>(p.be + e0 + half * 32 + 8 * j) + 1);
+                const float4 b0 = *reinterpret_cast<const float4 *>(be_sh + half * 32 + 8 * j),
+                             b1 = *reinterpret_cast<const float4 *>(be_sh + half * 32 + 8 * j + 4);
                 const float b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
                 uint32_t o[4];
 #pragma unroll
@@ -174,11 +180,11 @@ __global__ void __launch_bounds__(FUSED_THREADS, 2)
     // depthwise: QB columns x 8 channels per item, as the window kernel does it
     const int qblk = (int)p.fd_qb.d;
     const int items = abort_sh ? 0 : (p1 - p0) * qblk * 8;
-    for (int it = threadIdx.x; it < items; it += FUSED_THREADS) {
+    for (int it = threadIdx.x; it < items; it += NT) {
         const int v = it & 7, pr = (int)fdiv((uint32_t)(it >> 3), p.fd_qb), q0 = ((it >> 3) - pr * qblk) * QB;
         const int c0 = e0 + v * 8;
         if (c0 >= p.E) continue;
-        const float4 b0 = __ldg(reinterpret_cast<const float4 *>(p.bd + c0)), b1 = __ldg(reinterpret_cast<const float4 *>(p.bd + c0) + 1);
+        const float4 b0 = *reinterpret_cast<const float4 *>(bd_sh + v * 8), b1 = *reinterpret_cast<const float4 *>(bd_sh + v * 8 + 4);
         const float b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
         constexpr int WN = (QB - 1) * SW + KS;
         const int pout = p0 + pr, wbase = q0 * SW - p.pw;
@@ -351,18 +357,25 @@ cudaError_t expand_dw(const LaunchArgs &a, const LaunchArgs &b, const ExpandDwPl
     const size_t smem = smem_of(pl.MT, p.cblocks);
     const uint32_t cols = pl.MT == 1 ? 64u : pl.MT == 2 ? 128u : 256u;
     const dim3 grid((unsigned)((p.E + 63) / 64), (unsigned)pl.bands, (unsigned)in.n);
+    const bool big = (int64_t)grid.x * grid.y * grid.z > num_sms();  // two CTAs share an SM
     auto go = [&](auto kern) -> cudaError_t {
         const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        return launch_pdl(kern, grid, dim3(FUSED_THREADS), smem, a.stream, mA, mB, p, (int)pl.MT, cols);
+        return launch_pdl(kern, grid, dim3(big ? 256u : 512u), smem, a.stream, mA, mB, p, (int)pl.MT, cols);
     };
     const int ks = dw.conv.kh, sw = dw.conv.sw;
-    if (dt == SN_F16) {
-        if (ks == 3) return sw == 1 ? go(expand_dw_kernel<__half, 3, 1>) : go(expand_dw_kernel<__half, 3, 2>);
-        return sw == 1 ? go(expand_dw_kernel<__half, 5, 1>) : go(expand_dw_kernel<__half, 5, 2>);
-    }
-    if (ks == 3) return sw == 1 ? go(expand_dw_kernel<__nv_bfloat16, 3, 1>) : go(expand_dw_kernel<__nv_bfloat16, 3, 2>);
-    return sw == 1 ? go(expand_dw_kernel<__nv_bfloat16, 5, 1>) : go(expand_dw_kernel<__nv_bfloat16, 5, 2>);
+#define SN_EXPAND_DW(T, KS, SW) return big ? go(expand_dw_kernel<T, KS, SW, 256>) : go(expand_dw_kernel<T, KS, SW, 512>)
+#define SN_EXPAND_DW_T(T)                      \
+    do {                                       \
+        if (ks == 3 && sw == 1) SN_EXPAND_DW(T, 3, 1); \
+        if (ks == 3) SN_EXPAND_DW(T, 3, 2);    \
+        if (sw == 1) SN_EXPAND_DW(T, 5, 1);    \
+        SN_EXPAND_DW(T, 5, 2);                 \
+    } while (0)
+    if (dt == SN_F16) SN_EXPAND_DW_T(__half);
+    SN_EXPAND_DW_T(__nv_bfloat16);
+#undef SN_EXPAND_DW_T
+#undef SN_EXPAND_DW
 }
 
 }  // namespace k
