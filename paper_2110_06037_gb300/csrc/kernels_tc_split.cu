@@ -24,10 +24,12 @@
 // output pixels x BN channels.  A stage holds one 64-channel block of one tap:
 // all planes of A as one TMA box and all planes of B as another (a box costs
 // about the same whatever its size), so the six products of a stage read three
-// + three staged blocks.  Warp 0 issues the copies, warp 1 the MMAs, warps 2-9
-// drain: TMEM -> registers, and after a tile's last chunk through a swizzled
-// staging block to rows of 32 channels (bias, residual, activation or
-// requantisation, 128-byte coalesced global accesses).
+// + three staged blocks.  Warp 0 issues the copies (the first stages' weights
+// before the dependency wait), warp 1 the MMAs, warps 2-9 drain: TMEM ->
+// registers, and after a tile's last chunk bias, residual, activation or
+// requantisation and 16-byte stores of a thread's own row (32 or 64 consecutive
+// channels).  No staging: its 32 KB are a third fp32 stage, without which a
+// stage's copy was exposed once its MMAs were done.
 // What bounds it: 24 MMAs of K = 16 per stage and fp32 tile (six products),
 // i.e. a sixth of the bf16 rate, against the FFMA rate that the CUDA-core
 // routines stay below; small layers are bound by latency.  Every wait is
@@ -36,7 +38,6 @@
 
 #include <algorithm>
 #include <cstdio>
-#include <cstring>
 #include <string>
 #include <type_traits>
 #include <vector>
@@ -51,7 +52,6 @@ namespace tcs {
 using namespace tc;
 
 constexpr int SPLIT_THREADS = 320;  // producer, MMA issuer, eight epilogue warps
-constexpr uint32_t STAGE_OUT = 32 * 32 * 4;  // one warp's staging block: 32 rows x 32 values
 // K steps (64 values) per accumulator drain: 256 values bound the tensor
 // core's accumulation error in fp32; 1024 code products stay exact in qint8
 constexpr int chunk_of(int planes) { return planes == 3 ? 4 : 16; }
@@ -68,7 +68,7 @@ struct SParams {
     const void *res;
     int *err;
     long long wait_limit;
-    int32_t act, vec;                        // vec: four output values per access (K and the bases allow it)
+    int32_t act, vec;                        // vec: output (and residual) accesses of 16 bytes (2), four elements (1), one (0)
     const float *x32, *w32;                  // fp32: the operands themselves (x NHWC, w [K][R*S][C])
     const float *ws;                         // qint8: weight scales
     float s_x, s_r, inv_out;
@@ -99,14 +99,12 @@ template <int PLANES, int BN>
 struct Lay {
     static constexpr uint32_t A_PL = BM * BK * 2, B_PL = BN * BK * 2;
     static constexpr uint32_t A_BYTES = PLANES * A_PL, STAGE = A_BYTES + PLANES * B_PL;
-    static constexpr int STAGES = (227 * 1024 - 2048 - EPI_WARPS * (int)STAGE_OUT) / (int)STAGE < 6
-                                      ? (227 * 1024 - 2048 - EPI_WARPS * (int)STAGE_OUT) / (int)STAGE
-                                      : 6;
+    static constexpr int STAGES = (226 * 1024 - 2048) / (int)STAGE < 8 ? (226 * 1024 - 2048) / (int)STAGE : 8;
     static constexpr bool STACK = PLANES == 3 && BN == 64;          // planes of B as rows of one operand
     static constexpr int ACC = PLANES == 1 ? 1 : STACK ? 3 : 2;     // accumulators per buffer
     static constexpr int BUF = STACK ? 256 : ACC * BN;              // TMEM columns from one buffer to the other
     static constexpr uint32_t COLS = 2 * BUF;
-    static constexpr size_t SMEM = (size_t)STAGES * STAGE + EPI_WARPS * STAGE_OUT + 1024;
+    static constexpr size_t SMEM = (size_t)STAGES * STAGE + 1024;
     static_assert(STAGES >= 2 && COLS <= 512, "stage ring and TMEM");
 };
 
@@ -131,10 +129,14 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1)
 
     griddep_launch();
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    uint8_t *stg = smem + STAGES * L::STAGE;
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     const int total = p.mtiles * p.ntiles;
     const int nchunks = (p.kiters + CH - 1) / CH;
+    if (threadIdx.x == 32) {  // the maps are kernel parameters, not data of the previous kernel
+        const CUtensorMap *maps[5] = {&mB, &mA0, &mA1, &mA2, &mA3};
+        for (int i = 0; i < (p.stride == 1 ? 2 : 5); ++i)
+            asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(maps[i])) : "memory");
+    }
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) {
             mbar_init(&full_bar[s], 1);
@@ -167,6 +169,20 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1)
             int g = 0, s = 0;
             uint32_t par = 0;
             bool stop = false;
+            // the weights of the first stages: not written by the previous kernel
+            const int early = (int)blockIdx.x < total ? min(STAGES, p.kiters) : 0;
+            {
+                int n0, q0, p0, i0, tap = 0, cb = 0;
+                tile((int)blockIdx.x, n0, q0, p0, i0);
+                for (int i = 0; i < early; ++i) {
+                    mbar_expect_tx(&full_bar[i], L::STAGE);
+                    tma_4d<1>(su32(smem + i * L::STAGE) + L::A_BYTES, &mB, su32(&full_bar[i]), cb * BK, tap, n0, 0);
+                    if (++cb == p.cblocks) {
+                        cb = 0;
+                        ++tap;
+                    }
+                }
+            }
             griddep_wait();
             for (int t = blockIdx.x; t < total && !stop; t += gridDim.x) {
                 int n0, q0, p0, i0;
@@ -177,12 +193,13 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1)
                         atomicOr(p.err, ERR_TMA_WAIT);
                         abort_sh = 1;
                     }
-                    if (abort_sh) {
+                    // (a stage whose weights are on their way gets its activations whatever happened)
+                    if (abort_sh && g >= early) {
                         stop = true;
                         break;
                     }
                     const uint32_t sa = su32(smem + s * L::STAGE), bar = su32(&full_bar[s]);
-                    mbar_expect_tx(&full_bar[s], L::STAGE);
+                    if (g >= early) mbar_expect_tx(&full_bar[s], L::STAGE);
                     const int oh = r * p.dh - p.gph, ow = ss * p.dw - p.gpw;
                     const CUtensorMap *m = &mA0;
                     int qa = q0 + ow, pa = p0 + oh;
@@ -193,7 +210,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1)
                         pa = p0 + ((oh - bh) >> 1);
                     }
                     tma_5d<1>(sa, m, bar, cb * BK, qa, pa, i0, 0);
-                    tma_4d<1>(sa + L::A_BYTES, &mB, bar, cb * BK, tap, n0, 0);
+                    if (g >= early) tma_4d<1>(sa + L::A_BYTES, &mB, bar, cb * BK, tap, n0, 0);
                     issued_sh = g + 1;
                     if (++s == STAGES) {
                         s = 0;
@@ -225,15 +242,16 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1)
                     if (first && !mbar_wait(&acce_bar[b], ((uint32_t)(u >> 1) & 1u) ^ 1u, p.wait_limit)) {
                         atomicOr(p.err, ERR_EPI_WAIT);
                         abort_sh = 1;
+                        stop = true;
                     }
-                    if (!abort_sh && !mbar_wait(&full_bar[s], par, p.wait_limit)) {
+                    // (no look at abort_sh: a shared-memory access of this thread
+                    // queues behind the MMAs' operand reads, ~200 cycles)
+                    if (!stop && !mbar_wait(&full_bar[s], par, p.wait_limit)) {
                         atomicOr(p.err, ERR_MMA_WAIT);
                         abort_sh = 1;
-                    }
-                    if (abort_sh) {
                         stop = true;
-                        break;
                     }
+                    if (stop) break;
                     tc_fence_after();
                     const uint32_t d = tmem + (uint32_t)(b * L::BUF);
                     const uint64_t da = desc0 + (uint64_t)((s * L::STAGE) >> 4), db = da + (L::A_BYTES >> 4);
@@ -241,10 +259,16 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1)
                     const int ks = min(BK / 16, (p.Cp - cb * BK + 15) / 16);
                     if constexpr (L::STACK) {
                         const uint32_t id3 = idesc_f16<__nv_bfloat16>(BM, 3 * BN), id2 = idesc_f16<__nv_bfloat16>(BM, 2 * BN);
-                        for (int k = 0; k < ks; ++k) {
+                        auto step = [&](int k) {
                             umma<1>(d, da + 2 * k, db + 2 * k, id3, (!first || k > 0) ? 1u : 0u);
                             umma<1>(d + BN, da + (L::A_PL >> 4) + 2 * k, db + 2 * k, id2, 1u);
                             umma<1>(d + 2 * BN, da + 2 * (L::A_PL >> 4) + 2 * k, db + 2 * k, idesc, 1u);
+                        };
+                        if (ks == BK / 16) {
+#pragma unroll
+                            for (int k = 0; k < BK / 16; ++k) step(k);
+                        } else {
+                            for (int k = 0; k < ks; ++k) step(k);
                         }
                     } else if constexpr (F32) {
                         // small products first within the block; each accumulator sums in its own order
@@ -255,6 +279,9 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1)
                                 umma<1>(e == 5 ? d : d + BN, da + I[e] * (L::A_PL >> 4) + 2 * k,
                                         db + J[e] * (L::B_PL >> 4) + 2 * k, idesc,
                                         (!first || k > 0 || (e > 0 && e < 5)) ? 1u : 0u);
+                    } else if (ks == BK / 16) {
+#pragma unroll
+                        for (int k = 0; k < BK / 16; ++k) umma<1>(d, da + 2 * k, db + 2 * k, idesc, (!first || k > 0) ? 1u : 0u);
                     } else {
                         for (int k = 0; k < ks; ++k) umma<1>(d, da + 2 * k, db + 2 * k, idesc, (!first || k > 0) ? 1u : 0u);
                     }
@@ -275,13 +302,22 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1)
     } else {  // ---------------- epilogue: warps 2..9
         constexpr int HC = BN / 2;  // columns of this warp: half of the tile's
         const int half = (warp - 2) >> 2, g4 = warp & 3;
-        uint8_t *buf = stg + (warp - 2) * STAGE_OUT;
+        const int tr = g4 * 32 + lane;  // this thread's row of the tile
         int u = 0;
         bool stop = false;
         griddep_wait();
         for (int t = blockIdx.x; t < total && !stop; t += gridDim.x) {
             int n0, q0, p0, i0;
             tile(t, n0, q0, p0, i0);
+            const int q = q0 + (tr & (p.BW - 1)), pp = p0 + ((tr >> p.lbw) & (p.BH - 1)), n = i0 + (tr >> p.lbwh);
+            const bool live = q < p.gQ && pp < p.gP && n < p.gN;
+            const int64_t pix = live ? ((int64_t)n * p.gP + pp) * p.gQ + q : 0;
+            // rows are handled by pairs of lanes when they are stored
+            const bool live2 = __shfl_xor_sync(0xffffffffu, (int)live, 1);
+            const int64_t pix2 = __shfl_xor_sync(0xffffffffu, (long long)pix, 1);
+            if (F32 && p.res && live)  // its residual, on its way into L1 while the tile is accumulated
+                for (int e = 0; e < HC && n0 + half * HC + e < p.K; e += 32)
+                    asm volatile("prefetch.global.L1 [%0];" ::"l"(static_cast<const float *>(p.res) + pix * p.K + n0 + half * HC + e));
             Acc acc[HC];
 #pragma unroll
             for (int e = 0; e < HC; ++e) acc[e] = 0;
@@ -295,6 +331,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1)
                     break;
                 }
                 tc_fence_after();
+                __syncwarp();
                 const uint32_t ta = tmem + ((uint32_t)(g4 * 32) << 16) + (uint32_t)(b * L::BUF + half * HC);
 #pragma unroll
                 for (int j = 0; j < HC; j += 32) {
@@ -322,76 +359,115 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1)
                 if (lane == 0) mbar_arrive(&acce_bar[b]);
             }
             if (stop) break;
+            using TR = typename std::conditional<F32, float, int8_t>::type;  // residual element
+            constexpr int G = 16;                                             // channels at a time
+            // one 16-byte piece, four elements or one element at a time, as K and the bases allow
+            auto group = [&](auto jc, auto epv) {
+                constexpr int j = decltype(jc)::value;
+                constexpr int EV = decltype(epv)::value;
+                const int k = n0 + half * HC + j;
+                const int64_t o0 = pix * p.K + k;
+                float rv[G];
 #pragma unroll
-            for (int j = 0; j < HC; j += 32) {
-                const int kb = n0 + half * HC + j;
-                if (kb >= p.K) break;
-                // 16-byte piece i of row `lane` at piece i ^ (lane & 7)
-                __syncwarp();
+                for (int e = 0; e < G; ++e) rv[e] = 0.f;
+                if (p.res && live) {
+                    constexpr int ER = EV == 1 ? 1 : EV == 4 ? 4 : 16 / (int)sizeof(TR);
+                    const TR *res = static_cast<const TR *>(p.res) + o0;
 #pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const Acc *a4 = acc + j + 4 * i;
-                    uint4 o;
-                    memcpy(&o.x, a4, 4), memcpy(&o.y, a4 + 1, 4), memcpy(&o.z, a4 + 2, 4), memcpy(&o.w, a4 + 3, 4);
-                    *reinterpret_cast<uint4 *>(buf + lane * 128 + ((i ^ (lane & 7)) << 4)) = o;
-                }
-                __syncwarp();
-                const int piece = lane & 7, k = kb + piece * 4;
-                const int nk = min(4, p.K - k);  // channels of this lane's piece (<= 0: none)
-                const bool vec = p.vec;
-                float bs[4], sw[4];
+                    for (int e = 0; e < G; e += ER) {
+                        if (k + e >= p.K) break;
+                        const Vec<TR, ER> r = *reinterpret_cast<const Vec<TR, ER> *>(res + e);
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    bs[e] = e < nk ? __ldg(p.bias + k + e) : 0.f;
-                    sw[e] = !F32 && e < nk ? __ldg(p.ws + k + e) : 0.f;
-                }
-                for (int it = 0; it < 8; ++it) {
-                    const int row = it * 4 + (lane >> 3), tr = g4 * 32 + row;
-                    const int q = q0 + (tr & (p.BW - 1)), pp = p0 + ((tr >> p.lbw) & (p.BH - 1)), n = i0 + (tr >> p.lbwh);
-                    if (nk <= 0 || q >= p.gQ || pp >= p.gP || n >= p.gN) continue;
-                    const int64_t pix = ((int64_t)n * p.gP + pp) * p.gQ + q, o0 = pix * p.K + k;
-                    const uint4 a4 = *reinterpret_cast<const uint4 *>(buf + row * 128 + ((piece ^ (row & 7)) << 4));
-                    if constexpr (F32) {
-                        float v[4] = {__uint_as_float(a4.x), __uint_as_float(a4.y), __uint_as_float(a4.z),
-                                      __uint_as_float(a4.w)};
-                        float rv[4] = {0.f, 0.f, 0.f, 0.f};
-                        const float *res = static_cast<const float *>(p.res);
-                        if (res) {
-                            if (vec) {
-                                const float4 r4 = *reinterpret_cast<const float4 *>(res + o0);
-                                rv[0] = r4.x, rv[1] = r4.y, rv[2] = r4.z, rv[3] = r4.w;
-                            } else {
-                                for (int e = 0; e < nk; ++e) rv[e] = res[o0 + e];
-                            }
-                        }
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            if (e < nk && !isfinite(v[e])) v[e] = plain_sum(p, pix, k + e);
-                            v[e] = act_apply(v[e] + bs[e] + rv[e], p.act);
-                        }
-                        float *yo = static_cast<float *>(p.y) + o0;
-                        if (vec) {
-                            *reinterpret_cast<float4 *>(yo) = make_float4(v[0], v[1], v[2], v[3]);
-                        } else {
-                            for (int e = 0; e < nk; ++e) yo[e] = v[e];
-                        }
-                    } else {
-                        const int v[4] = {(int)a4.x, (int)a4.y, (int)a4.z, (int)a4.w};
-                        const int8_t *res = static_cast<const int8_t *>(p.res);
-                        TO *yo = static_cast<TO *>(p.y) + o0;
-                        Vec<TO, 4> o;
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            const float r = res && e < nk ? __fmul_rn((float)res[o0 + e], p.s_r) : 0.0f;
-                            o.v[e] = q8_out<TO>(q8_value(v[e], p.s_x, sw[e], bs[e], r, p.act), p.inv_out);
-                        }
-                        if (vec) {
-                            *reinterpret_cast<Vec<TO, 4> *>(yo) = o;
-                        } else {
-                            for (int e = 0; e < nk; ++e) yo[e] = o.v[e];
-                        }
+                        for (int i = 0; i < ER; ++i) rv[e + i] = F32 ? (float)r.v[i] : __fmul_rn((float)r.v[i], p.s_r);
                     }
                 }
+                float bv[G];
+                [[maybe_unused]] float sv[G];
+#pragma unroll
+                for (int e = 0; e < G; e += 4) {  // (the bias is zero-padded to a multiple of 256 channels)
+                    const float4 b4 = __ldg(reinterpret_cast<const float4 *>(p.bias + k + e));
+                    bv[e] = b4.x, bv[e + 1] = b4.y, bv[e + 2] = b4.z, bv[e + 3] = b4.w;
+                    if constexpr (!F32) {  // (qint8: K is a multiple of four)
+                        const float4 s4 = k + e < p.K ? __ldg(reinterpret_cast<const float4 *>(p.ws + k + e)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                        sv[e] = s4.x, sv[e + 1] = s4.y, sv[e + 2] = s4.z, sv[e + 3] = s4.w;
+                    }
+                }
+                TO o[G];
+                if constexpr (F32) {
+                    // one test for the group: an infinity or a NaN has all exponent bits
+                    bool odd_value = false;
+#pragma unroll
+                    for (int e = 0; e < G; ++e) odd_value |= (__float_as_uint(acc[j + e]) & 0x7f800000u) == 0x7f800000u;
+                    if (odd_value && live) {
+#pragma unroll
+                        for (int e = 0; e < G; ++e)
+                            if (k + e < p.K && !isfinite(acc[j + e])) acc[j + e] = plain_sum(p, pix, k + e);
+                    }
+                }
+                auto finish = [&](auto act) {
+#pragma unroll
+                    for (int e = 0; e < G; ++e) {
+                        if constexpr (F32) o[e] = act(acc[j + e] + bv[e] + rv[e]);
+                        else o[e] = q8_out<TO>(act(__fadd_rn(__fadd_rn(__fmul_rn(__int2float_rn(acc[j + e]), __fmul_rn(p.s_x, sv[e])), bv[e]), rv[e])), p.inv_out);
+                    }
+                };
+                if (p.act == SN_ACT_RELU || p.act == SN_ACT_RELU6)
+                    finish([hi = p.act == SN_ACT_RELU ? INFINITY : 6.0f](float x) { return fminf(fmaxf(x, 0.0f), hi); });
+                else if (p.act == SN_ACT_NONE)
+                    finish([](float x) { return x; });
+                else
+                    finish([act = p.act](float x) {
+                        if constexpr (F32) return act_apply(x, act);
+                        else return q8_act(x, act);
+                    });
+                if constexpr (F32 && EV == 16) {
+                    // 32 contiguous bytes of a row per pair of lanes: the even lane
+                    // stores the first half of its own row, then of its neighbour's,
+                    // the odd lane the second halves (16-byte stores of 32 different
+                    // rows fill half a sector each)
+                    const bool odd = lane & 1;
+                    float *ya = static_cast<float *>(p.y) + (odd ? pix2 : pix) * p.K + k;   // the pair's even row
+                    float *yb = static_cast<float *>(p.y) + (odd ? pix : pix2) * p.K + k;   // its odd row
+                    const bool la = odd ? live2 : live, lb = odd ? live : live2;
+#pragma unroll
+                    for (int e = 0; e < G; e += 8) {
+                        float got[4];
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) got[i] = __shfl_xor_sync(0xffffffffu, odd ? o[e + i] : o[e + 4 + i], 1);
+                        const int at = e + (odd ? 4 : 0);
+                        if (k + at >= p.K) continue;
+                        const float4 a = odd ? make_float4(got[0], got[1], got[2], got[3])
+                                             : make_float4(o[e], o[e + 1], o[e + 2], o[e + 3]);
+                        const float4 b = odd ? make_float4(o[e + 4], o[e + 5], o[e + 6], o[e + 7])
+                                             : make_float4(got[0], got[1], got[2], got[3]);
+                        if (la) *reinterpret_cast<float4 *>(ya + at) = a;
+                        if (lb) *reinterpret_cast<float4 *>(yb + at) = b;
+                    }
+                    return;
+                }
+                if (!live) return;
+                TO *yo = static_cast<TO *>(p.y) + o0;
+                constexpr int EO = EV == 1 ? 1 : EV == 4 ? 4 : 16 / (int)sizeof(TO);
+#pragma unroll
+                for (int e = 0; e < G; e += EO) {
+                    if (k + e >= p.K) break;
+                    Vec<TO, EO> w;
+#pragma unroll
+                    for (int i = 0; i < EO; ++i) w.v[i] = o[e + i];
+                    *reinterpret_cast<Vec<TO, EO> *>(yo + e) = w;
+                }
+            };
+            auto groups = [&](auto jc) {
+                if (n0 + half * HC + decltype(jc)::value >= p.K) return;
+                if (p.vec == 2) group(jc, std::integral_constant<int, 16>{});
+                else if (p.vec == 1) group(jc, std::integral_constant<int, 4>{});
+                else group(jc, std::integral_constant<int, 1>{});
+            };
+            groups(std::integral_constant<int, 0>{});
+            groups(std::integral_constant<int, 16>{});
+            if constexpr (HC == 64) {
+                groups(std::integral_constant<int, 32>{});
+                groups(std::integral_constant<int, 48>{});
             }
         }
     }
@@ -621,7 +697,14 @@ cudaError_t conv_split(const LaunchArgs &a, int32_t v) {
     p.res = a.in[1];
     p.err = device_error_word();
     p.wait_limit = a.wait_limit > 0 ? a.wait_limit : WAIT_LIMIT;
-    p.vec = p.K % 4 == 0 && (uintptr_t)a.out % (4 * dtype_size(out_dt)) == 0 && (!f32 || (uintptr_t)p.res % 16 == 0);
+    {
+        const int eo = dtype_size(out_dt), er = f32 ? 4 : 1;
+        auto fits = [&](int bo, int br) {  // K and the bases admit pieces of bo and br bytes
+            return p.K % (bo / eo) == 0 && (uintptr_t)a.out % bo == 0 &&
+                   (!p.res || (p.K % (br / er) == 0 && (uintptr_t)p.res % br == 0));
+        };
+        p.vec = fits(16, 16) ? 2 : fits(4 * eo, 4 * er) ? 1 : 0;
+    }
     const int64_t pixels = in.n * in.h * in.w, plane = pixels * p.Cp;
     auto *xs = static_cast<__nv_bfloat16 *>(a.ws);
     // the planes of the activations
