@@ -153,27 +153,14 @@ __global__ void __launch_bounds__(NT, 512 / NT)
         tmem_ld32(tmem + ((uint32_t)(g4 * 32) << 16) + (uint32_t)(mt * 64 + half * 32), v);
         const int i = g4 * 32 + lane;
         uint8_t *row = mid(mt * BM + i);
-        auto put = [&](auto act) {
+        with_act2<T>(p.act_e, [&](auto fin) {
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-                const float4 b0 = *reinterpret_cast<const float4 *>(be_sh + half * 32 + 8 * j),
-                             b1 = *reinterpret_cast<const float4 *>(be_sh + half * 32 + 8 * j + 4);
-                const float b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-                uint32_t o[4];
-#pragma unroll
-                for (int e = 0; e < 4; ++e)
-                    // (+ 0: where a residual would join; it turns -0 into +0 there too)
-                    o[e] = pack2<T>(act(__uint_as_float(v[8 * j + 2 * e]) + b[2 * e] + 0.0f),
-                                    act(__uint_as_float(v[8 * j + 2 * e + 1]) + b[2 * e + 1] + 0.0f));
-                *reinterpret_cast<uint4 *>(row + (((half * 4 + j) ^ (i & 7)) << 4)) = make_uint4(o[0], o[1], o[2], o[3]);
+                const float4 *b4 = reinterpret_cast<const float4 *>(be_sh + half * 32 + 8 * j);
+                *reinterpret_cast<uint4 *>(row + (((half * 4 + j) ^ (i & 7)) << 4)) =
+                    finish8<T>(v + 8 * j, b4[0], b4[1], false, make_uint4(0u, 0u, 0u, 0u), fin);
             }
-        };
-        if (p.act_e == SN_ACT_RELU || p.act_e == SN_ACT_RELU6)
-            put([hi = p.act_e == SN_ACT_RELU ? INFINITY : 6.0f](float x) { return fminf(fmaxf(x, 0.0f), hi); });
-        else if (p.act_e == SN_ACT_NONE)
-            put([](float x) { return x; });
-        else
-            put([act = p.act_e](float x) { return act_apply(x, act); });
+        });
     }
     tc_fence_before();
     __syncthreads();

@@ -212,7 +212,7 @@ __global__ void __launch_bounds__(LAT_THREADS, 2)
         } else {
             tc_fence_after();
             const uint32_t ta = tmem + ((uint32_t)(warp * 32) << 16);
-            auto drain = [&](auto act) {
+            with_act2<T>(p.act, [&](auto fin) {
 #pragma unroll
                 for (int c = 0; c < BN / 32; ++c) {
                     const int k0 = w.n0 + 32 * c;
@@ -222,20 +222,10 @@ __global__ void __launch_bounds__(LAT_THREADS, 2)
                     tmem_ld32(ta + 32 * c, v);
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
-                        const float4 b0 = *reinterpret_cast<const float4 *>(bias_sh + 32 * c + 8 * j),
-                                     b1 = *reinterpret_cast<const float4 *>(bias_sh + 32 * c + 8 * j + 4);
-                        const float b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-                        const uint32_t rw[4] = {rq[j].x, rq[j].y, rq[j].z, rq[j].w};
-                        uint32_t o[4];
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            const float2 r2 = unpack2<T>(rw[e]);
-                            o[e] = pack2<T>(act(__uint_as_float(v[8 * j + 2 * e]) + b[2 * e] + r2.x),
-                                            act(__uint_as_float(v[8 * j + 2 * e + 1]) + b[2 * e + 1] + r2.y));
-                        }
+                        const float4 *b4 = reinterpret_cast<const float4 *>(bias_sh + 32 * c + 8 * j);
                         const int piece = (c & 1) * 4 + j;
                         *reinterpret_cast<uint4 *>(buf + lane * 128 + ((piece ^ (lane & 7)) << 4)) =
-                            make_uint4(o[0], o[1], o[2], o[3]);
+                            finish8<T>(v + 8 * j, b4[0], b4[1], p.res != nullptr, rq[j], fin);
                     }
                     if (c + 1 < BN / 32) load_res(k0 + 32);
                     if ((c & 1) || k0 + 32 >= p.K) {  // the 64-channel block is complete
@@ -250,13 +240,7 @@ __global__ void __launch_bounds__(LAT_THREADS, 2)
                         __syncwarp();
                     }
                 }
-            };
-            if (p.act == SN_ACT_RELU || p.act == SN_ACT_RELU6)
-                drain([hi = p.act == SN_ACT_RELU ? INFINITY : 6.0f](float x) { return fminf(fmaxf(x, 0.0f), hi); });
-            else if (p.act == SN_ACT_NONE)
-                drain([](float x) { return x; });
-            else
-                drain([act = p.act](float x) { return act_apply(x, act); });
+            });
             if (lane == 0) bulk_wait_read_0();  // the stores have read the stage memory
             __syncwarp();
         }
@@ -335,27 +319,15 @@ __global__ void __launch_bounds__(LAT_THREADS, 2)
                         sum[4 * j] += x.x, sum[4 * j + 1] += x.y, sum[4 * j + 2] += x.z, sum[4 * j + 3] += x.w;
                     }
                 T *y = static_cast<T *>(p.y) + pix * p.K + k0;
-                auto store = [&](auto act) {
+                with_act2<T>(p.act, [&](auto fin) {
 #pragma unroll
                     for (int j = 0; j < CW / 8; ++j) {
                         if (!valid || k0 + 8 * j >= p.K) break;
-                        const uint32_t rw[4] = {res[j].x, res[j].y, res[j].z, res[j].w};
-                        uint32_t o[4];
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            const float2 r2 = unpack2<T>(rw[e]);
-                            const int i = 8 * j + 2 * e;
-                            o[e] = pack2<T>(act(sum[i] + bias[i] + r2.x), act(sum[i + 1] + bias[i + 1] + r2.y));
-                        }
-                        *reinterpret_cast<uint4 *>(y + 8 * j) = make_uint4(o[0], o[1], o[2], o[3]);
+                        const float4 *b4 = reinterpret_cast<const float4 *>(bias + 8 * j);
+                        *reinterpret_cast<uint4 *>(y + 8 * j) =
+                            finish8<T>(sum + 8 * j, b4[0], b4[1], p.res != nullptr, res[j], fin);
                     }
-                };
-                if (p.act == SN_ACT_RELU || p.act == SN_ACT_RELU6)
-                    store([hi = p.act == SN_ACT_RELU ? INFINITY : 6.0f](float x) { return fminf(fmaxf(x, 0.0f), hi); });
-                else if (p.act == SN_ACT_NONE)
-                    store([](float x) { return x; });
-                else
-                    store([act = p.act](float x) { return act_apply(x, act); });
+                });
             }
         }
     }

@@ -176,6 +176,9 @@ __device__ __forceinline__ void prefetch_l2(const void *p, uint32_t bytes) {
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(reinterpret_cast<uint64_t>(p)), "r"(bytes)
                  : "memory");
 }
+__device__ __forceinline__ void prefetch_l1(const void *p) {
+    asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
+}
 
 // TMEM allocation; G = 2 allocates the same columns in both CTAs of the pair
 // (one warp of each CTA executes it)
@@ -395,7 +398,70 @@ template <>
 __device__ __forceinline__ float2 unpack2<__nv_bfloat16>(uint32_t v) {
     return __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&v));
 }
-
+// two fp32 sums in one instruction, each rounded as a scalar add rounds it
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+    float2 d;
+    asm("{\n\t.reg .b64 x, y, z;\n\t"
+        "mov.b64 x, {%2, %3};\n\t"
+        "mov.b64 y, {%4, %5};\n\t"
+        "add.rn.f32x2 z, x, y;\n\t"
+        "mov.b64 {%0, %1}, z;\n\t}"
+        : "=f"(d.x), "=f"(d.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return d;
+}
+// The end of an epilogue: activation and rounding of a pair of sums, for
+// relu and relu6 with both clamps after the rounding, on the packed pair (0, 6
+// and infinity are values of both types and rounding keeps order, so the result
+// is that of clamping first; a NaN becomes 0 either way).  fp32 min and max issue
+// at half rate and take two instructions a value: clamping first, they were a
+// third of the epilogue's issue slots.
+template <typename T>
+__device__ __forceinline__ uint32_t clamp2(uint32_t v, float hi);
+template <>
+__device__ __forceinline__ uint32_t clamp2<__half>(uint32_t v, float hi) {
+    const __half2 r = __hmin2(__hmax2(*reinterpret_cast<const __half2 *>(&v), __float2half2_rn(0.0f)), __float2half2_rn(hi));
+    return *reinterpret_cast<const uint32_t *>(&r);
+}
+template <>
+__device__ __forceinline__ uint32_t clamp2<__nv_bfloat16>(uint32_t v, float hi) {
+    const __nv_bfloat162 r =
+        __hmin2(__hmax2(*reinterpret_cast<const __nv_bfloat162 *>(&v), __float2bfloat162_rn(0.0f)), __float2bfloat162_rn(hi));
+    return *reinterpret_cast<const uint32_t *>(&r);
+}
+// calls body(f) with f the function of the activation from a pair of sums to
+// the packed pair, so that an unrolled body carries one activation's code
+template <typename T, typename F>
+__device__ __forceinline__ void with_act2(int act, F body) {
+    if (act == SN_ACT_RELU || act == SN_ACT_RELU6)
+        body([hi = act == SN_ACT_RELU ? INFINITY : 6.0f](float2 f) { return clamp2<T>(pack2<T>(f.x, f.y), hi); });
+    else if (act == SN_ACT_NONE)
+        body([](float2 f) { return pack2<T>(f.x, f.y); });
+    else
+        body([act](float2 f) { return pack2<T>(act_apply(f.x, act), act_apply(f.y, act)); });
+}
+// eight channels' sums plus bias plus (with has_res) residual to a 16-byte piece
+template <typename T, typename F>
+__device__ __forceinline__ uint4 finish8(const float *v, float4 b0, float4 b1, bool has_res, uint4 res, F fin) {
+    float2 f[4] = {add2(make_float2(v[0], v[1]), make_float2(b0.x, b0.y)),
+                   add2(make_float2(v[2], v[3]), make_float2(b0.z, b0.w)),
+                   add2(make_float2(v[4], v[5]), make_float2(b1.x, b1.y)),
+                   add2(make_float2(v[6], v[7]), make_float2(b1.z, b1.w))};
+    if (has_res) {
+        f[0] = add2(f[0], unpack2<T>(res.x));
+        f[1] = add2(f[1], unpack2<T>(res.y));
+        f[2] = add2(f[2], unpack2<T>(res.z));
+        f[3] = add2(f[3], unpack2<T>(res.w));
+    }
+    return make_uint4(fin(f[0]), fin(f[1]), fin(f[2]), fin(f[3]));
+}
+template <typename T, typename F>
+__device__ __forceinline__ uint4 finish8(const uint32_t *u, float4 b0, float4 b1, bool has_res, uint4 res, F fin) {
+    float v[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(u[i]);
+    return finish8<T>(v, b0, b1, has_res, res, fin);
+}
 
 
 // named barrier `id` over `count` threads (whole warps) that also ORs a

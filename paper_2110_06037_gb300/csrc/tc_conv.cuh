@@ -553,17 +553,11 @@ __global__ void __launch_bounds__(THREADS, 1)
             const int b = lt & 1;
             const uint32_t aph = (uint32_t)(lt >> 1) & 1u;
             const Work w = unit(ui, (int)rank);
-            // bias of this warp's channels (lane j holds channel chunk + 32h + j;
-            // the buffer is zero-padded to a multiple of 256 channels), loaded
-            // before the accumulator wait so that the latency is hidden
-            float bias_r[CPH][2];
-#pragma unroll
-            for (int cj = 0; cj < CPH; ++cj)
-#pragma unroll
-                for (int h = 0; h < 2; ++h)
-                    bias_r[cj][h] = (p.ksplit == 1 && cbase + cj < NCH)
-                                        ? __ldg(p.bias + w.n0 + 64 * (cbase + cj) + 32 * h + lane)
-                                        : 0.f;
+            // bias of this warp's channels (the buffer is zero-padded to a multiple
+            // of 256 channels): its lines into L1 before the accumulator wait, so
+            // that the broadcast 16-byte loads below hit
+            const float4 *bias4 = reinterpret_cast<const float4 *>(p.bias + w.n0 + 64 * cbase);
+            if (p.ksplit == 1 && lane < 2 * CPH && cbase * 2 + lane < BN / 32) prefetch_l1(bias4 + 8 * lane);
             bool valid;
             int64_t pix;
             if (IMPLICIT) {
@@ -680,51 +674,20 @@ __global__ void __launch_bounds__(THREADS, 1)
                                 acc[4 * q + 3] += x.w;
                             }
                         }
-                        // this row's residual (the output's NHWC layout), 8 channels per piece
-                        uint32_t rv[2][16];
-#pragma unroll
-                        for (int h = 0; h < 2; ++h)
-#pragma unroll
-                            for (int q = 0; q < 16; ++q) rv[h][q] = 0u;
-                        if (p.res && valid) {
-                            const uint4 *rr = reinterpret_cast<const uint4 *>(static_cast<const T *>(p.res) + pix * p.K + k0);
-#pragma unroll
-                            for (int q = 0; q < 8; ++q)
-                                if (k0 + 8 * q < p.K) {
-                                    const uint4 u = rr[q];
-                                    rv[q >> 2][4 * (q & 3)] = u.x;
-                                    rv[q >> 2][4 * (q & 3) + 1] = u.y;
-                                    rv[q >> 2][4 * (q & 3) + 2] = u.z;
-                                    rv[q >> 2][4 * (q & 3) + 3] = u.w;
-                                }
-                        }
                         if (lane == 0) bulk_wait_read_0();  // the previous store has read the block
                         __syncwarp();
-                        auto finish_rows = [&](auto act) {
+                        // this row's residual (the output's NHWC layout), 8 channels per piece
+                        const uint4 *rr = reinterpret_cast<const uint4 *>(static_cast<const T *>(p.res) + pix * p.K + k0);
+                        const bool row_res = p.res && valid;
+                        with_act2<T>(p.act, [&](auto fin) {
 #pragma unroll
                             for (int q = 0; q < 8; ++q) {
-                                const int h = q >> 2;
-                                uint32_t wq[4];
-#pragma unroll
-                                for (int e = 0; e < 4; ++e) {
-                                    const int jp = 4 * (q & 3) + e;  // pair index within the half
-                                    const float2 r2 = unpack2<T>(rv[h][jp]);
-                                    const float f0 = act(acc[32 * h + 2 * jp] +
-                                                         __shfl_sync(0xffffffffu, bias_r[cj][h], 2 * jp) + r2.x);
-                                    const float f1 = act(acc[32 * h + 2 * jp + 1] +
-                                                         __shfl_sync(0xffffffffu, bias_r[cj][h], 2 * jp + 1) + r2.y);
-                                    wq[e] = pack2<T>(f0, f1);
-                                }
+                                const bool r = row_res && k0 + 8 * q < p.K;
                                 *reinterpret_cast<uint4 *>(buf + lane * 128 + ((q ^ (lane & 7)) << 4)) =
-                                    make_uint4(wq[0], wq[1], wq[2], wq[3]);
+                                    finish8<T>(acc + 8 * q, __ldg(bias4 + 16 * cj + 2 * q), __ldg(bias4 + 16 * cj + 2 * q + 1),
+                                               r, r ? rr[q] : make_uint4(0u, 0u, 0u, 0u), fin);
                             }
-                        };
-                        if (p.act == SN_ACT_RELU || p.act == SN_ACT_RELU6)
-                            finish_rows([hi = p.act == SN_ACT_RELU ? INFINITY : 6.0f](float x) { return fminf(fmaxf(x, 0.0f), hi); });
-                        else if (p.act == SN_ACT_NONE)
-                            finish_rows([](float x) { return x; });
-                        else
-                            finish_rows([act = p.act](float x) { return act_apply(x, act); });
+                        });
                         fence_proxy_async_smem();
                         __syncwarp();
                         if (lane == 0) {
@@ -749,12 +712,6 @@ __global__ void __launch_bounds__(THREADS, 1)
                     // bias + activation -> 16-bit, staged with the 128-byte swizzle
                     // (row = lane, 16-byte chunk j at j ^ (row & 7)), then one TMA
                     // tensor store of the warp's 32 x 64 block, clipped at the edges
-                    // this row's residual: 16-byte piece j of the row at j ^ (row & 7)
-                    uint32_t rv[2][16];
-#pragma unroll
-                    for (int h = 0; h < 2; ++h)
-#pragma unroll
-                        for (int j = 0; j < 16; ++j) rv[h][j] = 0u;
                     if (!has_res && lane == 0) bulk_wait_read_0();  // the previous store has read the block
                     if (has_res) {
                         const bool landed = mbar_wait(&res_bar[warp - 2], rpar, p.wait_limit);
@@ -765,14 +722,6 @@ __global__ void __launch_bounds__(THREADS, 1)
                             break;
                         }
                         ++res_landed;
-#pragma unroll
-                        for (int j = 0; j < 8; ++j) {
-                            const uint4 u = *reinterpret_cast<const uint4 *>(buf + lane * 128 + ((j ^ (lane & 7)) << 4));
-                            rv[j >> 2][4 * (j & 3)] = u.x;
-                            rv[j >> 2][4 * (j & 3) + 1] = u.y;
-                            rv[j >> 2][4 * (j & 3) + 2] = u.z;
-                            rv[j >> 2][4 * (j & 3) + 3] = u.w;
-                        }
                     }
                     uint32_t v[64];
                     __syncwarp();
@@ -796,34 +745,16 @@ __global__ void __launch_bounds__(THREADS, 1)
                         mbar_arrive_cluster(mapa(su32(&xfree_bar[warp - 2]), 1u));
                         xph ^= 1u;
                     }
-                    // every 4 packed pairs (8 channels) go to their 16-byte piece
-                    // of the row as soon as they are computed; the activation is
-                    // chosen once per chunk, so the unrolled body carries only its own
-                    auto stage_rows = [&](auto act) {
+                    // every 8 channels go to their 16-byte piece of the row as soon as
+                    // they are computed, in place of the residual's piece
+                    with_act2<T>(p.act, [&](auto fin) {
 #pragma unroll
                         for (int q = 0; q < 8; ++q) {
-                            const int h = q >> 2;
-                            uint32_t wq[4];
-#pragma unroll
-                            for (int e = 0; e < 4; ++e) {
-                                const int j = 4 * (q & 3) + e;  // pair index within the half
-                                const float2 r2 = unpack2<T>(rv[h][j]);
-                                const float f0 = act(__uint_as_float(v[32 * h + 2 * j]) +
-                                                     __shfl_sync(0xffffffffu, bias_r[cj][h], 2 * j) + r2.x);
-                                const float f1 = act(__uint_as_float(v[32 * h + 2 * j + 1]) +
-                                                     __shfl_sync(0xffffffffu, bias_r[cj][h], 2 * j + 1) + r2.y);
-                                wq[e] = pack2<T>(f0, f1);
-                            }
-                            *reinterpret_cast<uint4 *>(buf + lane * 128 + ((q ^ (lane & 7)) << 4)) =
-                                make_uint4(wq[0], wq[1], wq[2], wq[3]);
+                            uint4 *piece = reinterpret_cast<uint4 *>(buf + lane * 128 + ((q ^ (lane & 7)) << 4));
+                            *piece = finish8<T>(v + 8 * q, __ldg(bias4 + 16 * cj + 2 * q), __ldg(bias4 + 16 * cj + 2 * q + 1),
+                                                has_res, has_res ? *piece : make_uint4(0u, 0u, 0u, 0u), fin);
                         }
-                    };
-                    if (p.act == SN_ACT_RELU || p.act == SN_ACT_RELU6)
-                        stage_rows([hi = p.act == SN_ACT_RELU ? INFINITY : 6.0f](float x) { return fminf(fmaxf(x, 0.0f), hi); });
-                    else if (p.act == SN_ACT_NONE)
-                        stage_rows([](float x) { return x; });
-                    else
-                        stage_rows([act = p.act](float x) { return act_apply(x, act); });
+                    });
                     fence_proxy_async_smem();
                     __syncwarp();
                     if (!p.y_nchw) {
