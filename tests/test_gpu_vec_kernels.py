@@ -107,3 +107,20 @@ def test_depthwise_windows(ks, st, dil, c, h, w, dt):
     layer["bias"] = rng.standard_normal(c).astype(np.float32)
     ref = run_layer(layer, [stored_values(x, dt)], dt)
     assert maxrel(run_float([layer], x, (dt, "nhwc")), ref) <= TOL[dt]
+
+
+@pytest.mark.parametrize("ks,st,pd", [(3, 2, 1), (3, 2, 0), (2, 2, 0), (2, 2, 1), (3, 1, 1)])
+@pytest.mark.parametrize("n,c,h,w", [(1, 8, 3, 3), (2, 24, 7, 9), (3, 264, 10, 35), (8, 64, 113, 112)])
+@pytest.mark.parametrize("dt", ["f32", "f16", "bf16"])
+def test_maxpool_windows(ks, st, pd, n, c, h, w, dt):
+    # one row a thread and (the last size) four, the last group cut short;
+    # windows over every edge, infinities and a NaN (which the maximum passes over)
+    rng = np.random.default_rng(ks + h)
+    x = rng.standard_normal((n, c, h, w)).astype(np.float32)
+    x[0, 0] = -np.inf
+    x[-1, 1, 0, 0] = np.inf
+    x[0, 2, 1, 1] = np.nan
+    net = [{"type": "maxpool", "inputs": [-1], "params": dict(kh=ks, kw=ks, sh=st, sw=st, ph=pd, pw=pd)}]
+    xs = stored_values(x, dt)
+    ref = run_layer(net[0], [np.where(np.isnan(xs), -np.inf, xs)], dt)
+    np.testing.assert_array_equal(run_float(net, x, (dt, "nhwc")), ref)
