@@ -16,14 +16,13 @@ constexpr int BK = 64;
 // 12 warps: producer 0, MMA, 8 epilogue, producers 1-2.  Three warps per SM
 // sub-partition leave the epilogue up to 168 registers a thread.
 constexpr int THREADS = 384;
-// TMA producer threads for a ring of `stages` stages: one issuing thread
-// walks the stages s with s % n == its index, so n must divide the depth.
-// Two for an even depth; the third producer warp then waits on the MMA
-// issuer's barriers for it (see waits_for_mma).
-constexpr int producers_for(int stages) { return stages % 2 == 0 ? 2 : 3; }
+// TMA producer threads for a ring of `stages` stages: producer i issues the K
+// steps g with g % n == i.  Three for a ring of three; otherwise two, and the
+// third producer warp waits on the MMA issuer's barriers for it (see waits_for_mma).
+constexpr int producers_for(int stages) { return stages == 3 ? 3 : 2; }
 // A shared-memory access by the MMA-issuing thread (an mbarrier wait included)
 // queues behind the tensor core's operand reads and costs ~250 cycles, as much
-// as four MMAs: with an even ring depth, warp 11 waits on the stage-full and
+// as four MMAs: with two producers, warp 11 waits on the stage-full and
 // accumulator-drained barriers instead and hands each result to the MMA warp
 // through a hardware named barrier (bar.red.or: both warps pass it together,
 // and the OR of their predicates tells both whether to stop).
@@ -35,6 +34,11 @@ constexpr int stages_for(int bn, int g, int kb, int ms = 1, int extra = 0) {
     return (198656 - extra) / (kb * (16384 * ms + bn / g * 128)) < 8
                ? (198656 - extra) / (kb * (16384 * ms + bn / g * 128))
                : 8;
+}
+// epilogue staging blocks per warp: two where that leaves four stages, so that a
+// block's residual is loaded, and its store read, while the other is worked on
+constexpr int staging_blocks(int bn, int g, int kb, int ms) {
+    return g == 1 && stages_for(bn, g, kb, ms, 32768) >= 4 ? 2 : 1;
 }
 // halo tiles (3x3, stride 1): 8 x 16 output pixels of one image; a stage
 // holds the 10 x 16 input pixels one tap row reads (all three column taps)
@@ -497,6 +501,8 @@ __device__ __forceinline__ void tma_store_4d(const CUtensorMap *m, const void *s
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 // at most one store group may still be reading shared memory
 __device__ __forceinline__ void bulk_wait_read_0() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+// all but the latest of this thread's store groups have read their shared memory
+__device__ __forceinline__ void bulk_wait_read_1() { asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
 // one unit of work: a 128 x BN tile and the K-range [it0, it1) it accumulates

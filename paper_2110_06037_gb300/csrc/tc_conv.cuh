@@ -67,7 +67,7 @@ namespace tc {
 // any row offset and group stride work): one A box per three taps instead of
 // three, and 10/8 of the rows instead of three times them.
 template <typename T, int BN, int STAGES, bool IMPLICIT, int G, int KB, bool BST, int MS, int CSK, bool SK,
-          bool HALO>
+          bool HALO, int NBUF>
 __global__ void __launch_bounds__(THREADS, 1)
     conv_tc_kernel(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ CUtensorMap mA1,
                    const __grid_constant__ CUtensorMap mA2, const __grid_constant__ CUtensorMap mA3,
@@ -92,7 +92,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     __shared__ __align__(8) uint64_t empty_bar[STAGES];
     __shared__ __align__(8) uint64_t accf_bar[2];  // MMA -> epilogue: accumulator ready
     __shared__ __align__(8) uint64_t acce_bar[2];  // epilogue -> MMA: accumulator drained
-    __shared__ __align__(8) uint64_t res_bar[EPI_WARPS];  // residual tile landed in a warp's staging block
+    __shared__ __align__(8) uint64_t res_bar[EPI_WARPS * NBUF];  // residual tile landed in a warp's staging block
     __shared__ __align__(8) uint64_t bst_bar;              // weight-stationary B landed
     // CSK = 2 (cluster K split): the two CTAs of a cluster take the two halves
     // of a tile's K steps; CTA 1's epilogue warps write their fp32 partial
@@ -180,9 +180,7 @@ __global__ void __launch_bounds__(THREADS, 1)
             // one arrival per epilogue warp draining it, in both CTAs of a pair
             mbar_init(&acce_bar[b], G * (BN >= 128 || MS == 2 ? EPI_WARPS : EPI_WARPS / 2));
         }
-        for (int i = 0; i < EPI_WARPS; ++i) {
-            mbar_init(&res_bar[i], 1);
-        }
+        for (int i = 0; i < EPI_WARPS * NBUF; ++i) mbar_init(&res_bar[i], 1);
         mbar_init(&bst_bar, 1);
         for (int i = 0; i < EPI_WARPS; ++i) {
             mbar_init(&xfull_bar[i], 32);  // every lane of the peer warp arrives after its stores
@@ -535,7 +533,8 @@ __global__ void __launch_bounds__(THREADS, 1)
         const int g4 = warp & 3;
         const int msub = MS == 2 ? half : 0;          // the 128-row half this warp drains
         const int row = msub * BM + g4 * 32 + lane;    // row within the unit's tile
-        uint8_t *buf = stg + (warp - 2) * STG_BYTES;  // one 32 x 64 staging block per warp
+        uint8_t *const blocks = stg + (warp - 2) * NBUF * STG_BYTES;  // this warp's 32 x 64 staging blocks
+        uint64_t *const rbars = res_bar + (warp - 2) * NBUF;
         const int r0 = msub * BM + g4 * 32;
         const int wq0 = IMPLICIT ? r0 & (p.BW - 1) : 0;
         const int hp0 = IMPLICIT ? (r0 >> p.lbw) & (p.BH - 1) : 0;
@@ -545,8 +544,11 @@ __global__ void __launch_bounds__(THREADS, 1)
         constexpr bool ALT = NCH == 1 && MS == 1;        // alternate units between the groups
         const int cbase = (ALT || MS == 2) ? 0 : half * CPH;  // first chunk of this warp
         int lt = ALT ? half : 0;
-        uint32_t rpar = 0;  // phase parity of this warp's residual barrier
-        int res_issued = 0, res_landed = 0;  // residual loads issued / waited for (warp-uniform)
+        // residual loads issued / waited for (warp-uniform); load i goes to block
+        // i % NBUF.  With two blocks there is a load for every 64-channel chunk or
+        // for none, and chunk `nchunk` uses block nchunk % 2
+        int res_issued = 0, res_landed = 0, nchunk = 0;
+        bool primed = false;  // the load of this unit's first chunk was issued during the previous unit
         uint32_t xph = 0;   // cluster K split: phase parity of this warp's exchange block
         bool waited = false;
         for (int ui = ALT ? half : 0; ui < nunits; ui += ALT ? 2 : 1, lt += ALT ? 2 : 1) {
@@ -581,30 +583,37 @@ __global__ void __launch_bounds__(THREADS, 1)
             // the idle CTA of a pair whose group has one tile stores nothing
             const bool tile_live = w.mt < p.mtiles;
             // residual (fused add): the warp's 32 x 64 block of it is loaded by
-            // TMA into the warp's staging block (the box and coordinates of the
-            // output store; zero outside the tensor) once the previous store has
-            // read that block; the first chunk's load is issued before the
-            // accumulator wait, the next one's after the current chunk's store
+            // TMA into a staging block (the box and coordinates of the output
+            // store; zero outside the tensor) once the store before has read that
+            // block.  One block: the first chunk's load is issued before the
+            // accumulator wait, the next one's after the current chunk's store.  Two
+            // blocks: the next chunk's (or next unit's) before the current chunk's
+            // arithmetic, which hides the load's latency (32 x 56 x 56, 64 -> 256 with
+            // a residual: 25 -> 21 us)
             if (!waited) {
                 griddep_wait();
                 waited = true;
             }
             // (a stream-K part reads the residual only if it finishes the tile)
             const bool has_res = p.res != nullptr && p.ksplit == 1 && (!SK || w.sk_n == 1);
-            auto issue_res = [&](int k0) {
+            auto issue_res = [&](const Work &wk, int k0) {
                 // no new copies once the kernel is stopping
-                if (!has_res || !tile_live || k0 >= p.K || __shfl_sync(0xffffffffu, (int)abort_sh, 0)) return;
+                if (!has_res || wk.mt >= p.mtiles || k0 >= p.K || __shfl_sync(0xffffffffu, (int)abort_sh, 0)) return;
+                const int i = NBUF == 2 ? res_issued & 1 : 0;
                 ++res_issued;
                 if (lane == 0) {
+                    uint64_t *bar = &rbars[i];
+                    const uint32_t dst = su32(blocks + i * STG_BYTES);
                     bulk_wait_read_0();
-                    mbar_expect_tx(&res_bar[warp - 2], STG_BYTES);
+                    mbar_expect_tx(bar, STG_BYTES);
                     if (IMPLICIT)
-                        tma_4d<1>(su32(buf), &mR, su32(&res_bar[warp - 2]), k0, w.q0 + wq0, w.p0 + hp0, w.i0 + ni0);
+                        tma_4d<1>(dst, &mR, su32(bar), k0, wk.q0 + wq0, wk.p0 + hp0, wk.i0 + ni0);
                     else
-                        tma_2d<1>(su32(buf), &mR, su32(&res_bar[warp - 2]), k0, (int)(w.m0 + r0));
+                        tma_2d<1>(dst, &mR, su32(bar), k0, (int)(wk.m0 + r0));
                 }
             };
-            issue_res(w.n0 + 64 * cbase);
+            if (!primed) issue_res(w, w.n0 + 64 * cbase);
+            primed = false;
             if (!mbar_wait(&accf_bar[b], aph, p.wait_limit)) {
                 if (lane == 0) atomicOr(p.err, ERR_ACC_WAIT);
                 set_abort();
@@ -674,6 +683,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                                 acc[4 * q + 3] += x.w;
                             }
                         }
+                        uint8_t *buf = blocks;
                         if (lane == 0) bulk_wait_read_0();  // the previous store has read the block
                         __syncwarp();
                         // this row's residual (the output's NHWC layout), 8 channels per piece
@@ -712,10 +722,15 @@ __global__ void __launch_bounds__(THREADS, 1)
                     // bias + activation -> 16-bit, staged with the 128-byte swizzle
                     // (row = lane, 16-byte chunk j at j ^ (row & 7)), then one TMA
                     // tensor store of the warp's 32 x 64 block, clipped at the edges
-                    if (!has_res && lane == 0) bulk_wait_read_0();  // the previous store has read the block
+                    const int blk = NBUF == 2 ? nchunk & 1 : 0;
+                    uint8_t *buf = blocks + blk * STG_BYTES;
+                    if (!has_res && lane == 0) {  // the last store of this block has read it
+                        if (NBUF == 2) bulk_wait_read_1();
+                        else bulk_wait_read_0();
+                    }
                     if (has_res) {
-                        const bool landed = mbar_wait(&res_bar[warp - 2], rpar, p.wait_limit);
-                        rpar ^= 1u;
+                        const uint32_t par = (uint32_t)(NBUF == 2 ? res_landed >> 1 : res_landed) & 1u;
+                        const bool landed = mbar_wait(&rbars[blk], par, p.wait_limit);
                         if (!__all_sync(0xffffffffu, landed)) {
                             if (lane == 0) atomicOr(p.err, ERR_EPI_WAIT);
                             set_abort();
@@ -723,6 +738,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                         }
                         ++res_landed;
                     }
+                    ++nchunk;
                     uint32_t v[64];
                     __syncwarp();
                     tmem_ld64(taddr, v);
@@ -744,6 +760,15 @@ __global__ void __launch_bounds__(THREADS, 1)
                         }
                         mbar_arrive_cluster(mapa(su32(&xfree_bar[warp - 2]), 1u));
                         xph ^= 1u;
+                    }
+                    if (NBUF == 2) {  // the next chunk's residual (all of this loop's conditions, one chunk on)
+                        if (cj + 1 < CPH && k0 + 64 < p.K) {
+                            issue_res(w, k0 + 64);
+                        } else if (ui + (ALT ? 2 : 1) < nunits) {
+                            const Work wn = unit(ui + (ALT ? 2 : 1), (int)rank);
+                            issue_res(wn, wn.n0 + 64 * cbase);
+                            primed = true;
+                        }
                     }
                     // every 8 channels go to their 16-byte piece of the row as soon as
                     // they are computed, in place of the residual's piece
@@ -782,7 +807,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                         fence_proxy_async_smem();  // these reads before TMA writes the block again
                     }
                     __syncwarp();
-                    if (cj + 1 < CPH) issue_res(k0 + 64);
+                    if (NBUF == 1 && cj + 1 < CPH) issue_res(w, k0 + 64);
                 } else {
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
@@ -822,7 +847,8 @@ __global__ void __launch_bounds__(THREADS, 1)
             bulk_wait_read_0();
             const long long t0 = clock64();
             for (int i = res_landed; i < res_issued; ++i)
-                while (!mbar_try(&res_bar[warp - 2], (uint32_t)i & 1u) && clock64() - t0 < WAIT_LIMIT) {
+                while (!mbar_try(&rbars[NBUF == 2 ? i & 1 : 0], (uint32_t)(NBUF == 2 ? i >> 1 : i) & 1u) &&
+                       clock64() - t0 < WAIT_LIMIT) {
                 }
         }
         __syncwarp();
@@ -900,16 +926,18 @@ template <typename T, int BN, bool IMPLICIT, int G, int KB, bool BST = false, in
 static cudaError_t launch(const CUtensorMap *mA, const CUtensorMap &mB, const CUtensorMap &mY, const CUtensorMap &mR,
                           const Params &p,
                           cudaStream_t st) {
-    constexpr int STAGES = BST ? BST_STAGES : HALO ? halo_stages(BN / G) : stages_for(BN, G, KB, MS);
+    constexpr int NBUF = BST || HALO || SK || CSK > 1 ? 1 : staging_blocks(BN, G, KB, MS);
+    constexpr uint32_t STG = NBUF * EPI_WARPS * STG_BYTES;
+    constexpr int STAGES = BST ? BST_STAGES : HALO ? halo_stages(BN / G) : stages_for(BN, G, KB, MS, (NBUF - 1) * 32768);
     // bytes of one pipeline stage (A and this CTA's share of B), as the kernel lays them out
     constexpr size_t STAGE = HALO ? (size_t)HALO_ROWS * BK * 2 + 3 * (size_t)(BN / G) * BK * 2
                                   : (size_t)KB * (MS * BM * BK * 2 + (BN / G) * BK * 2);
     static_assert(CSK == 1 || (size_t)STAGES * KB * (BM * BK * 2 + BN * BK * 2) >= EPI_WARPS * XBLK_BYTES,
                   "cluster K split: the exchange blocks live in the stage memory");
     constexpr size_t smem_max = 227 * 1024;
-    const size_t smem = BST ? (size_t)STAGES * BM * BK * 2 + p.bst_bytes + EPI_WARPS * STG_BYTES + 1024
-                            : (size_t)STAGES * STAGE + EPI_WARPS * STG_BYTES + 1024;
-    static_assert(BST || (size_t)STAGES * STAGE + EPI_WARPS * STG_BYTES + 1024 <= smem_max, "shared memory per CTA");
+    const size_t smem = BST ? (size_t)STAGES * BM * BK * 2 + p.bst_bytes + STG + 1024
+                            : (size_t)STAGES * STAGE + STG + 1024;
+    static_assert(BST || (size_t)STAGES * STAGE + STG + 1024 <= smem_max, "shared memory per CTA");
     static_assert(!HALO || (IMPLICIT && KB == 1 && MS == 1 && !BST && CSK == 1 && !SK),
                   "halo tiles: implicit tiles of one CTA or a pair, one channel block per stage");
     static_assert(!BST || (G == 1 && KB == 1 && MS == 1), "weight-stationary tiles are one-CTA, one block per stage");
@@ -918,7 +946,7 @@ static cudaError_t launch(const CUtensorMap *mA, const CUtensorMap &mB, const CU
     static_assert(!SK || (G == 1 && MS == 1 && !BST && CSK == 1 && BN >= 128), "stream-K: one-CTA tiles of >= 2 chunks");
     static_assert(STAGES >= 2, "pipeline depth");
     if (smem > smem_max) return cudaErrorInvalidValue;
-    auto kern = conv_tc_kernel<T, BN, STAGES, IMPLICIT, G, KB, BST, MS, CSK, SK, HALO>;
+    auto kern = conv_tc_kernel<T, BN, STAGES, IMPLICIT, G, KB, BST, MS, CSK, SK, HALO, NBUF>;
     constexpr bool CLUSTER = G == 2 || CSK == 2;
     static int max_groups = 0;  // co-resident CTAs (G = 1) or clusters of two (pairs, K split)
     cudaLaunchConfig_t cfg = {};

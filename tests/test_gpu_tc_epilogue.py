@@ -66,3 +66,41 @@ def test_values_of_the_epilogue(act, residual, dt):
         np.testing.assert_array_equal(y, ref, err_msg=g.candidate_desc(int(c)))
         seen += 1
     assert seen > 4
+
+
+@pytest.mark.parametrize("dt", ["f16", "bf16"])
+@pytest.mark.parametrize("c,k", [(64, 136), (72, 320)])
+def test_residual_over_many_tiles(c, k, dt):
+    # several tiles a CTA, the last ones ragged in pixels and channels: the
+    # residual of the next tile is loaded while this one is stored
+    import torch
+    rng = np.random.default_rng(k)
+    x = rng.standard_normal((9, c, 57, 57)).astype(np.float32)
+    pick = rng.integers(0, c, k)
+    w = np.zeros((k, c, 1, 1), np.float32)
+    w[np.arange(k), pick] = 1.0
+    bias = rng.integers(-2, 3, k).astype(np.float32)
+    first = dict(synth.conv(c, k, 1, 1, 0, act="none"), weight=w, bias=np.zeros(k, np.float32), inputs=[-1])
+    conv = dict(synth.conv(c, k, 1, 1, 0, act="relu"), weight=w, bias=bias, inputs=[-1, 0])
+    sch = (dt, "nhwc")
+    f = stored_values(x, dt)[:, pick]
+    # the library's order: (sum + bias) + residual, each rounded to fp32
+    v = (f.astype(np.float32) + bias[None, :, None, None]).astype(np.float32) + f.astype(np.float32)
+    ref = stored_values(np.maximum(v, 0.0), dt)
+    g = build_graph([first, conv], x.shape, sch, sch, [sch])
+    t = g.cost_table()
+    p = [int(np.flatnonzero(t["layer"] == i)[0]) for i in range(t["n_layers"])]
+    desc = {int(c): g.candidate_desc(int(c)) for c in np.flatnonzero((t["layer"] == 1) | (t["layer"] == 2))}
+    p[1] = [i for i, d in desc.items() if t["layer"][i] == 1 and f"conv2/igemm_tc {dt}.nhwc [" in d][0]
+    xd = to_device(x, sch)
+    seen = 0
+    for i, d in desc.items():
+        if t["layer"][i] != 2 or f"conv2/igemm_tc {dt}.nhwc [" not in d:
+            continue
+        p[2] = i
+        g.set_path(p)
+        y = from_device(g.run(xd), sch)
+        torch.cuda.synchronize()
+        np.testing.assert_array_equal(y, ref, err_msg=d)
+        seen += 1
+    assert seen > 4
