@@ -158,41 +158,49 @@ __global__ void __launch_bounds__(THREADS, 1)
         if (CLUSTER) st_cluster_u32(mapa(su32((const void *)&abort_sh), crank ^ 1u), 1u);
     };
 
-    if (threadIdx.x == 0) {
+    // Set-up, spread over the warps: a CTA that fills an SM starts it only when
+    // the previous kernel's CTA has left, so it is on the critical path (one
+    // thread doing all but the allocation took ~1700 cycles, this ~1300).
+    if (warp == 0) {
+        tmem_alloc<G>(&tmem_sh, TMEM_COLS);
+    } else if (warp == 1) {
+        if (lane < STAGES) mbar_init(&full_bar[lane], 1);  // the (leader's) producer of the stage
+        if (lane >= 16 && lane < 16 + STAGES) mbar_init(&empty_bar[lane - 16], 1);
+        fence_mbar_init();
+    } else if (warp == 2) {
         // the tensor maps are kernel parameters, not data of the previous kernel
-        const CUtensorMap *maps[7] = {&mA0, &mA1, &mA2, &mA3, &mB, &mY, &mR};
-        for (int i = 0; i < 7; ++i) asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(maps[i])) : "memory");
+        const CUtensorMap *m = lane == 0 ? &mA0 : lane == 1 ? &mB : lane == 2 ? &mY : lane == 3 ? &mR
+                             : lane == 4 ? &mA1 : lane == 5 ? &mA2 : &mA3;
+        if (lane < 7) asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(m)) : "memory");
+    } else if (warp == 3) {
         // this CTA's slice of the weights into L2 while the previous kernel
         // finishes (after an L2 flush they would otherwise come from HBM
         // on the critical path of the first K steps)
-        if (p.wt_bytes > 0) {
+        if (lane == 0 && p.wt_bytes > 0) {
             const int64_t slice = ((p.wt_bytes + gridDim.x - 1) / gridDim.x + 15) & ~(int64_t)15;
             const int64_t off = (int64_t)blockIdx.x * slice;
             if (off < p.wt_bytes)
                 prefetch_l2(static_cast<const uint8_t *>(p.wt) + off, (uint32_t)min(slice, p.wt_bytes - off));
         }
-        for (int s = 0; s < STAGES; ++s) {
-            mbar_init(&full_bar[s], 1);  // the (leader's) producer of the stage
-            mbar_init(&empty_bar[s], 1);
+    } else if (warp == 4) {
+        if (lane < 2) mbar_init(&accf_bar[lane], 1);
+        // one arrival per epilogue warp draining it, in both CTAs of a pair
+        if (lane >= 2 && lane < 4) mbar_init(&acce_bar[lane - 2], G * (BN >= 128 || MS == 2 ? EPI_WARPS : EPI_WARPS / 2));
+        if (lane == 4) mbar_init(&bst_bar, 1);
+        if (lane >= 8 && lane < 12) issued_sh[lane - 8] = 0;
+        if (lane == 12) {
+            abort_sh = 0;
+            consumed_sh = 0;
         }
-        for (int b = 0; b < 2; ++b) {
-            mbar_init(&accf_bar[b], 1);
-            // one arrival per epilogue warp draining it, in both CTAs of a pair
-            mbar_init(&acce_bar[b], G * (BN >= 128 || MS == 2 ? EPI_WARPS : EPI_WARPS / 2));
-        }
-        for (int i = 0; i < EPI_WARPS * NBUF; ++i) mbar_init(&res_bar[i], 1);
-        mbar_init(&bst_bar, 1);
-        for (int i = 0; i < EPI_WARPS; ++i) {
-            mbar_init(&xfull_bar[i], 32);  // every lane of the peer warp arrives after its stores
-            mbar_init(&xfree_bar[i], 32);
-        }
-        abort_sh = 0;
-        issued_sh[0] = issued_sh[1] = issued_sh[2] = issued_sh[3] = 0;
-        consumed_sh = 0;
+        fence_mbar_init();
+    } else if (warp == 5) {
+        if (lane < EPI_WARPS * NBUF) mbar_init(&res_bar[lane], 1);
+        // every lane of the peer warp arrives after its stores
+        if (CSK == 2 && lane >= 16 && lane < 16 + EPI_WARPS) mbar_init(&xfull_bar[lane - 16], 32);
+        if (CSK == 2 && lane >= 24 && lane < 24 + EPI_WARPS) mbar_init(&xfree_bar[lane - 24], 32);
         fence_mbar_init();
     }
     if (CLUSTER) cluster_sync_all();  // both CTAs' barriers exist before either signals the other
-    if (warp == 0) tmem_alloc<G>(&tmem_sh, TMEM_COLS);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -255,7 +263,18 @@ __global__ void __launch_bounds__(THREADS, 1)
             const int brow = (int)rank * (BN / G);
             int g = 0, s = prod, issued = 0;
             uint32_t par = 0;
-            bool stop = false, waited = false;
+            bool stop = false;
+            // the weights of K step `it` (block cb of tap `tap`) to its stage
+            auto load_b = [&](const Work &w, int st, int tap, int cb) {
+                const uint32_t sb = su32(smem + st * STAGE_BYTES) + A_BYTES;
+                const uint32_t bar = G == 2 ? mapa(su32(&full_bar[st]), 0u) : su32(&full_bar[st]);
+                if (HALO)  // the three taps of row `tap`: map [C][K][R*S], box 64 x BN x 3
+                    tma_3d<G>(sb, &mB, bar, cb * BK, w.n0 + brow, tap * 3);
+                else if (KB == 1)
+                    tma_3d<G>(sb, &mB, bar, cb * BK, tap, w.n0 + brow);
+                else
+                    tma_4d<G>(sb, &mB, bar, 0, tap, w.n0 + brow, cb);
+            };
             if (BST && prod == 0) {
                 // the weights are not written by the previous kernel: loaded
                 // before the dependency wait, one box per K step
@@ -269,6 +288,26 @@ __global__ void __launch_bounds__(THREADS, 1)
                     }
                 }
             }
+            // the weights of the first unit's first stages too (the barrier's bytes
+            // are those of the whole stage; A follows below whatever happens, so
+            // that every stage begun completes)
+            int early = 0;
+            if (!BST && nunits > 0) {
+                const Work w = unit(0, (int)rank);
+                early = min(STAGES, w.it1 - w.it0);
+                int tap = (int)fdiv((uint32_t)w.it0, p.fd_spt), cb = (w.it0 - tap * p.fd_spt.d) * KB;
+                for (int st = 0; st < early; ++st) {
+                    if (st % NPROD == prod) {
+                        if (leader) mbar_expect_tx(&full_bar[st], G * STAGE_BYTES);
+                        load_b(w, st, tap, cb);
+                    }
+                    if ((cb += KB) == cblocks) {
+                        cb = 0;
+                        ++tap;
+                    }
+                }
+            }
+            if (nunits > 0) griddep_wait();
             for (int ui = 0; ui < nunits && !stop; ++ui) {
                 const Work w = unit(ui, (int)rank);
                 int tap = (int)fdiv((uint32_t)w.it0, p.fd_spt);
@@ -276,17 +315,15 @@ __global__ void __launch_bounds__(THREADS, 1)
                 int r = (int)fdiv((uint32_t)tap, p.fd_S), ss = tap - r * S;
                 for (int it = w.it0; it < w.it1; ++it, ++g) {
                     if (g % NPROD == prod) {
-                        if (!mbar_wait(&empty_bar[s], par ^ 1u, p.wait_limit)) {
-                            atomicOr(p.err, ERR_TMA_WAIT);
-                            set_abort();
-                        }
-                        if (abort_sh) {
-                            stop = true;
-                            break;
-                        }
-                        if (!waited) {
-                            griddep_wait();
-                            waited = true;
+                        if (g >= early) {  // (the first ring's stages start empty)
+                            if (!mbar_wait(&empty_bar[s], par ^ 1u, p.wait_limit)) {
+                                atomicOr(p.err, ERR_TMA_WAIT);
+                                set_abort();
+                            }
+                            if (abort_sh) {
+                                stop = true;
+                                break;
+                            }
                         }
                         const uint32_t sa = su32(smem + s * STAGE_BYTES);
                         // KB = 1: channel coordinate cb * 64 on the innermost axis;
@@ -294,7 +331,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                         // box spans KB blocks
                         const int c0 = cb * BK;
                         // the leader's barrier counts the bytes of both CTAs
-                        if (leader) mbar_expect_tx(&full_bar[s], G * STAGE_BYTES);  // A only when BST
+                        if (leader && g >= early) mbar_expect_tx(&full_bar[s], G * STAGE_BYTES);  // A only when BST
                         const uint32_t bar = G == 2 ? mapa(su32(&full_bar[s]), 0u) : su32(&full_bar[s]);
                         if (IMPLICIT) {
                             const int oh = r * dh - ph0, ow = ss * dw - pw0;
@@ -316,14 +353,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                             else
                                 tma_3d<G>(sa, &mA0, bar, 0, (int)w.m0, cb);
                         }
-                        if (HALO) {  // the three taps of row `tap`: map [C][K][R*S], box 64 x BN x 3
-                            tma_3d<G>(sa + A_BYTES, &mB, bar, c0, w.n0 + brow, tap * 3);
-                        } else if (!BST) {  // weight-stationary B is already resident
-                            if (KB == 1)
-                                tma_3d<G>(sa + A_BYTES, &mB, bar, c0, tap, w.n0 + brow);
-                            else
-                                tma_4d<G>(sa + A_BYTES, &mB, bar, 0, tap, w.n0 + brow, cb);
-                        }
+                        if (!BST && g >= early) load_b(w, s, tap, cb);  // weight-stationary B is already resident
                         issued = g + 1;
                         s += NPROD;
                         if (s >= STAGES) {
