@@ -100,6 +100,11 @@ __global__ void __launch_bounds__(THREADS, 1)
     // block handed to CTA 1 once CTA 0's stages are done with (xfree)
     __shared__ __align__(8) uint64_t xfull_bar[EPI_WARPS];  // CTA 0: a partial block landed
     __shared__ __align__(8) uint64_t xfree_bar[EPI_WARPS];  // CTA 1: CTA 0 has read the block
+    // the bias of the two units whose accumulators are in flight (tiles of 256
+    // channels leave no room beside the stages, and a stream-K part may be
+    // finished after its accumulator: those read it through L1)
+    constexpr bool BIAS_SH = BN <= 128 && !SK;
+    __shared__ __align__(16) float bias_sh[BIAS_SH ? 2 * BN : 4];
     __shared__ uint32_t tmem_sh;
     __shared__ volatile int abort_sh;
     __shared__ int issued_sh[4], consumed_sh;
@@ -263,7 +268,7 @@ __global__ void __launch_bounds__(THREADS, 1)
             const int brow = (int)rank * (BN / G);
             int g = 0, s = prod, issued = 0;
             uint32_t par = 0;
-            bool stop = false;
+            bool stop = false, waited = false;
             // the weights of K step `it` (block cb of tap `tap`) to its stage
             auto load_b = [&](const Work &w, int st, int tap, int cb) {
                 const uint32_t sb = su32(smem + st * STAGE_BYTES) + A_BYTES;
@@ -307,7 +312,6 @@ __global__ void __launch_bounds__(THREADS, 1)
                     }
                 }
             }
-            if (nunits > 0) griddep_wait();
             for (int ui = 0; ui < nunits && !stop; ++ui) {
                 const Work w = unit(ui, (int)rank);
                 int tap = (int)fdiv((uint32_t)w.it0, p.fd_spt);
@@ -333,6 +337,10 @@ __global__ void __launch_bounds__(THREADS, 1)
                         // the leader's barrier counts the bytes of both CTAs
                         if (leader && g >= early) mbar_expect_tx(&full_bar[s], G * STAGE_BYTES);  // A only when BST
                         const uint32_t bar = G == 2 ? mapa(su32(&full_bar[s]), 0u) : su32(&full_bar[s]);
+                        if (!waited) {
+                            griddep_wait();
+                            waited = true;
+                        }
                         if (IMPLICIT) {
                             const int oh = r * dh - ph0, ow = ss * dw - pw0;
                             const CUtensorMap *m = &mA0;
@@ -586,10 +594,21 @@ __global__ void __launch_bounds__(THREADS, 1)
             const uint32_t aph = (uint32_t)(lt >> 1) & 1u;
             const Work w = unit(ui, (int)rank);
             // bias of this warp's channels (the buffer is zero-padded to a multiple
-            // of 256 channels): its lines into L1 before the accumulator wait, so
-            // that the broadcast 16-byte loads below hit
-            const float4 *bias4 = reinterpret_cast<const float4 *>(p.bias + w.n0 + 64 * cbase);
-            if (p.ksplit == 1 && lane < 2 * CPH && cbase * 2 + lane < BN / 32) prefetch_l1(bias4 + 8 * lane);
+            // of 256 channels), fetched before the accumulator wait; the accumulator's
+            // slot of bias_sh is free after it, as the accumulator was
+            const float *bias = p.bias + w.n0 + 64 * cbase;
+            float *bsh = bias_sh + (BIAS_SH ? b * BN + 64 * cbase : 0);
+            float bias_r[2 * CPH];
+            if constexpr (BIAS_SH) {
+#pragma unroll
+                for (int j = 0; j < 2 * CPH; ++j) bias_r[j] = p.ksplit == 1 ? __ldg(bias + 32 * j + lane) : 0.f;
+            } else if (p.ksplit == 1 && lane < 2 * CPH) {
+                prefetch_l1(bias + 32 * lane);
+            }
+            auto bias4 = [&](int i) {
+                if constexpr (BIAS_SH) return reinterpret_cast<const float4 *>(bsh)[i];
+                else return __ldg(reinterpret_cast<const float4 *>(bias) + i);
+            };
             bool valid;
             int64_t pix;
             if (IMPLICIT) {
@@ -650,6 +669,11 @@ __global__ void __launch_bounds__(THREADS, 1)
                 break;
             }
             tc_fence_after();
+            if constexpr (BIAS_SH) {
+#pragma unroll
+                for (int j = 0; j < 2 * CPH; ++j) bsh[32 * j + lane] = bias_r[j];
+                __syncwarp();
+            }
             // cluster K split: this CTA's MMAs have read their last stage, so
             // the stage memory may now take CTA 1's partials
             if (CSK == 2) mbar_arrive_cluster(mapa(su32(&xfree_bar[warp - 2]), 1u));
@@ -724,7 +748,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                             for (int q = 0; q < 8; ++q) {
                                 const bool r = row_res && k0 + 8 * q < p.K;
                                 *reinterpret_cast<uint4 *>(buf + lane * 128 + ((q ^ (lane & 7)) << 4)) =
-                                    finish8<T>(acc + 8 * q, __ldg(bias4 + 16 * cj + 2 * q), __ldg(bias4 + 16 * cj + 2 * q + 1),
+                                    finish8<T>(acc + 8 * q, bias4(16 * cj + 2 * q), bias4(16 * cj + 2 * q + 1),
                                                r, r ? rr[q] : make_uint4(0u, 0u, 0u, 0u), fin);
                             }
                         });
@@ -806,7 +830,7 @@ __global__ void __launch_bounds__(THREADS, 1)
 #pragma unroll
                         for (int q = 0; q < 8; ++q) {
                             uint4 *piece = reinterpret_cast<uint4 *>(buf + lane * 128 + ((q ^ (lane & 7)) << 4));
-                            *piece = finish8<T>(v + 8 * q, __ldg(bias4 + 16 * cj + 2 * q), __ldg(bias4 + 16 * cj + 2 * q + 1),
+                            *piece = finish8<T>(v + 8 * q, bias4(16 * cj + 2 * q), bias4(16 * cj + 2 * q + 1),
                                                 has_res, has_res ? *piece : make_uint4(0u, 0u, 0u, 0u), fin);
                         }
                     });
