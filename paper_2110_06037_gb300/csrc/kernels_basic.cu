@@ -1325,14 +1325,15 @@ __global__ void gap_nchw(const T *__restrict__ x, T *__restrict__ y, int64_t NC,
 
 // NHWC, 16-byte channel vectors: a block owns eight of them (128 contiguous
 // bytes of every pixel) of one image; the other thread axis cuts the pixels
-// into blockDim / 8 slices, each summed in f32 with four loads in flight.  The
-// four slices of a warp are added by shuffles, the warps in order through
-// shared memory, so the sum does not depend on timing.  What bounds the kernel
-// is the chain of load latencies of one slice, not bytes: at 28 x 28 one block
+// into blockDim / 8 slices, each summed in f32 with eight loads in flight.  The
+// four slices of a warp are added by shuffles, the warps' sums by a warp per
+// channel, so the sum does not depend on timing.  What bounds the kernel
+// is the chain of latencies of one slice, not bytes: at 28 x 28 one block
 // of 32 vectors x 8 slices per image walked 98 pixels per thread and took
 // longer than an adapt plus the NCHW kernel (8 x 28 x 28 x 120 bf16, each op
 // between timing nodes of a replayed net, an empty op reading about 5 us: 15.5
-// us for the pair, 9.1 us for this kernel).
+// us for the pair, 9.1 us for this kernel; four loads in flight and the warps
+// added by one thread a channel: 5.0 us by itself, now 4.6).
 template <typename T>
 __global__ void __launch_bounds__(1024) gap_nhwc_vec(const T *__restrict__ x, T *__restrict__ y, int C, int HW) {
     griddep_launch();
@@ -1348,23 +1349,18 @@ __global__ void __launch_bounds__(1024) gap_nhwc_vec(const T *__restrict__ x, T 
     for (int e = 0; e < E; ++e) s[e] = 0.f;
     if (cv < CV) {
         const T *xn = x + (size_t)n * HW * C + (size_t)cv * E;
-        int p = sl;
-        for (; p + 3 * slices < HW; p += 4 * slices) {
-            uint4 q[4];
+        for (int p = sl; p < HW; p += 8 * slices) {  // eight loads in flight, the last ones too
+            uint4 q[8];
 #pragma unroll
-            for (int k = 0; k < 4; ++k) q[k] = *reinterpret_cast<const uint4 *>(xn + (size_t)(p + k * slices) * C);
+            for (int k = 0; k < 8; ++k)
+                q[k] = p + k * slices < HW ? *reinterpret_cast<const uint4 *>(xn + (size_t)(p + k * slices) * C)
+                                           : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
+            for (int k = 0; k < 8; ++k) {
                 const T *pv = reinterpret_cast<const T *>(&q[k]);
 #pragma unroll
                 for (int e = 0; e < E; ++e) s[e] += ldf<T>(pv + e);
             }
-        }
-        for (; p < HW; p += slices) {
-            const uint4 q = *reinterpret_cast<const uint4 *>(xn + (size_t)p * C);
-            const T *pv = reinterpret_cast<const T *>(&q);
-#pragma unroll
-            for (int e = 0; e < E; ++e) s[e] += ldf<T>(pv + e);
         }
     }
 #pragma unroll
@@ -1378,11 +1374,12 @@ __global__ void __launch_bounds__(1024) gap_nhwc_vec(const T *__restrict__ x, T 
         for (int e = 0; e < E; ++e) part[warp][v * E + e] = s[e];
     }
     __syncthreads();
-    const int c = threadIdx.x;  // channel within the block's 8 * E
-    if (c < 8 * E && blockIdx.x * 8 * E + c < C) {
-        float t = 0.f;
-        for (int k = 0; k < (int)(blockDim.x >> 5); ++k) t += part[k][c];
-        stf<T>(y + (size_t)n * C + blockIdx.x * 8 * E + c, t / (float)HW);
+    // a warp per channel of the block's 8 * E: the warps' sums, one a lane
+    const int lane = threadIdx.x & 31, warps = blockDim.x >> 5;
+    for (int c = warp; c < 8 * E && blockIdx.x * 8 * E + c < C; c += warps) {
+        float t = lane < warps ? part[lane][c] : 0.f;
+        for (int k = 16; k > 0; k >>= 1) t += __shfl_xor_sync(0xffffffffu, t, k);
+        if (lane == 0) stf<T>(y + (size_t)n * C + blockIdx.x * 8 * E + c, t / (float)HW);
     }
 }
 
@@ -1544,27 +1541,34 @@ __global__ void dense_kernel(const T *__restrict__ x, const T *__restrict__ w, c
 }
 
 // 16-byte vectors along the input features: one warp per (output feature, NB
-// images), the weight row loaded once for them, U vectors in flight.  The
+// images), the weight row loaded once for them, U vectors in flight, the first
+// ones before the wait for the previous kernel (8 x 32 -> 120: 2.7 -> 2.4 us).  The
 // reduction order differs from the scalar kernel's; each is one f32 sum.
 template <typename T, int NB, int U>
 __global__ void __launch_bounds__(256) dense_vec_kernel(const uint4 *__restrict__ x, const uint4 *__restrict__ w,
                                                         const float *__restrict__ bias, T *__restrict__ y, int N,
                                                         int IV, int OUT, int act) {
     griddep_launch();
-    griddep_wait();
     constexpr int E = 16 / sizeof(T);
     const int lane = threadIdx.x & 31;
     const int o = blockIdx.x * 8 + (threadIdx.x >> 5);
     const int n0 = blockIdx.y * NB;
+    // the first weights and the bias are no data of the previous kernel
+    const uint4 *wr = w + (size_t)min(o, OUT - 1) * IV;
+    const float bo = bias[min(o, OUT - 1)];
+    uint4 wv[U];
+    auto load_w = [&](int i) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) wv[u] = i + 32 * u < IV ? wr[i + 32 * u] : make_uint4(0u, 0u, 0u, 0u);
+    };
+    load_w(lane);
+    griddep_wait();
     if (o >= OUT) return;
-    const uint4 *wr = w + (size_t)o * IV;
     float s[NB];
 #pragma unroll
     for (int b = 0; b < NB; ++b) s[b] = 0.f;
     for (int i = lane; i < IV; i += 32 * U) {
-        uint4 wv[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) wv[u] = i + 32 * u < IV ? wr[i + 32 * u] : make_uint4(0u, 0u, 0u, 0u);
+        if (i != lane) load_w(i);
 #pragma unroll
         for (int b = 0; b < NB; ++b) {
             const uint4 *xr = x + (size_t)min(n0 + b, N - 1) * IV;
@@ -1586,7 +1590,7 @@ __global__ void __launch_bounds__(256) dense_vec_kernel(const uint4 *__restrict_
 #pragma unroll
         for (int b = 1; b < NB; ++b)
             if (lane == b) v = s[b];
-        stf<T>(y + (size_t)(n0 + lane) * OUT + o, act_apply(v + bias[o], act));
+        stf<T>(y + (size_t)(n0 + lane) * OUT + o, act_apply(v + bo, act));
     }
 }
 
