@@ -665,17 +665,23 @@ __global__ void __launch_bounds__(256) q8_dense_kernel(const int8_t *__restrict_
                                                        TO *__restrict__ y, int N, int I, int O, int act,
                                                        Q8Scales q) {
     griddep_launch();
-    griddep_wait();
     const int lane = threadIdx.x & 31;
     const int o = blockIdx.x * 8 + (threadIdx.x >> 5);
+    // this feature's first weights and constants are no data of the previous kernel
+    const int8_t *wr = w + (int64_t)min(o, O - 1) * I;
+    const float so = ws[min(o, O - 1)], bo = bias[min(o, O - 1)];
+    int4 w0 = make_int4(0, 0, 0, 0);  // V = 16: the first 16 codes of this lane; V = 4: the first two words
+    if (V == 16 && lane * 16 < I) w0 = *reinterpret_cast<const int4 *>(wr + lane * 16);
+    if (V == 4 && lane * 4 < I) w0.x = *reinterpret_cast<const int *>(wr + lane * 4);
+    if (V == 4 && lane * 4 + 128 < I) w0.y = *reinterpret_cast<const int *>(wr + lane * 4 + 128);
+    griddep_wait();
     if (o >= O) return;
-    const int8_t *wr = w + (int64_t)o * I;
     for (int n0 = blockIdx.y * NB; n0 < N; n0 += gridDim.y * NB) {
         int acc[NB] = {};
         if (V == 16) {
             int i = lane * 16;
             for (; i < I; i += 512) {
-                const int4 wv = *reinterpret_cast<const int4 *>(wr + i);
+                const int4 wv = i < 512 ? w0 : *reinterpret_cast<const int4 *>(wr + i);
 #pragma unroll
                 for (int b = 0; b < NB; ++b) {
                     if (n0 + b >= N) break;
@@ -688,7 +694,7 @@ __global__ void __launch_bounds__(256) q8_dense_kernel(const int8_t *__restrict_
             }
         } else if (V == 4) {
             for (int i = lane * 4; i < I; i += 128) {
-                const int wv = *reinterpret_cast<const int *>(wr + i);
+                const int wv = i < 128 ? w0.x : i < 256 ? w0.y : *reinterpret_cast<const int *>(wr + i);
 #pragma unroll
                 for (int b = 0; b < NB; ++b)
                     if (n0 + b < N) acc[b] = dp4a(*reinterpret_cast<const int *>(x + (int64_t)(n0 + b) * I + i), wv, acc[b]);
@@ -709,7 +715,7 @@ __global__ void __launch_bounds__(256) q8_dense_kernel(const int8_t *__restrict_
 #pragma unroll
             for (int b = 1; b < NB; ++b)
                 if (lane == b) v = acc[b];
-            y[(int64_t)(n0 + lane) * O + o] = q8_out<TO>(q8_value(v, q.s_x, ws[o], bias[o], 0.0f, act), q.inv_out);
+            y[(int64_t)(n0 + lane) * O + o] = q8_out<TO>(q8_value(v, q.s_x, so, bo, 0.0f, act), q.inv_out);
         }
     }
 }
@@ -897,11 +903,15 @@ __global__ void __launch_bounds__(1024) q8_gap_nhwc_kernel(const int8_t *__restr
     int s[4] = {};
     if (c0 < C) {
         const int8_t *xn = x + (int64_t)blockIdx.y * HW * C + c0;
-#pragma unroll 4
-        for (int p = sl; p < HW; p += slices) {
-            const int q = *reinterpret_cast<const int *>(xn + (int64_t)p * C);
+        for (int p = sl; p < HW; p += 8 * slices) {  // eight loads in flight, the last ones too
+            int q[8];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) s[e] = dp4a(q, 1 << (8 * e), s[e]);
+            for (int k = 0; k < 8; ++k)
+                q[k] = p + k * slices < HW ? *reinterpret_cast<const int *>(xn + (int64_t)(p + k * slices) * C) : 0;
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) s[e] = dp4a(q[k], 1 << (8 * e), s[e]);
         }
     }
 #pragma unroll
@@ -915,11 +925,13 @@ __global__ void __launch_bounds__(1024) q8_gap_nhwc_kernel(const int8_t *__restr
         for (int e = 0; e < 4; ++e) part[warp][v * 4 + e] = s[e];
     }
     __syncthreads();
-    const int c = blockIdx.x * 32 + threadIdx.x;
-    if (threadIdx.x < 32 && c < C) {
-        int sum = 0;
-        for (int k = 0; k < (int)(blockDim.x >> 5); ++k) sum += part[k][threadIdx.x];
-        y[(int64_t)blockIdx.y * C + c] = q8_out<TO>(__fdiv_rn(__fmul_rn(__int2float_rn(sum), s_x), (float)HW), inv);
+    // a warp per channel of the block's 32: the warps' sums, one a lane
+    const int lane = threadIdx.x & 31, warps = blockDim.x >> 5;
+    for (int i = warp; i < 32 && (int)blockIdx.x * 32 + i < C; i += warps) {
+        const int sum = __reduce_add_sync(0xffffffffu, lane < warps ? part[lane][i] : 0);
+        if (lane == 0)
+            y[(int64_t)blockIdx.y * C + blockIdx.x * 32 + i] =
+                q8_out<TO>(__fdiv_rn(__fmul_rn(__int2float_rn(sum), s_x), (float)HW), inv);
     }
 }
 
