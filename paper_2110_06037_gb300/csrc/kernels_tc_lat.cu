@@ -212,8 +212,10 @@ __global__ void __launch_bounds__(LAT_THREADS, 2)
         } else {
             tc_fence_after();
             const uint32_t ta = tmem + ((uint32_t)(warp * 32) << 16);
+            // (rolled: a CTA runs it once, so that straight-line code waits for its
+            // instructions; ResNet-50 at batch 32: 653 -> 639 us)
             with_act2<T>(p.act, [&](auto fin) {
-#pragma unroll
+#pragma unroll 1
                 for (int c = 0; c < BN / 32; ++c) {
                     const int k0 = w.n0 + 32 * c;
                     if (k0 >= p.K) break;
