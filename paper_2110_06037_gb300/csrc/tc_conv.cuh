@@ -766,7 +766,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                     continue;
                 }
             }
-#pragma unroll
+#pragma unroll 1
             for (int cj = 0; cj < CPH; ++cj) {
                 const int ci = cbase + cj;
                 const int k0 = w.n0 + 64 * ci;
@@ -793,27 +793,10 @@ __global__ void __launch_bounds__(THREADS, 1)
                         ++res_landed;
                     }
                     ++nchunk;
-                    uint32_t v[64];
-                    __syncwarp();
-                    tmem_ld64(taddr, v);
-                    if (CSK == 2) {
-                        // add CTA 1's partial of the same rows and channels, then
-                        // hand its exchange block back
-                        if (!mbar_wait_cluster(&xfull_bar[warp - 2], xph, p.wait_limit)) {
-                            if (lane == 0) atomicOr(p.err, ERR_EPI_WAIT);
-                            set_abort();
-                        }
-                        const uint8_t *xr = xbuf + (warp - 2) * XBLK_BYTES + lane * 256;
-#pragma unroll
-                        for (int j = 0; j < 16; ++j) {
-                            const uint4 x = *reinterpret_cast<const uint4 *>(xr + ((j ^ (lane & 15)) << 4));
-                            v[4 * j] = __float_as_uint(__uint_as_float(v[4 * j]) + __uint_as_float(x.x));
-                            v[4 * j + 1] = __float_as_uint(__uint_as_float(v[4 * j + 1]) + __uint_as_float(x.y));
-                            v[4 * j + 2] = __float_as_uint(__uint_as_float(v[4 * j + 2]) + __uint_as_float(x.z));
-                            v[4 * j + 3] = __float_as_uint(__uint_as_float(v[4 * j + 3]) + __uint_as_float(x.w));
-                        }
-                        mbar_arrive_cluster(mapa(su32(&xfree_bar[warp - 2]), 1u));
-                        xph ^= 1u;
+                    const uint8_t *xr = xbuf + (warp - 2) * XBLK_BYTES + lane * 256;
+                    if (CSK == 2 && !mbar_wait_cluster(&xfull_bar[warp - 2], xph, p.wait_limit)) {
+                        if (lane == 0) atomicOr(p.err, ERR_EPI_WAIT);
+                        set_abort();
                     }
                     if (NBUF == 2) {  // the next chunk's residual (all of this loop's conditions, one chunk on)
                         if (cj + 1 < CPH && k0 + 64 < p.K) {
@@ -824,16 +807,39 @@ __global__ void __launch_bounds__(THREADS, 1)
                             primed = true;
                         }
                     }
+                    __syncwarp();
                     // every 8 channels go to their 16-byte piece of the row as soon as
-                    // they are computed, in place of the residual's piece
+                    // they are computed, in place of the residual's piece (32 columns
+                    // at a time, rolled: straight-line code waits for its instructions
+                    // the few times that a CTA runs it)
                     with_act2<T>(p.act, [&](auto fin) {
+#pragma unroll 1
+                        for (int h = 0; h < 2; ++h) {
+                            uint32_t v[32];
+                            tmem_ld32(taddr + 32 * h, v);
+                            if (CSK == 2) {  // CTA 1's partial of the same rows and channels
 #pragma unroll
-                        for (int q = 0; q < 8; ++q) {
-                            uint4 *piece = reinterpret_cast<uint4 *>(buf + lane * 128 + ((q ^ (lane & 7)) << 4));
-                            *piece = finish8<T>(v + 8 * q, bias4(16 * cj + 2 * q), bias4(16 * cj + 2 * q + 1),
-                                                has_res, has_res ? *piece : make_uint4(0u, 0u, 0u, 0u), fin);
+                                for (int j = 0; j < 8; ++j) {
+                                    const uint4 x = *reinterpret_cast<const uint4 *>(xr + (((8 * h + j) ^ (lane & 15)) << 4));
+                                    v[4 * j] = __float_as_uint(__uint_as_float(v[4 * j]) + __uint_as_float(x.x));
+                                    v[4 * j + 1] = __float_as_uint(__uint_as_float(v[4 * j + 1]) + __uint_as_float(x.y));
+                                    v[4 * j + 2] = __float_as_uint(__uint_as_float(v[4 * j + 2]) + __uint_as_float(x.z));
+                                    v[4 * j + 3] = __float_as_uint(__uint_as_float(v[4 * j + 3]) + __uint_as_float(x.w));
+                                }
+                            }
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) {
+                                const int q = 4 * h + i;
+                                uint4 *piece = reinterpret_cast<uint4 *>(buf + lane * 128 + ((q ^ (lane & 7)) << 4));
+                                *piece = finish8<T>(v + 8 * i, bias4(16 * cj + 2 * q), bias4(16 * cj + 2 * q + 1), has_res,
+                                                    has_res ? *piece : make_uint4(0u, 0u, 0u, 0u), fin);
+                            }
                         }
                     });
+                    if (CSK == 2) {  // hand the exchange block back
+                        mbar_arrive_cluster(mapa(su32(&xfree_bar[warp - 2]), 1u));
+                        xph ^= 1u;
+                    }
                     fence_proxy_async_smem();
                     __syncwarp();
                     if (!p.y_nchw) {
