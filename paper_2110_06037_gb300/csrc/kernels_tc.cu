@@ -124,8 +124,8 @@ static std::vector<Config> configs(const Layer &l, const Shape &in, sn_schema s,
             cf.BN = bn;
             cf.G = 1;
             push_splits(cf, mtiles);
-            // two channel blocks per box: a TMA box costs the SM ~400 cycles
-            // whatever its size (up to 32 KB), so fewer, larger boxes
+            // two channel blocks per box: a TMA box costs its issuing thread ~350
+            // cycles whatever its size (up to 32 KB), so fewer, larger boxes
             if (bn <= 128 && c.c_in % 128 == 0) {
                 cf.KB = 2;
                 push_splits(cf, mtiles);
@@ -778,7 +778,7 @@ cudaError_t conv_im2col_tc_stage(const LaunchArgs &a, int stage) {
 // that (pixel stride 32 B, rows of 64 values), with a fifth axis over the
 // rows of taps (stride one X row), so one TMA box brings all A = 2 or 4 rows
 // of taps of a 128-pixel tile (A x 16 KB) and the implicit-GEMM kernel runs
-// one pipeline stage per tile: a TMA box costs about the same whatever its
+// one pipeline stage per tile: a TMA box costs its issuing thread the same whatever its
 // size, so few large boxes keep the tensor cores fed.
 // ---------------------------------------------------------------------------
 namespace {

@@ -2,8 +2,8 @@
 // maps): one tile per cluster, the tile's K steps split among the cluster's CTAs.
 //
 // What bounds such a layer is not the tensor core but a chain of latencies: the
-// dependency release, the copies of all its K steps through one SM (about 400
-// cycles a box), the MMAs, the drain.  So
+// dependency release, the copies of all its K steps through one SM (about 350
+// cycles a box for the thread that issues it), the MMAs, the drain.  So
 //   * a cluster of NCL CTAs takes the 128-pixel x BN-channel tile, each CTA
 //     1/NCL of the K steps (1 to 5 boxes of A instead of 9 to 36), and the
 //     partial sums meet on chip: every CTA sends each peer the columns that the
