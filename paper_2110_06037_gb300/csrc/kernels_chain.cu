@@ -211,7 +211,6 @@ __global__ void __launch_bounds__(THREADS, 1) conv_chain_kernel(const ChainArgs 
     __shared__ volatile int abort_sh;
     __shared__ int issued_sh[2], consumed_sh, last_sh;
 
-    griddep_launch();
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint8_t *stg = smem + CH_STAGES * CH_SLOT;  // epilogue staging: one 4 KB block per warp
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
@@ -245,6 +244,7 @@ __global__ void __launch_bounds__(THREADS, 1) conv_chain_kernel(const ChainArgs 
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tmem_sh;
+    griddep_launch();  // (behind the allocation: see tmem_alloc)
 
     if (warp == 11) {  // ---------------- the MMA issuer's waiter
         int l = 0, lt = 0, s = 0;

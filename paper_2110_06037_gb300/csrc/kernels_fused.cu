@@ -58,7 +58,6 @@ __global__ void __launch_bounds__(NT, 512 / NT)
     __shared__ volatile int abort_sh;
     __shared__ int issued_sh, done_sh;
 
-    griddep_launch();
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const uint32_t tile_bytes = (uint32_t)p.cblocks * (BM * BK * 2);  // one 128-pixel tile of A
     uint8_t *sb = smem + MT * tile_bytes;
@@ -97,6 +96,7 @@ __global__ void __launch_bounds__(NT, 512 / NT)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tmem_sh;
+    griddep_launch();  // (behind the allocation: see tmem_alloc)
     if (threadIdx.x == 0) {
         mbar_expect_tx(&b_bar, (uint32_t)p.cblocks * (64 * BK * 2));
         for (int cb = 0; cb < p.cblocks; ++cb) tma_2d<1>(su32(sb + cb * (64 * BK * 2)), &mB, su32(&b_bar), cb * BK, e0);
@@ -270,8 +270,7 @@ __global__ void __launch_bounds__(NT, 512 / NT)
 }
 
 // at least a third of an SM, so that no more than two CTAs share one: each
-// holds at most half of its tensor memory, and an allocation that waited for a
-// CTA of the next kernel, itself waiting for this one, would never return
+// holds at most half of its tensor memory, so neither waits for the other's
 static size_t smem_of(int MT, int cblocks) {
     return std::max<size_t>((size_t)MT * cblocks * (BM * BK * 2) + (size_t)cblocks * (64 * BK * 2) + 1024, 80 * 1024);
 }

@@ -64,7 +64,6 @@ __global__ void __launch_bounds__(LAT_THREADS, 2)
     __shared__ int issued_sh[LAT_STAGES], consumed_sh;
     __shared__ __align__(16) float bias_sh[BN];  // like all weights not written by the previous kernel
 
-    griddep_launch();
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     // partial sums from the peers: [rank][CW / 4][128 rows] float4
     float4 *xch = reinterpret_cast<float4 *>(smem + LAT_STAGES * STAGE);
@@ -101,6 +100,7 @@ __global__ void __launch_bounds__(LAT_THREADS, 2)
     else __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tmem_sh;
+    griddep_launch();  // (behind the allocation: see tmem_alloc)
     if (warp > 4) {
         if (lane == 0) {  // ---------------- producer of stage s: the K steps it0 + s, it0 + s + LAT_STAGES, ...
             const int s = warp - 5;
@@ -364,8 +364,8 @@ __global__ void __launch_bounds__(LAT_THREADS, 2)
 template <typename T, int BN, int NCL>
 static cudaError_t launch_lat_t(const CUtensorMap *mA, const CUtensorMap &mB, const CUtensorMap &mY, const Params &p,
                                 cudaStream_t st) {
-    // (at least a third of an SM: no more than two CTAs share one, so tensor
-    // memory never runs out while a CTA of the next kernel waits for this one)
+    // (at least a third of an SM: no more than two CTAs share one, so that a third
+    // does not wait for tensor memory behind them)
     constexpr size_t need = (size_t)LAT_STAGES * (BM + BN) * BK * 2 + (NCL > 1 ? (size_t)BM * BN * 4 : 0) + 1024;
     constexpr size_t smem = need > 80 * 1024 ? need : 80 * 1024;
     auto kern = conv_tc_lat_kernel<T, BN, NCL>;

@@ -127,7 +127,6 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1)
     __shared__ volatile int abort_sh;
     __shared__ int issued_sh, consumed_sh;
 
-    griddep_launch();
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     const int total = p.mtiles * p.ntiles;
@@ -155,6 +154,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tmem_sh;
+    griddep_launch();  // (behind the allocation: see tmem_alloc)
     // tile t: output channels n0.., pixel box at (q0, p0, i0)
     auto tile = [&](int t, int &n0, int &q0, int &p0, int &i0) {
         const int mt = (int)fdiv((uint32_t)t, p.fd_nt);

@@ -185,7 +185,12 @@ __device__ __forceinline__ void prefetch_l1(const void *p) {
 }
 
 // TMEM allocation; G = 2 allocates the same columns in both CTAs of the pair
-// (one warp of each CTA executes it)
+// (one warp of each CTA executes it).  It waits without a limit while other CTAs
+// of the SM hold the columns, so no such CTA may in turn wait for this one: a
+// kernel calls griddep_launch() only behind the barrier that follows its
+// allocation.  The next kernel's CTAs then start when every CTA of this one has
+// its columns, whatever the two take of an SM, and a CTA that holds columns
+// waits only for kernels whose CTAs hold theirs.
 template <int G>
 __device__ __forceinline__ void tmem_alloc(uint32_t *dst, uint32_t ncols) {
     if constexpr (G == 2) {

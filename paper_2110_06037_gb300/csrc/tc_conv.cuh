@@ -109,7 +109,6 @@ __global__ void __launch_bounds__(THREADS, 1)
     __shared__ volatile int abort_sh;
     __shared__ int issued_sh[4], consumed_sh;
 
-    griddep_launch();
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint8_t *bst = smem + STAGES * STAGE_BYTES;  // weight-stationary B (BST), 1024-B aligned
     uint8_t *stg = bst + (BST ? p.bst_bytes : 0);  // epilogue staging: one block per warp, 1024-B aligned
@@ -210,6 +209,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tmem_sh;
+    griddep_launch();  // (behind the allocation: see tmem_alloc)
     // Everything up to each role's griddep_wait() overlaps the previous
     // kernel's tail: the producers wait before their first TMA load, the
     // epilogue warps before their first residual load or store (the MMA warp
