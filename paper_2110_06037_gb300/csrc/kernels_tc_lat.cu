@@ -271,6 +271,13 @@ __global__ void __launch_bounds__(LAT_THREADS, 2)
         if (!__all_sync(0xffffffffu, ok)) {
             if (lane == 0) atomicOr(p.err, ERR_ACC_WAIT);
             abort_sh = 1;
+            // the peers count on these bytes, and may leave only when they are there
+#pragma unroll 1
+            for (int i = 0; i < (NCL - 1) * (CW / 4); ++i) {
+                const uint32_t dst = (rank + 1 + (uint32_t)(i / (CW / 4))) % NCL;
+                const uint32_t at = su32(xch + ((int)rank * (CW / 4) + i % (CW / 4)) * BM + row);
+                st_async_v4(mapa(at, dst), mapa(su32(&x_bar[warp]), dst), 0u, 0u, 0u, 0u);
+            }
         } else {
             tc_fence_after();
             const uint32_t ta = tmem + ((uint32_t)(warp * 32) << 16);
@@ -337,9 +344,12 @@ __global__ void __launch_bounds__(LAT_THREADS, 2)
     __syncthreads();
     if (warp == 4) {
         if (abort_sh && lane == 0) {
-            // let this CTA's copies and MMAs land before its memory goes away
-            // (one deadline for the whole drain)
+            // let this CTA's copies and MMAs and the peers' sums land before its
+            // memory goes away (one deadline for the whole drain)
             const long long t0 = clock64();
+            for (int i = 0; i < 4 && NCL > 1; ++i)
+                while (!mbar_try(&x_bar[i], 0u) && clock64() - t0 < WAIT_LIMIT) {
+                }
             for (int s = 0; s < LAT_STAGES; ++s)
                 if (issued_sh[s] > 0)
                     while (!mbar_try(&full_bar[s], (uint32_t)(issued_sh[s] - 1) & 1u) && clock64() - t0 < WAIT_LIMIT) {
@@ -355,9 +365,11 @@ __global__ void __launch_bounds__(LAT_THREADS, 2)
         tc_fence_after();
         tmem_dealloc<1>(tmem, BN);
     }
-    // no CTA leaves while a peer may still write into its shared memory (relaxed:
-    // nothing read after it depends on it; a releasing arrive would wait for
-    // this CTA's global stores to be performed, ~1800 cycles)
+    // What the peers send has landed by now: the epilogue warps, or the drain
+    // above, have waited for x_bar, and a CTA whose own sums are missing sends
+    // zeros.  The barrier is for a CTA whose drain ran out.  (Relaxed: nothing read
+    // after it depends on it; a releasing arrive would wait for this CTA's global
+    // stores to be performed, ~1800 cycles.)
     if (NCL > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
 }
 

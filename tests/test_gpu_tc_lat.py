@@ -91,3 +91,28 @@ def test_expired_wait_in_a_cluster_reports_timeout_and_recovers(size):
     y1 = g.run(xd)
     torch.cuda.synchronize()
     assert torch.equal(y0, y1)
+
+
+@pytest.mark.parametrize("size", [2, 8])
+def test_expired_wait_in_every_cta_of_a_cluster(size):
+    """Every CTA gives up with its peers' sums under way, many times in a row;
+    the next run has its values."""
+    import torch
+    x, layers = synth.single_conv(2, 14, 512, 128, 1, 1)
+    sch = ("f16", "nhwc")
+    g = build_graph(layers, x.shape, sch, sch, [sch])
+    cands, t = lat(g, 1)
+    c = [c for c in cands if f"cluster={size} " in g.candidate_desc(c)][0]
+    g.set_path(path(t, 1, c))
+    g.set_option(SN_OPT_CHECK, 1)
+    xd = to_device(x, sch)
+    y0 = g.run(xd).clone()
+    for _ in range(20):
+        g.set_option(SN_OPT_WAIT_LIMIT, 1)
+        with pytest.raises(SnError) as e:
+            g.run(xd)
+        assert e.value.status == _sn.SN_ETIMEOUT
+    g.set_option(SN_OPT_WAIT_LIMIT, 0)
+    y1 = g.run(xd)
+    torch.cuda.synchronize()
+    assert torch.equal(y0, y1)

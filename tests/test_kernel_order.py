@@ -34,3 +34,14 @@ def test_no_kernel_lets_its_successor_start_before_it_holds_its_tensor_memory():
             seen[name] = len(launches) == 1 and launches[0] > barrier
     assert {"conv_tc_kernel", "conv_tc_lat_kernel", "conv_split_kernel", "expand_dw_kernel", "conv_chain_kernel"} <= set(seen)
     assert all(seen.values()), seen
+
+
+def test_a_cluster_tile_that_gives_up_still_sends_and_receives_its_sums():
+    """A peer's st.async completes only through the mbarrier of the CTA that it
+    writes into: a CTA may leave once x_bar has counted every byte, on the error
+    path too, and so every CTA has to send, on the error path too."""
+    body = dict(kernels())["conv_tc_lat_kernel"]
+    drain = body[body.index("if (abort_sh && lane == 0)"):]
+    assert "x_bar" in drain[:drain.index("tmem_dealloc")]
+    failed = body[body.rindex("ERR_ACC_WAIT"):]  # in the epilogue of a cluster, the last of the roles
+    assert "st_async_v4" in failed[:failed.index("} else {")]
