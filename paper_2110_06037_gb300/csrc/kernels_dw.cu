@@ -371,6 +371,19 @@ bool dw3_ring_applies(const LaunchArgs &a, const ConvDims &d) {
     return (int64_t)d.N * d.C / (16 / es) * d.P < ((int64_t)1 << 30);
 }
 
+// The depthwise kernels add in one order (bias, rows, columns), the fp16 3x3 ones
+// in fp16, but for the shared-memory halo kernel, which adds in fp32: variant 1
+// where the rows do not fit the ring.
+bool dw_sums_as_window(const Layer &l, const Shape &in, sn_schema s, int32_t v) {
+    const sn_conv_params &c = l.conv;
+    if (v != 1 || s.dtype != SN_F16 || c.kh != 3 || c.kw != 3) return true;
+    const ConvDims d{(int32_t)in.n, (int32_t)in.c, (int32_t)in.h, (int32_t)in.w, c.c_out, (int32_t)l.out.h,
+                     (int32_t)l.out.w, 3, 3, c.sh, c.sw, c.ph, c.pw, c.dh, c.dw, c.groups, c.act};
+    LaunchArgs a{};  // (aligned buffers)
+    a.schema = s;
+    return dw3_ring_applies(a, d) && plan_ring(d, 2, true).score >= 0;
+}
+
 cudaError_t dw3_nhwc_ring(const LaunchArgs &a, const ConvDims &d) {
     if (!dw3_ring_applies(a, d)) return cudaErrorNotSupported;
     const int es = dtype_size(a.schema.dtype);

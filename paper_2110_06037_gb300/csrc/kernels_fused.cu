@@ -9,6 +9,9 @@
 // over the staged input; the depthwise taps read them from there and only the
 // depthwise result goes to memory.  Every value is what the two layers compute
 // one after the other: the same products, the same order, the same roundings.
+// (A cluster variant of the convolution adds up its CTAs' sums: their ranges of K
+// steps get an accumulator each here.  Variants that group the steps otherwise
+// are not paired.)
 // What it saves is a launch and its dependency (about 3 of 8 us at batch 1) and
 // the expanded map's trip through memory; what it costs is the KS - 1 halo rows
 // of every band, expanded twice.  MobileNetV2
@@ -28,10 +31,11 @@ namespace fused {
 using namespace tc;
 
 constexpr int MAX_MT = 4;
+constexpr int MAX_COLS = 256;  // of tensor memory: half of an SM's
 
 struct FParams {
     int32_t H, W, C, E, P, Q, ph, pw;
-    int32_t PB, cblocks, act_e, act_d;
+    int32_t PB, cblocks, parts, act_e, act_d;
     FastDiv fd_qb;  // column blocks of an output row
     const float *be, *bd;
     const void *wd;  // depthwise weights [KS * KS][E]
@@ -121,12 +125,15 @@ __global__ void __launch_bounds__(NT, 512 / NT)
             ok = mbar_wait(&full_bar[mt], 0u, p.wait_limit);
             if (!ok) break;
             tc_fence_after();
-            for (int cb = 0; cb < p.cblocks; ++cb) {
-                const int ks = min(BK / 16, (p.C - cb * BK + 15) / 16);  // 16-value steps that hold channels
-                for (int k = 0; k < ks; ++k)
-                    umma<1>(tmem + (uint32_t)(mt * 64), da0 + (uint64_t)((mt * tile_bytes + cb * (BM * BK * 2)) >> 4) + 2 * k,
-                            db0 + (uint64_t)((cb * (64 * BK * 2)) >> 4) + 2 * k, idesc, (cb > 0 || k > 0) ? 1u : 0u);
-            }
+            int cb = 0;
+            for (int r = 0; r < p.parts; ++r)
+                for (const int cb0 = cb, cb1 = p.cblocks * (r + 1) / p.parts; cb < cb1; ++cb) {
+                    const int ks = min(BK / 16, (p.C - cb * BK + 15) / 16);  // 16-value steps that hold channels
+                    for (int k = 0; k < ks; ++k)
+                        umma<1>(tmem + (uint32_t)((mt * p.parts + r) * 64),
+                                da0 + (uint64_t)((mt * tile_bytes + cb * (BM * BK * 2)) >> 4) + 2 * k,
+                                db0 + (uint64_t)((cb * (64 * BK * 2)) >> 4) + 2 * k, idesc, (cb > cb0 || k > 0) ? 1u : 0u);
+                }
             umma_commit<1>(&accf_bar[mt]);
         }
         if (!ok) {
@@ -150,7 +157,15 @@ __global__ void __launch_bounds__(NT, 512 / NT)
         tc_fence_after();
         __syncwarp();
         uint32_t v[32];
-        tmem_ld32(tmem + ((uint32_t)(g4 * 32) << 16) + (uint32_t)(mt * 64 + half * 32), v);
+        const uint32_t ta = tmem + ((uint32_t)(g4 * 32) << 16) + (uint32_t)(mt * p.parts * 64 + half * 32);
+        tmem_ld32(ta, v);
+        for (int r = 1; r < p.parts; ++r) {  // (from zero, as the cluster's CTAs add)
+            uint32_t x[32];
+            tmem_ld32(ta + (uint32_t)(r * 64), x);
+#pragma unroll
+            for (int e = 0; e < 32; ++e)
+                v[e] = __float_as_uint((r == 1 ? 0.f + __uint_as_float(v[e]) : __uint_as_float(v[e])) + __uint_as_float(x[e]));
+        }
         const int i = g4 * 32 + lane;
         uint8_t *row = mid(mt * BM + i);
         with_act2<T>(p.act_e, [&](auto fin) {
@@ -285,9 +300,10 @@ static size_t smem_of(int MT, int cblocks) {
 // the two layers (a block with its projection: 32 x 28 x 28, 32 -> 192: 17.8 ->
 // 15.7 us and 14 x 14, 96 -> 576 at batch 1: 10.7 -> 8.9 in one wave; 32 x 56 x
 // 56, 24 -> 144: 43.3 -> 47.5 and 32 x 112 x 112, 16 -> 96: 61 -> 84 in more)
-ExpandDwPlan expand_dw_plan(const Layer &conv, const Shape &in, const Layer &dw, sn_schema s) {
+ExpandDwPlan expand_dw_plan(const Layer &conv, const Shape &in, int32_t conv_variant, const Layer &dw, int32_t dw_variant,
+                            sn_schema s) {
     using namespace fused;
-    const ExpandDwPlan none{0, 0, 0};
+    const ExpandDwPlan none{0, 0, 0, 0};
     const sn_conv_params &c = conv.conv, &d = dw.conv;
     if (conv.type != SN_L_CONV2 || dw.type != SN_L_DWCONV2 || s.layout != SN_NHWC || (s.dtype != SN_F16 && s.dtype != SN_BF16))
         return none;
@@ -295,12 +311,14 @@ ExpandDwPlan expand_dw_plan(const Layer &conv, const Shape &in, const Layer &dw,
     if (d.c_in != c.c_out || d.kh != d.kw || (d.kh != 3 && d.kh != 5) || d.sh != d.sw || (d.sh != 1 && d.sh != 2) || d.dh != 1 ||
         d.dw != 1)
         return none;
+    const int32_t parts = conv_tc_sum_parts(conv, in, s, conv_variant);
+    if (parts < 1 || !dw_sums_as_window(dw, conv.out, s, dw_variant)) return none;
     const int64_t N = in.n, H = in.h, W = in.w, P = dw.out.h, slices = (c.c_out + 63) / 64;
     const int cblocks = (c.c_in + BK - 1) / BK;
     if (N > 65535 || P > 65535 || N * H * W >= ((int64_t)1 << 31) - BM * MAX_MT) return none;
     for (int MT = 1; MT <= MAX_MT; ++MT) {
         const size_t sm = smem_of(MT, cblocks);
-        if (sm > 220 * 1024) break;
+        if (sm > 220 * 1024 || MT * parts * 64 > MAX_COLS) break;
         const int64_t rows = std::min<int64_t>(MT * BM / W, H);  // input rows that fit
         int64_t PB = rows >= H ? P : rows < d.kh ? 0 : (rows - d.kh) / d.sh + 1;
         if (PB < 1) continue;
@@ -308,7 +326,7 @@ ExpandDwPlan expand_dw_plan(const Layer &conv, const Shape &in, const Layer &dw,
         const int64_t bands = (P + PB - 1) / PB;
         PB = (P + bands - 1) / bands;
         const int64_t grid = slices * bands * N, slots = 152 * (sm <= 110 * 1024 ? 2 : 1);
-        if (grid <= slots) return ExpandDwPlan{MT, (int32_t)PB, (int32_t)bands};
+        if (grid <= slots) return ExpandDwPlan{MT, (int32_t)PB, (int32_t)bands, parts};
     }
     return none;
 }
@@ -317,11 +335,12 @@ cudaError_t expand_dw(const LaunchArgs &a, const LaunchArgs &b, const ExpandDwPl
     using namespace fused;
     const Layer &conv = *a.layer, &dw = *b.layer;
     const Shape &in = a.in_shapes[0];
-    if (pl.MT < 1 || (uintptr_t)b.out % 16 || (uintptr_t)b.wt % 16) return cudaErrorInvalidValue;
+    if (pl.MT < 1 || pl.parts < 1 || pl.MT * pl.parts * 64 > MAX_COLS || (uintptr_t)b.out % 16 || (uintptr_t)b.wt % 16) return cudaErrorInvalidValue;
     FParams p{};
     p.H = (int)in.h, p.W = (int)in.w, p.C = (int)in.c, p.E = conv.conv.c_out;
     p.P = (int)dw.out.h, p.Q = (int)dw.out.w, p.ph = dw.conv.ph, p.pw = dw.conv.pw;
     p.PB = pl.PB;
+    p.parts = pl.parts;
     p.cblocks = (p.C + BK - 1) / BK;
     p.act_e = conv.conv.act, p.act_d = dw.conv.act;
     p.fd_qb = make_fastdiv((uint32_t)((p.Q + 3) / 4));
@@ -343,7 +362,8 @@ cudaError_t expand_dw(const LaunchArgs &a, const LaunchArgs &b, const ExpandDwPl
         if (!tma_encode(&mB, dt, 2, a.wt, dims, str, box, CU_TENSOR_MAP_SWIZZLE_128B)) return cudaErrorInvalidValue;
     }
     const size_t smem = smem_of(pl.MT, p.cblocks);
-    const uint32_t cols = pl.MT == 1 ? 64u : pl.MT == 2 ? 128u : 256u;
+    uint32_t cols = 64;  // a power of two
+    while (cols < (uint32_t)(pl.MT * pl.parts * 64)) cols *= 2;
     const dim3 grid((unsigned)((p.E + 63) / 64), (unsigned)pl.bands, (unsigned)in.n);
     const bool big = (int64_t)grid.x * grid.y * grid.z > num_sms();  // two CTAs share an SM
     auto go = [&](auto kern) -> cudaError_t {

@@ -346,6 +346,16 @@ std::vector<char> conv_tc_nchw_ok(const Layer &l, const Shape &in, sn_schema s, 
     return ok;
 }
 
+// the fp32 sums that variant v adds up, in order, for an output: the K steps in
+// equal ranges, one per CTA of a cluster; 0 for the variants that group them
+// otherwise (through memory, in pairs of CTAs or by SM)
+int32_t conv_tc_sum_parts(const Layer &l, const Shape &in, sn_schema s, int32_t v) {
+    const std::vector<tc::Config> cfgs = tc::configs(l, in, s);
+    if (v < 0 || v >= (int)cfgs.size()) return 0;
+    const tc::Config &c = cfgs[v];
+    return c.lat ? c.lat : c.ksplit == 1 && c.csk == 1 && !c.sk ? 1 : 0;
+}
+
 size_t conv_tc_ws(const Layer &l, const Shape &in, sn_schema s, int32_t v, int32_t a_blocks, bool odd) {
     const std::vector<tc::Config> cfgs = tc::configs(l, in, s, a_blocks, odd);
     if (v < 0 || v >= (int)cfgs.size()) return 0;

@@ -62,7 +62,8 @@ sn_status ensure_tile_counts(Graph *g, cudaStream_t st) {
 // Pairs of plan ops that one launch can run: a 1x1 stride-1 convolution on the
 // tensor-core routine and the depthwise convolution next in the plan that alone
 // reads its (graph-owned) output, both in one 16-bit NHWC schema.  The values
-// are those of the two launches, so the selected path and its routines stay.
+// are those of the two launches of the selected variants (expand_dw_plan leaves
+// out those whose sums it cannot form), so the path and its routines stay.
 bool paired(const Graph *g, size_t q) { return q < g->op_pair.size() && g->op_pair[q]; }
 
 static void find_pairs(Graph *g) {
@@ -81,7 +82,8 @@ static void find_pairs(Graph *g) {
             for (int32_t s : op.in_slots) readers += s == a.out_slot;
         const Layer &la = g->layers[a.layer];
         if (readers == 1 && la.inputs.size() == 1 &&
-            k::expand_dw_plan(la, g->layers[la.inputs[0]].out, g->layers[b.layer], g->schemas[ca.schema]).MT > 0)
+            k::expand_dw_plan(la, g->layers[la.inputs[0]].out, ca.variant, g->layers[b.layer], cb.variant,
+                              g->schemas[ca.schema]).MT > 0)
             g->op_pair[q] = 1;
     }
 }
@@ -418,7 +420,8 @@ static sn_status launch_pair(Graph *g, size_t q, const IoPtrs &io, cudaStream_t 
         const sn_status rc = launch_op(g, g->plan[q], io, st);
         return rc != SN_OK ? rc : launch_op(g, g->plan[q + 1], io, st);
     }
-    const cudaError_t e = k::expand_dw(a, b, k::expand_dw_plan(*a.layer, a.in_shapes[0], *b.layer, a.schema));
+    const cudaError_t e =
+        k::expand_dw(a, b, k::expand_dw_plan(*a.layer, a.in_shapes[0], a.variant, *b.layer, b.variant, a.schema));
     if (e != cudaSuccess) return fail(SN_ECUDA, std::string("expand + depthwise: ") + cudaGetErrorString(e));
     return SN_OK;
 }

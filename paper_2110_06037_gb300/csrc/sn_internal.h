@@ -363,6 +363,7 @@ size_t conv_tc_ws(const Layer &l, const Shape &in, sn_schema s, int32_t v, int32
 size_t dense_tc_ws(const Layer &l, const Shape &in, sn_schema s, int32_t v);
 const char *conv_tc_variant_name(int32_t v);
 std::vector<char> conv_tc_nchw_ok(const Layer &l, const Shape &in, sn_schema s, bool odd = false);  // per variant
+int32_t conv_tc_sum_parts(const Layer &l, const Shape &in, sn_schema s, int32_t v);
 std::string conv_tc_config_desc(const Layer &l, const Shape &in, sn_schema s, int32_t v, bool odd = false);
 // chained launches of consecutive tensor-core convolutions
 bool conv_tc_chain_shape(const Layer &l, const Shape &in, sn_schema s, int32_t v, bool *implicit, int *bn, int *kb,
@@ -390,13 +391,16 @@ size_t split_weight_bytes(int64_t K, int64_t C, int64_t RS, int dt);
 cudaError_t weight_split(const float *w_kcrs, void *out, int dt, int64_t K, int64_t C, int64_t RS, cudaStream_t st);
 cudaError_t conv_split(const LaunchArgs &a, int32_t v);
 // a pointwise convolution and the depthwise convolution that alone reads it in
-// one launch: pixel tiles per CTA (0: not this pair), output rows per band, bands
+// one launch: pixel tiles per CTA (0: not this pair), output rows per band,
+// bands, partial sums per expanded value (those of the convolution's variant)
 struct ExpandDwPlan {
-    int32_t MT, PB, bands;
+    int32_t MT, PB, bands, parts;
 };
-ExpandDwPlan expand_dw_plan(const Layer &conv, const Shape &in, const Layer &dw, sn_schema s);
+ExpandDwPlan expand_dw_plan(const Layer &conv, const Shape &in, int32_t conv_variant, const Layer &dw, int32_t dw_variant,
+                            sn_schema s);
 cudaError_t expand_dw(const LaunchArgs &conv, const LaunchArgs &dw, const ExpandDwPlan &pl);
 cudaError_t dwconv(const LaunchArgs &a);
+bool dw_sums_as_window(const Layer &l, const Shape &in, sn_schema s, int32_t v);  // NHWC: variant v's sums are the window kernel's
 bool dw3_band_applies(const Layer &l, const Shape &in, sn_schema s);  // NHWC small-map depthwise kernel
 cudaError_t maxpool(const LaunchArgs &a);
 cudaError_t gap(const LaunchArgs &a);

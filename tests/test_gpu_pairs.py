@@ -130,3 +130,42 @@ def test_larger_layers_stay_two_launches():
     x = np.zeros((64, 16, 56, 56), np.float32)
     g = graph(layers, x, sch)
     assert g.plan_stats() == (2, 2)
+
+
+@pytest.mark.parametrize("case", [(1, 96, 14, 14, 72, 3, 1), (2, 160, 7, 7, 200, 5, 1), (1, 200, 9, 11, 136, 3, 2),
+                                  (1, 512, 7, 7, 256, 3, 1), (1, 16, 1, 300, 24, 3, 1)])
+@pytest.mark.parametrize("dt", ["f16", "bf16"])
+def test_pair_equals_two_launches_of_any_variants(case, dt):
+    """Whatever variants the path selected: clusters group the K steps among their
+    CTAs, and so does the pair; variants that group them otherwise, and the fp16
+    3x3 depthwise kernel that adds in fp32 (wide rows), stay two launches."""
+    import torch
+    N, C, H, W, E, k, s = case
+    sch = (dt, "nhwc")
+    layers = weights([dict(synth.conv(C, E, 1, act="relu6"), inputs=[-1]),
+                      dict(synth.dwconv(E, k, s, act="hswish"), inputs=[0])], zlib.crc32(repr(case).encode()))
+    x = np.random.default_rng(4).standard_normal((N, C, H, W)).astype(np.float32)
+    g = build_graph(layers, x.shape, sch, sch, [sch])
+    t = g.cost_table()
+    xd = to_device(x, sch)
+    tc = [int(c) for c in np.flatnonzero(t["layer"] == 1) if routine_name(int(t["routine"][c])) == "conv2/igemm_tc"]
+    dw = [int(c) for c in np.flatnonzero(t["layer"] == 2)]
+    seen = set()
+    for c in tc:
+        for d in dw if c in (tc[0], tc[-1]) else dw[:1]:
+            g.set_option(SN_OPT_PAIR, 1)
+            g.set_path([int(np.flatnonzero(t["layer"] == 0)[0]), c, d, int(np.flatnonzero(t["layer"] == 3)[0])])
+            what = g.candidate_desc(c) + " + " + g.candidate_desc(d)
+            split = "ksplit=1" not in what and "cluster=" not in what or "csk=2" in what or "streamk" in what
+            one = g.plan_stats()[1] == 1
+            assert not (one and split), what
+            assert one or split or "cluster=8" in what or W == 300, what
+            seen.add((one, what.split("cluster=")[-1][:1] if "cluster=" in what else split))
+            y = g.run(xd).clone()
+            g.set_option(SN_OPT_PAIR, 0)
+            y2 = g.run(xd)
+            torch.cuda.synchronize()
+            assert torch.equal(y.view(torch.int16), y2.view(torch.int16)), what
+    assert (True, False) in seen and ((True, "2") in seen or C <= 64)
+    if W == 300 and dt == "f16":
+        assert any(not one for one, _ in seen)
