@@ -348,10 +348,6 @@ cudaError_t weight_format_q8(const float *w, void *out, int fmt, int64_t K, int6
 // conv2 / dwconv2, direct: one output code per thread (any layout, groups,
 // stride, dilation; optional residual)
 // ===========================================================================
-struct Q8Scales {
-    float s_x, s_r, inv_out;
-};
-
 template <bool NHWC, typename TO>
 __global__ void q8_conv_direct_kernel(const int8_t *__restrict__ x, const int8_t *__restrict__ w,
                                       const float *__restrict__ ws, const float *__restrict__ bias,
@@ -402,7 +398,6 @@ __global__ void q8_conv_direct_kernel(const int8_t *__restrict__ x, const int8_t
 
 // the schema dtype the routine writes: qint8, or a float type when the
 // dequantisation is fused into its epilogue
-static int out_dtype(const LaunchArgs &a) { return a.out_schema.dtype < 0 ? a.schema.dtype : a.out_schema.dtype; }
 
 #define SN_Q8_OUT_SWITCH(dt, TO, ...)                               \
     switch (dt) {                                                   \
@@ -412,17 +407,6 @@ static int out_dtype(const LaunchArgs &a) { return a.out_schema.dtype < 0 ? a.sc
     case SN_F32: { using TO = float; __VA_ARGS__; break; }          \
     default: return cudaErrorInvalidValue;                          \
     }
-
-static Q8Scales scales_of(const LaunchArgs &a) {
-    return Q8Scales{a.qs_in[0], a.qs_in[1], a.qs_out > 0.0f ? 1.0f / a.qs_out : 0.0f};
-}
-
-// the input scales, and the output scale when the output is qint8
-static bool scales_ok(const LaunchArgs &a, int n_in) {
-    for (int i = 0; i < n_in; ++i)
-        if (!(a.qs_in[i] > 0.0f) || !std::isfinite(a.qs_in[i])) return false;
-    return out_dtype(a) != SN_QI8 || (a.qs_out > 0.0f && std::isfinite(a.qs_out));
-}
 
 // dwconv2 3x3 / 5x5, NHWC, dilation 1, C % 4 == 0: four channels (one word of
 // codes) and QB output columns per thread.  dp4a multiplies a word of four

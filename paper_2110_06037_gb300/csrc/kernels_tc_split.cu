@@ -681,7 +681,8 @@ cudaError_t conv_split(const LaunchArgs &a, int32_t v) {
     const bool f32 = a.schema.dtype == SN_F32;
     const int planes = f32 ? 3 : 1;
     const sn_conv_params &c = l.conv;
-    const int out_dt = a.out_schema.dtype < 0 ? a.schema.dtype : a.out_schema.dtype;
+    const int out_dt = out_dtype(a);
+    if (!f32 && !scales_ok(a, a.in[1] ? 2 : 1)) return cudaErrorInvalidValue;
     if (!a.ws || a.ws_bytes < conv_split_ws(l, in, a.schema) || (uintptr_t)a.ws % 16 || (uintptr_t)a.wt % 16)
         return cudaErrorInvalidValue;
     SParams p{};
@@ -740,8 +741,8 @@ cudaError_t conv_split(const LaunchArgs &a, int32_t v) {
         p.w32 = tail;
     } else {
         p.ws = tail;
-        p.s_x = a.qs_in[0], p.s_r = a.qs_in[1];
-        p.inv_out = a.qs_out > 0.0f ? 1.0f / a.qs_out : 0.0f;
+        const Q8Scales q = scales_of(a);
+        p.s_x = q.s_x, p.s_r = q.s_r, p.inv_out = q.inv_out;
     }
     CUtensorMap mA[4], mB;
     {

@@ -2,6 +2,7 @@
 // requantisation with one rounding per written operation, vector types.
 #pragma once
 
+#include <cmath>
 #include <type_traits>
 
 #include "kern_common.cuh"
@@ -47,6 +48,21 @@ __device__ __forceinline__ TO q8_out(float y, float inv) {
 // code of a weight of scale s
 __device__ __forceinline__ int q8_weight_code(float v, float s) {
     return max(-QMAX, min(QMAX, __float2int_rn(__fdiv_rn(v, s))));
+}
+
+// the scales that a launch reads and writes codes with
+struct Q8Scales {
+    float s_x, s_r, inv_out;
+};
+inline int out_dtype(const LaunchArgs &a) { return a.out_schema.dtype < 0 ? a.schema.dtype : a.out_schema.dtype; }
+inline Q8Scales scales_of(const LaunchArgs &a) {
+    return Q8Scales{a.qs_in[0], a.qs_in[1], a.qs_out > 0.0f ? 1.0f / a.qs_out : 0.0f};
+}
+// the input scales, and the output scale when the output is qint8
+inline bool scales_ok(const LaunchArgs &a, int n_in) {
+    for (int i = 0; i < n_in; ++i)
+        if (!(a.qs_in[i] > 0.0f) || !std::isfinite(a.qs_in[i])) return false;
+    return out_dtype(a) != SN_QI8 || (a.qs_out > 0.0f && std::isfinite(a.qs_out));
 }
 
 // per-output-channel scales max |w[k, .]| / 127 (1 for an all-zero channel) of fp32 weights [K][per_k]

@@ -150,6 +150,36 @@ def test_q8_bit_exact(case, extreme, out_dt):
         assert np.array_equal(got.reshape(want.shape), want.astype(got.dtype)), g.candidate_desc(c)
 
 
+def test_q8_refuses_an_infinite_scale_in_every_variant():
+    """Calibration of a layer whose sums overflow leaves an infinite scale: every
+    way to run the layer says so (zeros with a good status are no answer)."""
+    rng = np.random.default_rng(8)
+    sch = ("f32", "nhwc")
+    layers = [dict(conv_layer(rng, 16, 16, 1, 1, 0, 1), inputs=[-1]), dict(conv_layer(rng, 16, 16, 1, 1, 0, 1), inputs=[0])]
+    layers[0]["weight"][:] = 3e38
+    g = build_graph(layers, (1, 16, 8, 8), sch, sch, [sch, ("qi8", "nhwc")])
+    t = g.cost_table()
+    t["cost"] = np.where(t["routine"] == 0, 0, 1).astype(np.int64)
+    t["adapt"] = np.where(np.eye(t["adapt"].shape[1], dtype=bool), 0, 1).astype(np.int64) * np.ones_like(t["adapt"])
+    g.set_cost_table(t)
+    xd = to_device(np.ones((1, 16, 8, 8), np.float32), sch)
+    g.calibrate(xd)
+    assert np.isfinite(g.get_qscale(-1)) and g.get_qscale(0) == np.inf
+
+    def of(layer, out):
+        return [int(c) for c in np.flatnonzero((t["layer"] == layer) & (t["schema"] == 1) & (t["out_schema"] == out))]
+
+    io = [int(np.flatnonzero(t["layer"] == i)[0]) for i in (0, 3)]
+    last = [c for c in of(2, 0) if " [tc " in g.candidate_desc(c)][0]  # codes in, fp32 out: no adapt reads the scale
+    names = {c: g.candidate_desc(c) for c in of(1, 1)}
+    assert sum("dp4a" in d for d in names.values()) > 1 and any("direct" in d for d in names.values())
+    for c, d in names.items():
+        g.set_path([io[0], c, last, io[1]])
+        with pytest.raises(SnError):
+            g.run(xd)
+            pytest.fail(d)
+
+
 def test_expired_wait_reports_timeout_and_recovers():
     import torch
     x, layers = synth.single_conv(2, 14, 64, 128, 3, 1)
