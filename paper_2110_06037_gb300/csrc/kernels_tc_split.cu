@@ -52,9 +52,13 @@ namespace tcs {
 using namespace tc;
 
 constexpr int SPLIT_THREADS = 320;  // producer, MMA issuer, eight epilogue warps
-// K steps (64 values) per accumulator drain: 256 values bound the tensor
-// core's accumulation error in fp32; 1024 code products stay exact in qint8
-constexpr int chunk_of(int planes) { return planes == 3 ? 4 : 16; }
+// K steps (64 values) per accumulator drain.  The tensor core truncates each
+// accumulation of 16 products, an error of one sign where the products are: 128
+// values a drain keep operands of one sign below the fp32 routines' error (256 ->
+// 64 channels, 1x1, all positive: 1.6e-7 of the result, igemm_simt 2.2e-7; 256
+// values a drain: 3.5e-7; the bottleneck at batch 8: 52.0 -> 53.2 us).  1024 code
+// products stay exact in qint8.
+constexpr int chunk_of(int planes) { return planes == 3 ? 2 : 16; }
 
 struct SParams {
     int32_t N, H, W, C, K, P, Q, R, S;       // the layer (fix-up and output addressing)

@@ -44,11 +44,12 @@ def force(g, t, layer, c):
 @pytest.mark.parametrize("case", CASES)
 @pytest.mark.parametrize("residual", [False, True])
 def test_f32(case, residual):
-    """Error bound, per output, against fp64: a drain covers 256 products in 16
+    """Error bound, per output, against fp64: a drain covers 128 products in 8
     accumulation steps of 16 products; allowing a truncated unit (2^-23) for
-    each step and one for its alignment, 2^-18 of sum |x w| covers a drain, the
-    round-to-nearest sums of the drains (at most 54, 2^-24 each) and the dropped
-    plane products (2^-25); bias and residual add two roundings of the result."""
+    each step and one for its alignment, 2^-19 of sum |x w| covers a drain, and
+    2^-18 the round-to-nearest sums of the drains (at most 27, 2^-24 each) and the
+    dropped plane products (2^-25) besides; bias and residual add two roundings
+    of the result."""
     import torch
     N, C, H, W, K, k, s, pd, dil = case
     sch = ("f32", "nhwc")
@@ -82,6 +83,33 @@ def test_f32(case, residual):
         assert (np.abs(got - want) <= bound).all(), (g.candidate_desc(c), float((np.abs(got - want) / bound).max()))
         # far below the bound in the mean: the error of an fp32 sum, not of a 16-bit one
         assert np.linalg.norm(got - want) <= 2e-6 * np.linalg.norm(want), g.candidate_desc(c)
+
+
+@pytest.mark.parametrize("C,k", [(128, 1), (256, 1), (384, 1), (512, 1), (16, 3), (128, 3)])
+def test_f32_operands_of_one_sign(C, k):
+    """The tensor core's truncation does not cancel: of each of a drain's 8
+    accumulation steps half a unit (2^-24) of the partial sum in the mean, and the
+    partial sums come to 4.5 times the drain's, so 4.5 * 2^-24 of the result; from
+    256 products on, no more than the fp32 multiply-adds of the direct kernel."""
+    import torch
+    sch = ("f32", "nhwc")
+    rng = np.random.default_rng(C + k)
+    x = np.abs(rng.standard_normal((2, C, 14, 14))).astype(np.float32)
+    layer = synth.conv(C, 64, k, 1, k // 2, act="none")
+    layer["weight"] = np.abs(rng.standard_normal((64, C, k, k))).astype(np.float32)
+    layer["bias"] = np.zeros(64, np.float32)
+    want = run_layer(layer, [x.astype(np.float64)])
+    g = build_graph([dict(layer, inputs=[-1])], x.shape, sch, sch, [sch])
+    cands, t = tc_candidates(g, 1)
+    direct = [int(c) for c in np.flatnonzero(t["layer"] == 1) if routine_name(int(t["routine"][c])) == "conv2/direct"]
+    err = []
+    for c in direct + cands:
+        force(g, t, 1, c)
+        y = g.run(to_device(x, sch))
+        torch.cuda.synchronize()
+        err.append(np.linalg.norm(from_device(y, sch).reshape(want.shape) - want) / np.linalg.norm(want))
+    assert max(err[1:]) <= 4.5 * 2.0 ** -24, err
+    assert C * k * k < 256 or max(err[1:]) <= err[0], err
 
 
 def test_f32_infinities_and_large_values():
