@@ -1,8 +1,12 @@
 // Convolution whose operands are exact sums of bf16 planes, on the tcgen05
 // tensor cores: fp32 (three planes) and qint8 (one plane) implicit GEMM, NHWC.
 //
-//   fp32   x = x0 + x1 + x2 with x0 = bf16(x), x1 = bf16(x - x0), x2 = x - x0 -
-//          x1: 8 + 8 + 8 significant bits, so the sum is exact.  Of the nine
+//   fp32   2^24 x = x0 + x1 + x2 with x0 = bf16(2^24 x), x1 and x2 likewise of what
+//          is left: 8 + 8 + 8 significant bits, so the sum is exact for every
+//          |x| < 2^104 (unscaled, the last planes of an x below 2^-110 would fall
+//          under bf16's smallest value).  The sums, 2^48 times the result, are
+//          scaled back exactly; operands and sums too large for the planes are
+//          recomputed (plain_sum).  Of the nine
 //          plane products the six with i + j <= 2 are formed, each i + j in an
 //          accumulator of its own; the dropped ones are below 2^-26 of |x w|.
 //          With 64-channel tiles the planes of B lie behind one another as rows
@@ -78,9 +82,12 @@ struct SParams {
     float s_x, s_r, inv_out;
 };
 
-// y of one output element in plain fp32, for a sum that the planes cannot
+// the planes are those of SCALE * x and SCALE * w
+constexpr float SCALE = 16777216.0f, UNSCALE = 1.0f / SCALE / SCALE;
+
+// the sum of one output element in plain fp32, for one that the planes cannot
 // carry: an infinity or a NaN among the operands (the planes of an infinity
-// are inf, NaN, NaN), a value above bf16's range, or a sum above fp32's
+// are inf, NaN, NaN), an operand from 2^104 on, or sums from 2^80 on
 __device__ __noinline__ float plain_sum(const SParams &p, int64_t pix, int k) {
     const int q = (int)(pix % p.Q), pp = (int)((pix / p.Q) % p.P);
     const int64_t n = pix / ((int64_t)p.Q * p.P);
@@ -398,6 +405,8 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1)
                 }
                 TO o[G];
                 if constexpr (F32) {
+#pragma unroll
+                    for (int e = 0; e < G; ++e) acc[j + e] *= UNSCALE;
                     // one test for the group: an infinity or a NaN has all exponent bits
                     bool odd_value = false;
 #pragma unroll
@@ -498,8 +507,9 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1)
 }
 
 // ------------------------------------------------------- operand planes
-// the three bf16 planes of an fp32 value
+// the three bf16 planes of SCALE times an fp32 value
 __device__ __forceinline__ void planes_of(float x, __nv_bfloat16 (&o)[3]) {
+    x *= SCALE;
     o[0] = __float2bfloat16_rn(x);
     const float r = x - __bfloat162float(o[0]);
     o[1] = __float2bfloat16_rn(r);

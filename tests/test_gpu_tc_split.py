@@ -142,6 +142,31 @@ def test_f32_infinities_and_large_values():
         assert np.allclose(o[fine], outs[0][fine], rtol=1e-5, atol=1e-5)
 
 
+@pytest.mark.parametrize("sx,sw", [(2.0 ** -120, 2.0 ** 100), (2.0 ** -130, 2.0 ** 30), (1e-36, 1.0), (2.0 ** -60, 2.0 ** -60),
+                                   (2.0 ** 60, 2.0 ** 10), (2.0 ** 106, 2.0 ** -90), (1.0, 2.0 ** 105)])
+def test_f32_tiny_and_huge_operands(sx, sw):
+    """The bound of test_f32 for operands and results over fp32's whole range (a
+    subnormal operand or result counts with its own spacing, 2^-149)."""
+    import torch
+    sch = ("f32", "nhwc")
+    rng = np.random.default_rng(6)
+    x = (rng.standard_normal((1, 40, 7, 7)).astype(np.float32) * np.float32(sx)).astype(np.float32)
+    layer = synth.conv(40, 24, 3, 1, 1, act="none")
+    layer["weight"] = (rng.standard_normal((24, 40, 3, 3)).astype(np.float32) * np.float32(sw)).astype(np.float32)
+    layer["bias"] = np.zeros(24, np.float32)
+    mag = run_layer(dict(layer, weight=np.abs(layer["weight"])), [np.abs(x).astype(np.float64)])
+    want = run_layer(layer, [x.astype(np.float64)])
+    g = build_graph([dict(layer, inputs=[-1])], x.shape, sch, sch, [sch])
+    cands, t = tc_candidates(g, 1)
+    for c in cands:
+        force(g, t, 1, c)
+        y = g.run(to_device(x, sch))
+        torch.cuda.synchronize()
+        got = from_device(y, sch).reshape(want.shape)
+        bound = 2.0 ** -18 * mag + 2.0 ** -148
+        assert (np.abs(got - want) <= bound).all(), (g.candidate_desc(c), float((np.abs(got - want) / bound).max()))
+
+
 @pytest.mark.parametrize("case", [c for c in CASES if c[1] % 4 == 0 and c[4] % 4 == 0])
 @pytest.mark.parametrize("extreme", [False, True])
 @pytest.mark.parametrize("out_dt", ["qi8", "f16", "f32"])
