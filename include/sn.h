@@ -358,7 +358,14 @@ SN_API sn_status sn_plan_memory(sn_graph *g, int64_t *arena_bytes, int64_t *unsh
 SN_API sn_status sn_layer_shape(sn_graph *g, int32_t layer, int64_t out_nchw[4]);
 
 /* Save / restore the tuned state (cost table + selected path) as JSON.  A
- * loaded file must describe the same net (same layers and candidates). */
+ * loaded file must describe the same net (same layers and candidates).  A file
+ * of a build with fewer routines or routine parameters loads too: what it lists
+ * must be candidates of this net (each carries an id of its routine,
+ * parameters, schemas, layer and shapes), in order, at least one a layer; the
+ * others stay unprofiled (infinite cost), as they do for a shortened list.
+ * Files without ids, of the first format, must list exactly this net's
+ * candidates or exactly those that the builds of that format had.
+ * Errors: SN_EINVAL (the file, or a list that differs). */
 SN_API sn_status sn_save_plan(sn_graph *g, const char *path);
 SN_API sn_status sn_load_plan(sn_graph *g, const char *path);
 

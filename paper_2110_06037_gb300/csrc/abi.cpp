@@ -1,12 +1,11 @@
 // extern "C" boundary of the library (declared in include/sn.h).  Every entry
 // point catches C++ exceptions and turns them into a status, so nothing but
 // an sn_status crosses the ABI.
-#include <array>
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
 #include <fstream>
-#include <map>
 #include <sstream>
 #include <string>
 
@@ -597,14 +596,14 @@ sn_status sn_save_plan(sn_graph *gg, const char *path) {
         if (rc != SN_OK) return rc;
         std::ofstream f(path);
         if (!f) return fail(SN_EINVAL, std::string("cannot open ") + path);
-        f << "{\n \"format\": \"softneuro-gb300-plan-1\",\n";
+        f << "{\n \"format\": \"softneuro-gb300-plan-2\",\n";
         f << " \"n_layers\": " << g->n_layers() << ",\n \"n_schemas\": " << g->n_schemas()
           << ",\n \"n_edges\": " << g->edges.size() << ",\n \"n_candidates\": " << g->cands.size() << ",\n";
         f << " \"candidates\": [";
         for (size_t c = 0; c < g->cands.size(); ++c) {
             const Candidate &k = g->cands[c];
             f << (c ? ", " : "") << "[" << k.routine << ", " << k.variant << ", " << k.schema << ", "
-              << k.layer << ", " << k.cost << "]";
+              << k.layer << ", " << k.cost << ", " << cand_out(k) << ", " << candidate_id(*g, (int32_t)c) << "]";
         }
         f << "],\n \"adapt_cost\": [";
         for (size_t i = 0; i < g->adapt_cost.size(); ++i) f << (i ? ", " : "") << g->adapt_cost[i];
@@ -669,30 +668,37 @@ sn_status sn_load_plan(sn_graph *gg, const char *path) {
             !read_int_array(doc, "candidates", cands) || !read_int_array(doc, "adapt_cost", ac) ||
             !read_int_array(doc, "path", pth))
             return fail(SN_EINVAL, "sn_load_plan: malformed plan file");
-        if (nl != g->n_layers() || ns != g->n_schemas() || ne != (int64_t)g->edges.size() || nc < 0 ||
-            cands.size() != (size_t)nc * 5 || ac.size() != g->adapt_cost.size())
+        const size_t width = cands.size() == (size_t)nc * 7 ? 7 : 5;
+        if (nl != g->n_layers() || ns != g->n_schemas() || ne != (int64_t)g->edges.size() || nc < 1 ||
+            cands.size() != (size_t)nc * width || ac.size() != g->adapt_cost.size())
             return fail(SN_EINVAL, "sn_load_plan: plan describes a different net");
-        // the file's candidates, in order, among the graph's: a build with more
-        // routines or routine parameters than the one that wrote the file keeps
-        // its own as not profiled (infinite cost)
-        std::vector<int32_t> at((size_t)nc);
-        {
-            typedef std::array<int64_t, 4> Key;  // routine, variant, schema, layer
-            std::map<Key, std::vector<int32_t>> where;  // several when a routine writes several schemas
-            std::map<Key, size_t> used;
-            for (size_t c = 0; c < g->cands.size(); ++c) {
-                const Candidate &k = g->cands[c];
-                where[Key{k.routine, k.variant, k.schema, k.layer}].push_back((int32_t)c);
-            }
-            for (size_t c = 0; c < (size_t)nc; ++c) {
-                const Key k{cands[5 * c], cands[5 * c + 1], cands[5 * c + 2], cands[5 * c + 3]};
-                const auto it = where.find(k);
-                const size_t i = used[k]++;
-                if (it == where.end() || i >= it->second.size())
-                    return fail(SN_EINVAL, "sn_load_plan: candidate list differs");
-                at[c] = it->second[i];
+        // the file's candidates among the graph's: all of them in order; or, from
+        // a build with fewer routines or routine parameters, those that carry
+        // the same id, at least one of every layer; or, in the first format, which
+        // has no ids, exactly those that the builds of that format listed
+        const int32_t nmine = (int32_t)g->cands.size();
+        auto same = [&](int32_t c, size_t e) {
+            const Candidate &k = g->cands[c];
+            return cands[e] == k.routine && cands[e + 1] == k.variant && cands[e + 2] == k.schema && cands[e + 3] == k.layer;
+        };
+        bool all = nc == nmine;
+        for (int32_t c = 0; all && c < nmine; ++c) all = same(c, (size_t)c * width);
+        std::vector<int32_t> at;
+        std::vector<char> has((size_t)nl, 0);
+        bool ok = true;
+        for (int32_t c = 0; ok && c < nmine && (int64_t)at.size() <= nc; ++c) {
+            const size_t e = at.size() * width;
+            const bool more = (int64_t)at.size() < nc;
+            if (all || (width == 7 ? more && same(c, e) && cands[e + 5] == cand_out(g->cands[c]) &&
+                                         cands[e + 6] == candidate_id(*g, c)
+                                   : candidate_in_plan1(*g, c))) {
+                ok = more && same(c, e);
+                at.push_back(c);
+                has[(size_t)g->cands[c].layer] = 1;
             }
         }
+        if (!ok || (int64_t)at.size() != nc || std::find(has.begin(), has.end(), 0) != has.end())
+            return fail(SN_EINVAL, "sn_load_plan: candidate list differs");
         std::vector<int32_t> path;
         if (!pth.empty()) {
             if ((int64_t)pth.size() != nl) return fail(SN_EINVAL, "sn_load_plan: bad path length");
@@ -704,7 +710,7 @@ sn_status sn_load_plan(sn_graph *gg, const char *path) {
             }
         }
         for (Candidate &k : g->cands) k.cost = kInf;
-        for (size_t c = 0; c < at.size(); ++c) g->cands[at[c]].cost = cands[5 * c + 4];
+        for (size_t c = 0; c < at.size(); ++c) g->cands[at[c]].cost = cands[width * c + 4];
         for (size_t i = 0; i < ac.size(); ++i) g->adapt_cost[i] = ac[i];
         g->has_path = !path.empty();
         if (g->has_path) {

@@ -925,6 +925,21 @@ int32_t dense_tc_variants(const Layer &l, const Shape &in, sn_schema s) {
     return (int32_t)tc::configs(gl, in, nhwc).size();
 }
 
+int32_t tc_first_variants(int32_t r, const Layer &l, const Shape &in, sn_schema s) {
+    std::vector<tc::Config> cfgs;
+    if (r == R_CONV_TC) {
+        cfgs = tc::configs(l, in, s);
+    } else if (r == R_CONV_IM2COL_TC) {
+        cfgs = tc::configs(gemm_layer((int)im2col_kpad(l), l.conv.c_out, l.conv.act, l.out),
+                           Shape{l.out.n, im2col_kpad(l), l.out.h, l.out.w}, s);
+    } else if (r == R_DENSE_TC) {
+        cfgs = tc::configs(gemm_layer(l.dense_in, l.dense_out, l.act, l.out), in, sn_schema{s.dtype, SN_NHWC});
+    } else {
+        return INT32_MAX;
+    }
+    return (int32_t)std::count_if(cfgs.begin(), cfgs.end(), [](const tc::Config &x) { return x.lat == 0; });
+}
+
 size_t dense_tc_ws(const Layer &l, const Shape &in, sn_schema s, int32_t v) {
     const Layer gl = gemm_layer(l.dense_in, l.dense_out, l.act, l.out);
     return conv_tc_ws(gl, in, sn_schema{s.dtype, SN_NHWC}, v);

@@ -4,6 +4,7 @@
 //
 // Every routine reads its inputs and writes its output in its own schema;
 // conversions between schemas are separate adapt routines on the edges.
+#include <sstream>
 #include <string>
 
 #include "sn_internal.h"
@@ -67,6 +68,33 @@ std::string candidate_desc(const Graph &g, int32_t cand) {
         params = variant_name(c.routine, c.variant);
     if (!params.empty()) d += " [" + params + "]";
     return d;
+}
+
+int64_t candidate_id(const Graph &g, int32_t cand) {
+    const Layer &l = g.layers[g.cands[cand].layer];
+    std::ostringstream s;
+    s << candidate_desc(g, cand) << '|' << g.cands[cand].variant << '|' << g.cands[cand].layer << '|' << l.type;
+    const sn_conv_params &c = l.conv;
+    for (int32_t v : {c.c_in, c.c_out, c.kh, c.kw, c.sh, c.sw, c.ph, c.pw, c.dh, c.dw, c.groups, c.act, l.pool.kh,
+                      l.pool.kw, l.pool.sh, l.pool.sw, l.pool.ph, l.pool.pw, l.act, l.dense_in, l.dense_out})
+        s << ',' << v;
+    auto shape = [&](const Shape &x) { s << '|' << x.n << 'x' << x.c << 'x' << x.h << 'x' << x.w; };
+    for (int32_t j : l.inputs) shape(g.layers[j].out);
+    shape(l.out);
+    uint64_t h = 14695981039346656037ull;  // FNV-1a
+    for (const char ch : s.str()) h = (h ^ (uint8_t)ch) * 1099511628211ull;
+    return (int64_t)(h >> 2);
+}
+
+// Plan files of the first format come from builds without the half-SM tiles,
+// conv2/igemm_tc_odd and the convolutions on bf16 planes
+bool candidate_in_plan1(const Graph &g, int32_t cand) {
+    const Candidate &c = g.cands[cand];
+    if (c.routine == R_CONV_TC_ODD || c.routine == R_CONV_TC_F32) return false;
+    if (c.routine == R_CONV_DP4A) return c.variant == 0;
+    if (c.routine != R_CONV_TC && c.routine != R_CONV_IM2COL_TC && c.routine != R_DENSE_TC) return true;
+    const Layer &l = g.layers[c.layer];
+    return c.variant < k::tc_first_variants(c.routine, l, g.layers[l.inputs[0]].out, g.schemas[c.schema]);
 }
 
 static bool is_conv(const Layer &l) { return l.type == SN_L_CONV2; }

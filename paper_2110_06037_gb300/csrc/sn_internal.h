@@ -278,6 +278,8 @@ const char *routine_name(int32_t routine);
 const char *variant_name(int32_t routine, int32_t variant);
 // descriptor of one candidate of a graph: routine name, schema and routine parameters
 std::string candidate_desc(const Graph &g, int32_t cand);
+int64_t candidate_id(const Graph &g, int32_t cand);     // of its routine, parameters, schemas, layer and shapes
+bool candidate_in_plan1(const Graph &g, int32_t cand);  // in the lists of plan files of the first format
 size_t routine_workspace(int32_t routine, int32_t variant, const Layer &layer,
                          const std::vector<Shape> &in, sn_schema s);
 // prepare weights for (layer, routine, variant, schema); returns device pointer
@@ -361,6 +363,8 @@ int32_t conv_tc_variants(const Layer &l, const Shape &in, sn_schema s, bool odd 
 size_t conv_tc_ws(const Layer &l, const Shape &in, sn_schema s, int32_t v, int32_t a_blocks = 0,
                   bool odd = false);  // K-split partials
 size_t dense_tc_ws(const Layer &l, const Shape &in, sn_schema s, int32_t v);
+// how many of a tensor-core routine's variants come before its half-SM tiles, the last ones
+int32_t tc_first_variants(int32_t r, const Layer &l, const Shape &in, sn_schema s);
 const char *conv_tc_variant_name(int32_t v);
 std::vector<char> conv_tc_nchw_ok(const Layer &l, const Shape &in, sn_schema s, bool odd = false);  // per variant
 int32_t conv_tc_sum_parts(const Layer &l, const Shape &in, sn_schema s, int32_t v);

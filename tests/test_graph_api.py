@@ -251,3 +251,87 @@ def test_plan_file_of_a_build_with_fewer_candidates(tmp_path):
     f.write_text(json.dumps(doc))
     with pytest.raises(Exception):
         g2.load_plan(f)
+
+
+def _one_conv_net(n, c, k, hw=8):
+    import synth
+    layer = synth.conv(c, k, 3, 1)
+    layer["weight"] = np.ones((k, c, 3, 3), np.float32)
+    sch = [("f16", "nchw"), ("f16", "nhwc"), ("f32", "nhwc"), ("qi8", "nhwc")]
+    g = build_graph([dict(layer, inputs=[-1])], (n, c, hw, hw), sch[0], sch[0], sch)
+    t = g.cost_table()
+    t["cost"] = np.arange(len(t["cost"])) + 100
+    t["adapt"][t["adapt"] > 0] = 7
+    g.set_cost_table(t)
+    mine = np.flatnonzero(t["layer"] == 1)
+    g.set_path([int(np.flatnonzero(t["layer"] == 0)[0]), int(mine[5]), int(np.flatnonzero(t["layer"] == 2)[0])])
+    return g
+
+
+def _first_format(doc, keep):
+    """The document as the first format had it: five numbers a candidate, those in `keep` only."""
+    doc = dict(doc, format="softneuro-gb300-plan-1", n_candidates=len(keep),
+               candidates=[doc["candidates"][i][:5] for i in keep])
+    doc["path"] = [keep.index(c) for c in doc["path"]]
+    return doc
+
+
+def test_plan_file_of_the_first_format(tmp_path):
+    """Without ids, a list must be this net's or the one that the builds of that
+    format made of it; any other is another net's."""
+    import json
+
+    from paper_2110_06037_gb300._sn import COST_INF
+    g = _one_conv_net(2, 128, 64)
+    f = tmp_path / "plan.json"
+    g.save_plan(f)
+    doc = json.loads(f.read_text())
+    desc = [g.candidate_desc(c) for c in range(doc["n_candidates"])]
+    later = [d for d in desc if "cluster=" in d or "igemm_tc_odd" in d or "igemm_tc_f32" in d or " [tc " in d]
+    assert any("cluster=" in d for d in later) and any("igemm_tc_f32" in d for d in later) and any("dp4a" in d for d in later)
+    old = [i for i, d in enumerate(desc) if d not in later]
+    for keep in (list(range(len(desc))), old):
+        f.write_text(json.dumps(_first_format(doc, keep)))
+        g2 = _one_conv_net(2, 128, 64)
+        g2.load_plan(f)
+        cost = list(g2.cost_table()["cost"])
+        assert cost == [doc["candidates"][i][4] if i in keep else COST_INF for i in range(len(desc))]
+        g2.save_plan(tmp_path / "back.json")
+        assert json.loads((tmp_path / "back.json").read_text())["path"] == doc["path"]
+    for drop in (old[-2], [i for i in range(len(desc)) if i not in old][0]):
+        for keep in (list(range(len(desc))), old):
+            if drop in keep and drop not in doc["path"]:
+                f.write_text(json.dumps(_first_format(doc, [i for i in keep if i != drop])))
+                with pytest.raises(SnError):
+                    g.load_plan(f)
+
+
+def test_plan_file_of_another_net_with_a_shorter_list(tmp_path):
+    """Same layers, another batch or channel count: fewer variants apply there, and
+    those of the same index are other tiles here."""
+    import json
+    f = tmp_path / "plan.json"
+    here = _one_conv_net(1, 64, 128, 14)
+    shorter = 0
+    for other in (_one_conv_net(32, 64, 128, 14), _one_conv_net(1, 64, 64, 14), _one_conv_net(1, 256, 128, 14)):
+        other.save_plan(f)
+        doc = json.loads(f.read_text())
+        keys = [tuple(c[:4]) for c in doc["candidates"]]
+        here.save_plan(tmp_path / "here.json")
+        mine = [tuple(c[:4]) for c in json.loads((tmp_path / "here.json").read_text())["candidates"]]
+        assert keys != mine
+        shorter += all(keys.count(k) <= mine.count(k) for k in keys)
+        with pytest.raises(SnError):
+            here.load_plan(f)
+        f.write_text(json.dumps(_first_format(doc, list(range(len(keys))))))
+        with pytest.raises(SnError):
+            here.load_plan(f)
+    assert shorter
+    # a layer without candidates, and candidates in another order
+    here.save_plan(f)
+    doc = json.loads(f.read_text())
+    for cands in ([c for c in doc["candidates"] if c[3] != 1], doc["candidates"][:1] + doc["candidates"][2:0:-1] + doc["candidates"][3:]):
+        bad = dict(doc, candidates=cands, n_candidates=len(cands), path=[])
+        f.write_text(json.dumps(bad))
+        with pytest.raises(SnError):
+            here.load_plan(f)
