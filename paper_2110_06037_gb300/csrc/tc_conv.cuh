@@ -981,12 +981,9 @@ __global__ void splitk_reduce_kernel(const float *__restrict__ part, const float
     }
 }
 
-template <typename T, int BN, bool IMPLICIT, int G, int KB, bool BST = false, int MS = 1, int CSK = 1,
-          bool SK = false, bool HALO = false>
-static cudaError_t launch(const CUtensorMap *mA, const CUtensorMap &mB, const CUtensorMap &mY, const CUtensorMap &mR,
-                          const Params &p,
-                          cudaStream_t st) {
-    constexpr int NBUF = BST || HALO || SK || CSK > 1 ? 1 : staging_blocks(BN, G, KB, MS);
+template <typename T, int BN, bool IMPLICIT, int G, int KB, bool BST, int MS, int CSK, bool SK, bool HALO, int NBUF>
+static cudaError_t launch_n(const CUtensorMap *mA, const CUtensorMap &mB, const CUtensorMap &mY, const CUtensorMap &mR,
+                            const Params &p, cudaStream_t st) {
     constexpr uint32_t STG = NBUF * EPI_WARPS * STG_BYTES;
     constexpr int STAGES = BST ? BST_STAGES : HALO ? halo_stages(BN / G) : stages_for(BN, G, KB, MS, (NBUF - 1) * 32768);
     // bytes of one pipeline stage (A and this CTA's share of B), as the kernel lays them out
@@ -1063,6 +1060,18 @@ static cudaError_t launch(const CUtensorMap *mA, const CUtensorMap &mB, const CU
                static_cast<T *>(p.y), p.Mout, p.K,
                                                                p.ksplit, p.act);
     return cudaGetLastError();
+}
+
+// two staging blocks a warp where a residual comes through them and the ring
+// keeps four stages; a layer without one has all the stages there are
+template <typename T, int BN, bool IMPLICIT, int G, int KB, bool BST = false, int MS = 1, int CSK = 1,
+          bool SK = false, bool HALO = false>
+static cudaError_t launch(const CUtensorMap *mA, const CUtensorMap &mB, const CUtensorMap &mY, const CUtensorMap &mR,
+                          const Params &p, cudaStream_t st) {
+    constexpr int NBUF = BST || HALO || SK || CSK > 1 ? 1 : staging_blocks(BN, G, KB, MS);
+    if (NBUF == 1 || (p.res && p.ksplit == 1))
+        return launch_n<T, BN, IMPLICIT, G, KB, BST, MS, CSK, SK, HALO, NBUF>(mA, mB, mY, mR, p, st);
+    return launch_n<T, BN, IMPLICIT, G, KB, BST, MS, CSK, SK, HALO, 1>(mA, mB, mY, mR, p, st);
 }
 
 // halo launches (kernels_tc_halo.cu): 3x3 stride-1 tiles of 8 x 16 pixels per
