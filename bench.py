@@ -57,6 +57,21 @@ def job_throughput(ms_local, ws, batch, dist=None, device="cpu"):
     return ms, ws * batch / (ms / 1e3)
 
 
+# what the benchmark reports besides its line, on stderr: with these tables in it
+# the line was 20 KB, too long for a reader that keeps the end of the output
+DETAILS = ("tuning_s", "path_cost_ns", "plan", "activation_memory", "per_routine_ms", "per_layer", "extras")
+
+
+def emit(line):
+    """The one JSON line on stdout, the details as another on stderr."""
+    def short(v):
+        if isinstance(v, dict):
+            return {k: short(x) for k, x in v.items()}
+        return float("%.7g" % v) if isinstance(v, float) else [short(x) for x in v] if isinstance(v, list) else v
+    print(json.dumps({"details": {k: line[k] for k in DETAILS if k in line}}), file=sys.stderr, flush=True)
+    print(json.dumps({k: short(v) for k, v in line.items() if k not in DETAILS}), flush=True)
+
+
 def dist_env():
     ws = int(os.environ.get("WORLD_SIZE", "1"))
     rank = int(os.environ.get("RANK", "0"))
@@ -519,7 +534,7 @@ def main():
                 "activation_memory": {"arena_bytes": arena_b, "unshared_bytes": unshared_b},
                 "per_routine_ms": {k: round(v["ms"], 4) for k, v in per_routine.items()},
                 "per_layer": per_layer, "extras": extras}
-        print(json.dumps(line))
+        emit(line)
     if dist:
         dist.destroy_process_group()
 
