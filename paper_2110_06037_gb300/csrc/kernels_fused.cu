@@ -325,7 +325,7 @@ ExpandDwPlan expand_dw_plan(const Layer &conv, const Shape &in, int32_t conv_var
         PB = std::min(PB, P);
         const int64_t bands = (P + PB - 1) / PB;
         PB = (P + bands - 1) / bands;
-        const int64_t grid = slices * bands * N, slots = 152 * (sm <= 110 * 1024 ? 2 : 1);
+        const int64_t grid = slices * bands * N, slots = (int64_t)num_sms() * (sm <= 110 * 1024 ? 2 : 1);
         if (grid <= slots) return ExpandDwPlan{MT, (int32_t)PB, (int32_t)bands, parts};
     }
     return none;
