@@ -77,10 +77,14 @@ inline unsigned grid_for(int64_t n, int block, int64_t cap = 152LL * 64) {
 // dispatch a runtime dtype to a C++ type
 // Programmatic dependent launch.  Every kernel of the library is launched
 // with launch_pdl, which lets it start (set up, fetch descriptors) while the
-// previous kernel on the stream drains; the kernel calls griddep_wait()
-// before its first global-memory access, which returns once the previous
-// grid has completed and its writes are visible, and griddep_launch() to let
-// its own successor start early.  Both are no-ops for a plain launch.
+// previous kernel on the stream drains; the kernel calls griddep_wait() before
+// its first access to memory that an earlier kernel writes or reads (blobs,
+// workspace, counters), which returns once the previous grid has completed and
+// its writes are visible.  Weights and biases may be read before it: no kernel
+// of a plan writes them, and their preparation is waited for on the host.
+// griddep_launch() lets the kernel's own successor start early; a kernel that
+// allocates tensor memory calls it behind the allocation (tmem_alloc in
+// tc_common.cuh).  Both are no-ops for a plain launch.
 __device__ __forceinline__ void griddep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
