@@ -35,7 +35,7 @@ constexpr int MAX_COLS = 256;  // of tensor memory: half of an SM's
 
 struct FParams {
     int32_t H, W, C, E, P, Q, ph, pw;
-    int32_t PB, cblocks, parts, act_e, act_d;
+    int32_t PB, cblocks, act_e, act_d;
     FastDiv fd_qb;  // column blocks of an output row
     const float *be, *bd;
     const void *wd;  // depthwise weights [KS * KS][E]
@@ -45,8 +45,9 @@ struct FParams {
 };
 
 // T: storage type; KS: 3 or 5; SW: stride; NT: threads (512 while a CTA has an SM
-// to itself, where the depthwise part is a latency)
-template <typename T, int KS, int SW, int NT>
+// to itself, where the depthwise part is a latency); PARTS: accumulators that an
+// expanded value is the sum of
+template <typename T, int KS, int SW, int NT, int PARTS>
 __global__ void __launch_bounds__(NT, 512 / NT)
     expand_dw_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUtensorMap mB,
                      const __grid_constant__ FParams p, int MT, uint32_t tmem_cols) {
@@ -126,11 +127,12 @@ __global__ void __launch_bounds__(NT, 512 / NT)
             if (!ok) break;
             tc_fence_after();
             int cb = 0;
-            for (int r = 0; r < p.parts; ++r)
-                for (const int cb0 = cb, cb1 = p.cblocks * (r + 1) / p.parts; cb < cb1; ++cb) {
+#pragma unroll
+            for (int r = 0; r < PARTS; ++r)
+                for (const int cb0 = cb, cb1 = p.cblocks * (r + 1) / PARTS; cb < cb1; ++cb) {
                     const int ks = min(BK / 16, (p.C - cb * BK + 15) / 16);  // 16-value steps that hold channels
                     for (int k = 0; k < ks; ++k)
-                        umma<1>(tmem + (uint32_t)((mt * p.parts + r) * 64),
+                        umma<1>(tmem + (uint32_t)((mt * PARTS + r) * 64),
                                 da0 + (uint64_t)((mt * tile_bytes + cb * (BM * BK * 2)) >> 4) + 2 * k,
                                 db0 + (uint64_t)((cb * (64 * BK * 2)) >> 4) + 2 * k, idesc, (cb > cb0 || k > 0) ? 1u : 0u);
                 }
@@ -157,9 +159,10 @@ __global__ void __launch_bounds__(NT, 512 / NT)
         tc_fence_after();
         __syncwarp();
         uint32_t v[32];
-        const uint32_t ta = tmem + ((uint32_t)(g4 * 32) << 16) + (uint32_t)(mt * p.parts * 64 + half * 32);
+        const uint32_t ta = tmem + ((uint32_t)(g4 * 32) << 16) + (uint32_t)(mt * PARTS * 64 + half * 32);
         tmem_ld32(ta, v);
-        for (int r = 1; r < p.parts; ++r) {  // (from zero, as the cluster's CTAs add)
+#pragma unroll
+        for (int r = 1; r < PARTS; ++r) {  // (from zero, as the cluster's CTAs add)
             uint32_t x[32];
             tmem_ld32(ta + (uint32_t)(r * 64), x);
 #pragma unroll
@@ -340,7 +343,6 @@ cudaError_t expand_dw(const LaunchArgs &a, const LaunchArgs &b, const ExpandDwPl
     p.H = (int)in.h, p.W = (int)in.w, p.C = (int)in.c, p.E = conv.conv.c_out;
     p.P = (int)dw.out.h, p.Q = (int)dw.out.w, p.ph = dw.conv.ph, p.pw = dw.conv.pw;
     p.PB = pl.PB;
-    p.parts = pl.parts;
     p.cblocks = (p.C + BK - 1) / BK;
     p.act_e = conv.conv.act, p.act_d = dw.conv.act;
     p.fd_qb = make_fastdiv((uint32_t)((p.Q + 3) / 4));
@@ -372,7 +374,15 @@ cudaError_t expand_dw(const LaunchArgs &a, const LaunchArgs &b, const ExpandDwPl
         return launch_pdl(kern, grid, dim3(big ? 256u : 512u), smem, a.stream, mA, mB, p, (int)pl.MT, cols);
     };
     const int ks = dw.conv.kh, sw = dw.conv.sw;
-#define SN_EXPAND_DW(T, KS, SW) return big ? go(expand_dw_kernel<T, KS, SW, 256>) : go(expand_dw_kernel<T, KS, SW, 512>)
+#define SN_EXPAND_DW_P(T, KS, SW, PARTS) \
+    return big ? go(expand_dw_kernel<T, KS, SW, 256, PARTS>) : go(expand_dw_kernel<T, KS, SW, 512, PARTS>)
+#define SN_EXPAND_DW(T, KS, SW)                          \
+    do {                                                 \
+        if (pl.parts == 1) SN_EXPAND_DW_P(T, KS, SW, 1); \
+        if (pl.parts == 2) SN_EXPAND_DW_P(T, KS, SW, 2); \
+        if (pl.parts == 4) SN_EXPAND_DW_P(T, KS, SW, 4); \
+        return cudaErrorInvalidValue;                    \
+    } while (0)
 #define SN_EXPAND_DW_T(T)                      \
     do {                                       \
         if (ks == 3 && sw == 1) SN_EXPAND_DW(T, 3, 1); \
@@ -383,6 +393,7 @@ cudaError_t expand_dw(const LaunchArgs &a, const LaunchArgs &b, const ExpandDwPl
     if (dt == SN_F16) SN_EXPAND_DW_T(__half);
     SN_EXPAND_DW_T(__nv_bfloat16);
 #undef SN_EXPAND_DW_T
+#undef SN_EXPAND_DW_P
 #undef SN_EXPAND_DW
 }
 
