@@ -56,6 +56,20 @@ __device__ __forceinline__ float act_apply(float v, int act) {
     return act == SN_ACT_HSWISH ? v * t : t;
 }
 
+// The same values by the division, for the direct convolutions: the compiler
+// unrolls their channel loop, so that several loads are in flight, where the
+// division's code follows it, and not where sixth() does (3 x 52 x 52, 22 -> 38
+// channels, 3x3, bf16 NHWC: 16.5 us, with sixth() 32.3; qint8 NCHW 11.1 and 19.8;
+// batches of loads written out by hand: 16.3 to 21 and 13.6).  One division an
+// output is nothing to them.
+__device__ __forceinline__ float act_apply_div(float v, int act) {
+    if (act == SN_ACT_RELU) return fmaxf(v, 0.0f);
+    if (act == SN_ACT_NONE) return v;
+    if (act == SN_ACT_RELU6) return fminf(fmaxf(v, 0.0f), 6.0f);
+    const float t = fminf(fmaxf(v + 3.0f, 0.0f), 6.0f) / 6.0f;
+    return act == SN_ACT_HSWISH ? v * t : t;
+}
+
 // streaming multiprocessors of the current device (host)
 inline int num_sms() {
     static int n = 0;

@@ -425,7 +425,7 @@ __global__ void conv_direct_nchw(const T *__restrict__ x, const T *__restrict__ 
             }
         }
         if (res) acc += ldf<T>(res + i);  // residual: same layout and index as the output
-        stf<T>(y + i, act_apply(acc + bias[kk], d.act));
+        stf<T>(y + i, act_apply_div(acc + bias[kk], d.act));
     }
 }
 
@@ -457,7 +457,7 @@ __global__ void conv_direct_nhwc(const T *__restrict__ x, const T *__restrict__ 
             }
         }
         if (res) acc += ldf<T>(res + i);  // residual: same layout and index as the output
-        stf<T>(y + i, act_apply(acc + bias[kk], d.act));
+        stf<T>(y + i, act_apply_div(acc + bias[kk], d.act));
     }
 }
 

@@ -392,7 +392,7 @@ __global__ void q8_conv_direct_kernel(const int8_t *__restrict__ x, const int8_t
             }
         }
         const float rv = res ? __fmul_rn((float)res[i], q.s_r) : 0.0f;  // residual: the output's index
-        y[i] = q8_out<TO>(q8_value(acc, q.s_x, ws[kk], bias[kk], rv, d.act), q.inv_out);
+        y[i] = q8_out<TO>(q8_value<true>(acc, q.s_x, ws[kk], bias[kk], rv, d.act), q.inv_out);
     }
 }
 

@@ -20,20 +20,24 @@ __device__ __forceinline__ int8_t q8_code(float y, float inv) {
     return (int8_t)max(-QMAX, min(QMAX, q));
 }
 
-// the fused activations with one rounding per operation
+// the fused activations with one rounding per operation (DIV: the same values by
+// the division, see act_apply_div)
+template <bool DIV = false>
 __device__ __forceinline__ float q8_act(float v, int act) {
     if (act == SN_ACT_RELU) return fmaxf(v, 0.0f);
     if (act == SN_ACT_NONE) return v;
     if (act == SN_ACT_RELU6) return fminf(fmaxf(v, 0.0f), 6.0f);
-    const float t = sixth(fminf(fmaxf(__fadd_rn(v, 3.0f), 0.0f), 6.0f));  // hard sigmoid: v / 6 to the bit
+    const float r = fminf(fmaxf(__fadd_rn(v, 3.0f), 0.0f), 6.0f);
+    const float t = DIV ? __fdiv_rn(r, 6.0f) : sixth(r);  // hard sigmoid: r / 6 to the bit
     return act == SN_ACT_HSWISH ? __fmul_rn(v, t) : t;
 }
 
 // act(float(acc) * (s_x * s_w) + bias [+ residual value]) in fp32
+template <bool DIV = false>
 __device__ __forceinline__ float q8_value(int acc, float s_x, float s_w, float bias, float resid, int act) {
     float y = __fadd_rn(__fmul_rn(__int2float_rn(acc), __fmul_rn(s_x, s_w)), bias);
     y = __fadd_rn(y, resid);
-    return q8_act(y, act);
+    return q8_act<DIV>(y, act);
 }
 
 // the output element: a code of the output blob's scale, or, when the routine
