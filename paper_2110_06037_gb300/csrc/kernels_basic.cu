@@ -529,8 +529,11 @@ __device__ __forceinline__ void fma16(float (&acc)[E], const uint4 &x, const uin
 
 // One thread: QB consecutive output columns x E channels (16 bytes) of one
 // output row.  Threads walk the (row, column block, channel vector) items with
-// the channel vector fastest (coalesced 16-byte accesses) and no thread idle at
-// a row's end; the three indices are divisions by launch constants.
+// the channel vector fastest (coalesced 16-byte accesses); the three indices are
+// divisions by launch constants.  On the window path no thread is idle at a row's
+// end.  On the other one a block stays in its row (row_items of fd_items.d are
+// work), whose input its threads read many times over: 32 x 14 x 14 x 96 fp32,
+// 7x7: 15.6 us, cut across rows 30.5; bf16, 8 x 28 x 28 x 144: 14.1 and 17.3.
 // SW = 1 or 2, KS = 3 or 5: the window path for that stride and kernel, where a
 // tap row's input columns are loaded once for the QB outputs that read them
 // (5x5, 4 outputs: 8 loads a row instead of 20 conditional ones; 8 x 28 x 28 x
@@ -539,7 +542,8 @@ __device__ __forceinline__ void fma16(float (&acc)[E], const uint4 &x, const uin
 template <typename T, int QB, int SW, int KS>
 __global__ void __launch_bounds__(256, 2) dw_nhwc_vec(const T *__restrict__ x, const T *__restrict__ w,
                                                       const float *__restrict__ bias, T *__restrict__ y, ConvDims d,
-                                                      FastDiv fd_items, FastDiv fd_cv, FastDiv fd_P, uint32_t total) {
+                                                      FastDiv fd_items, FastDiv fd_cv, FastDiv fd_P, int row_items,
+                                                      uint32_t total) {
     griddep_launch();
     griddep_wait();
     constexpr int E = 16 / sizeof(T);
@@ -547,6 +551,7 @@ __global__ void __launch_bounds__(256, 2) dw_nhwc_vec(const T *__restrict__ x, c
     if (t >= total) return;
     const int rowi = (int)fdiv(t, fd_items);
     const int item = (int)(t - (uint32_t)rowi * fd_items.d);
+    if (SW == 0 && item >= row_items) return;
     const int qb = (int)fdiv((uint32_t)item, fd_cv), cv = item - qb * (int)fd_cv.d;
     const int c0 = cv * E, q0 = qb * QB;
     float b[E];
@@ -1072,18 +1077,20 @@ cudaError_t dwconv(const LaunchArgs &a) {
                 else launch_pdl(dw3_nhwc_halo<T, 2, 3>, gb, 256, sm2, a.stream, x, w, a.bias, y, d);
             } else {
                 const int QBLK = (d.Q + 3) / 4, CV = (int)cvec;
-                const int64_t items = (int64_t)QBLK * CV, threads = (int64_t)d.N * d.P * items;
+                const bool k5 = d.R == 5 && d.S == 5 && d.dw == 1, window = (k3 || k5) && (d.sw == 1 || d.sw == 2);
+                const int64_t items = (int64_t)QBLK * CV, rows = (int64_t)d.N * d.P, whole = (items + 255) / 256 * 256;
+                const int64_t row = window || rows * whole >= ((int64_t)1 << 31) ? items : whole, threads = rows * row;
                 if (threads >= ((int64_t)1 << 31)) {
                     launch_pdl(dw_nhwc<T>, grid_for(total, 256), 256, 0, a.stream, x, w, a.bias, y, d);
                 } else {
                     // blocks of 128 until there are four of 256 for every SM
-                    const unsigned bs = threads < 152LL * 4 * 256 ? 128u : 256u;
+                    const unsigned bs = window && threads < 152LL * 4 * 256 ? 128u : 256u;
                     const unsigned gb = (unsigned)((threads + bs - 1) / bs);
-                    const FastDiv fi = make_fastdiv((uint32_t)items), fc = make_fastdiv((uint32_t)CV),
+                    const FastDiv fi = make_fastdiv((uint32_t)row), fc = make_fastdiv((uint32_t)CV),
                                   fp = make_fastdiv((uint32_t)d.P);
-                    const bool k5 = d.R == 5 && d.S == 5 && d.dw == 1;
                     auto go = [&](auto kern) {
-                        launch_pdl(kern, gb, bs, 0, a.stream, x, w, a.bias, y, d, fi, fc, fp, (uint32_t)threads);
+                        launch_pdl(kern, gb, bs, 0, a.stream, x, w, a.bias, y, d, fi, fc, fp, (int)items,
+                                   (uint32_t)threads);
                     };
                     if (k3 && d.sw == 1) go(dw_nhwc_vec<T, 4, 1, 3>);
                     else if (k3 && d.sw == 2) go(dw_nhwc_vec<T, 4, 2, 3>);

@@ -124,3 +124,16 @@ def test_maxpool_windows(ks, st, pd, n, c, h, w, dt):
     xs = stored_values(x, dt)
     ref = run_layer(net[0], [np.where(np.isnan(xs), -np.inf, xs)], dt)
     np.testing.assert_array_equal(run_float(net, x, (dt, "nhwc")), ref)
+
+
+@pytest.mark.parametrize("c,w", [(264, 37), (1032, 5), (8, 130)])
+@pytest.mark.parametrize("dt", ["f32", "bf16"])
+def test_depthwise_general_path_rows(c, w, dt):
+    """Blocks that stay in a row: rows of several blocks, the last one partly idle, and short rows."""
+    rng = np.random.default_rng(c + w)
+    x = rng.standard_normal((2, c, 4, w)).astype(np.float32)
+    layer = dict(synth.dwconv(c, 7, 1, act="relu6"), inputs=[-1])
+    layer["weight"] = (rng.standard_normal((c, 1, 7, 7)) / 7).astype(np.float32)
+    layer["bias"] = rng.standard_normal(c).astype(np.float32)
+    ref = run_layer(layer, [stored_values(x, dt)], dt)
+    assert maxrel(run_float([layer], x, (dt, "nhwc")), ref) <= TOL[dt]
