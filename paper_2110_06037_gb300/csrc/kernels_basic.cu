@@ -1610,10 +1610,12 @@ static cudaError_t dense_t(const LaunchArgs &a) {
                    (const T *)a.wt, a.bias, (T *)a.out, N, IN, OUT, a.layer->act);
         return cudaGetLastError();
     }
-    // images per warp: large weights are read once for as many as there are;
-    // small ones stay in L2, and a warp per (feature, image) fills the GPU
-    // better until there are eight a scheduler (152 SMs x 4 x 16 / 8 blocks)
-    const bool big = IN * OUT >= ((int64_t)1 << 19);
+    // images per warp: weights of half the L2 and more are read once for as many
+    // as there are; smaller ones stay there, and a warp per (feature, image) fills
+    // the GPU better until there are eight a scheduler (152 SMs x 4 x 16 / 8
+    // blocks).  8 images of 2048 -> 1000, fp32: 8.2 us, eight a warp 15.0; 4 images of
+    // 25088 -> 4096, fp16: 208, one a warp 310.
+    const bool big = IN * OUT * (int64_t)sizeof(T) >= ((int64_t)64 << 20);
     const int nb = big ? (N >= 4 ? 8 : N >= 2 ? 2 : 1) : N * OUT >= 8 * 9728 ? 8 : N * OUT >= 2 * 9728 ? 2 : 1;
     const dim3 g((unsigned)((OUT + 7) / 8), (unsigned)((N + nb - 1) / nb));
     auto go = [&](auto kern) {
