@@ -632,23 +632,41 @@ __global__ void __launch_bounds__(256, 2) dw_nhwc_vec(const T *__restrict__ x, c
             // columns) is loaded once and reused by the KS taps
             constexpr int WN = (QB - 1) * (SW > 0 ? SW : 1) + KS;
             const int wbase = q0 * SW - d.pw;
-#pragma unroll
-            for (int r = 0; r < KS; ++r) {
+            auto load = [&](int r, uint4 *win) {  // false: the row is padding
                 const int h = p * d.sh - d.ph + r * d.dh;
-                if (h < 0 || h >= d.H) continue;
+                const bool row = h >= 0 && h < d.H;
                 const T *xrow = x + (((int64_t)n * d.H + h) * d.W) * d.C + c0;
-                uint4 win[WN];
 #pragma unroll
                 for (int t = 0; t < WN; ++t) {
                     const int ww = wbase + t;
-                    win[t] = (ww >= 0 && ww < d.W) ? *reinterpret_cast<const uint4 *>(xrow + (int64_t)ww * d.C)
-                                                    : make_uint4(0u, 0u, 0u, 0u);
+                    win[t] = (row && ww >= 0 && ww < d.W) ? *reinterpret_cast<const uint4 *>(xrow + (int64_t)ww * d.C)
+                                                           : make_uint4(0u, 0u, 0u, 0u);
                 }
+                return row;
+            };
+            auto add = [&](int r, const uint4 *win) {
 #pragma unroll
                 for (int s = 0; s < KS; ++s) {
                     const uint4 wq = *reinterpret_cast<const uint4 *>(w + (int64_t)(r * KS + s) * d.C + c0);
 #pragma unroll
                     for (int j = 0; j < QB; ++j) fma16<T>(acc[j], win[j * (SW > 0 ? SW : 1) + s], wq);
+                }
+            };
+            if constexpr (KS == 3 && SW == 1 && sizeof(T) == 4) {
+                // the three rows' loads in flight together, as the registers allow in
+                // fp32 (8 x 28 x 28 x 96: 3.3 us, row by row 3.9; bf16 loses by it)
+                uint4 win[KS][WN];
+                bool row[KS];
+#pragma unroll
+                for (int r = 0; r < KS; ++r) row[r] = load(r, win[r]);
+#pragma unroll
+                for (int r = 0; r < KS; ++r)
+                    if (row[r]) add(r, win[r]);
+            } else {
+#pragma unroll
+                for (int r = 0; r < KS; ++r) {
+                    uint4 win[WN];
+                    if (load(r, win)) add(r, win);
                 }
             }
         } else {
